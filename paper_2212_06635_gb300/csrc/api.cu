@@ -371,8 +371,8 @@ static const void* clovH_ptr(const tm_ctx* c, int P) {
 // ---------------------------------------------------------------------------
 // blocks of a pass: one thread per site, except the direct two-flavour even pass
 // (a thread per site and flavour)
-static int pass_nblk(long vh, int nf, int kind, int staged) {
-    return staged ? nblk(vh, STAGED_BS) : nblk(nf == 2 && kind == K1_EO_INV ? 2 * vh : vh, DSLASH_BS);
+static int pass_nblk(int P, long vh, int nf, int kind, int staged) {
+    return staged ? nblk(vh, STAGED_BS) : nblk(nf == 2 && kind == K1_EO_INV ? 2 * vh : vh, dslash_bs(P));
 }
 
 // launch one pass in the variant the context chose for (P, NF, KIND)
@@ -389,7 +389,7 @@ static OpProb make_prob(const tm_ctx* c, int P, int nf, int kind, int sign, void
     OpProb p{};
     p.g = c->g;
     // (the double-word passes run a thread per site and flavour)
-    p.nblk = P == PDF ? nblk((long)nf * c->vh, DSLASH_BS) : pass_nblk(c->vh, nf, kind, c->variant[P][nf - 1][kind]);
+    p.nblk = P == PDF ? nblk((long)nf * c->vh, DSLASH_BS) : pass_nblk(P, c->vh, nf, kind, c->variant[P][nf - 1][kind]);
     p.bc_t = (float)c->params.bc_t;
     p.gauge[0] = gauge_ptr(c, P, 0);
     p.gauge[1] = gauge_ptr(c, P, 1);
@@ -666,14 +666,14 @@ static tm_status kernel_times_t(tm_ctx* c, int sign, const void* in, int reps, d
     CK(cudaEventCreate(&e1));
     CK(cudaEventCreate(&e2));
     b.p[0] = make_prob(c, P, NF, K1_EO_INV, sign, te, in, nullptr, nullptr, false);
-    int nb = b.p[0].nblk = pass_nblk(c->vh, NF, K1_EO_INV, v1);
+    int nb = b.p[0].nblk = pass_nblk(P, c->vh, NF, K1_EO_INV, v1);
     b.blk_start[1] = nb;
     CK((launch_pass<P, NF, K1_EO_INV, 1>(v1, b, nb, st)));   // warm-up
     CK(cudaEventRecord(e0, st));
     for (int r = 0; r < reps; ++r) CK((launch_pass<P, NF, K1_EO_INV, 1>(v1, b, nb, st)));
     CK(cudaEventRecord(e1, st));
     b.p[0] = make_prob(c, P, NF, K2_OE_LOCAL, sign, out, te, in, nullptr, false);
-    nb = b.p[0].nblk = pass_nblk(c->vh, NF, K2_OE_LOCAL, v2);
+    nb = b.p[0].nblk = pass_nblk(P, c->vh, NF, K2_OE_LOCAL, v2);
     b.blk_start[1] = nb;
     for (int r = 0; r < reps; ++r) CK((launch_pass<P, NF, K2_OE_LOCAL, 1>(v2, b, nb, st)));
     CK(cudaEventRecord(e2, st));
@@ -1672,7 +1672,7 @@ static tm_status batch_core(tm_ctx** cs, int n, tm_op op, const tm_solve_params*
         ob1 = ob2 = vbk = 0;
         for (int q = 0; q < n; ++q) {
             tm_ctx* c = cs[q];
-            const int nb1 = nblk(c->vh, v1 ? STAGED_BS : DSLASH_BS), nb2 = nblk(c->vh, v2 ? STAGED_BS : DSLASH_BS);
+            const int nb1 = pass_nblk(PS, c->vh, 1, K1_EO_INV, v1), nb2 = pass_nblk(PS, c->vh, 1, K2_OE_LOCAL, v2);
             const int nbb = nblk(c->vh, BLAS_BS);
             SolverCtl* ctl = c->ctl;
             k1.blk_start[q] = k1b.blk_start[q] = ob1;

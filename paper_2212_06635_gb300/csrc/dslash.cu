@@ -16,8 +16,21 @@
 
 namespace tmk {
 
+// Whether the first hop writes the accumulators instead of adding to zeros (which
+// saves 24 additions a flavour, but moves the register allocation): per pass what
+// measured faster.  Adding / writing, us: light FP16 even 106.6 / 110.6, odd 102.3 /
+// 100.8; FP32 even 198.7 / 180.4 (with the register cap below), odd 152.3 / 149.4;
+// BF16 at 18x22x26x44 30.7 / 31.3 and 28.7 / 29.5; two-flavour odd pass at 24^3x48
+// FP16 61.6 / 61.3, FP32 75.0 / 75.9.
+template <int P, int NF, int KIND>
+constexpr bool hop_first() {
+    if (P == P64) return true;
+    if (P == P32) return NF == 1;
+    return P == PF16 && (NF == 2 || KIND == K2_OE_LOCAL);
+}
+
 // All 8 hops for NF flavours into acc[NF][4][3]; output site (c, i) of parity po.
-template <int P, int NF, int MU>
+template <int P, int NF, int KIND, int MU>
 __device__ __forceinline__ void hop_mu(cpx<typename PT<P>::R> (&acc)[NF][4][3], const OpProb& pr,
                                        const Coord& c, long i, int po) {
     using R = typename PT<P>::R;
@@ -35,36 +48,91 @@ __device__ __forceinline__ void hop_mu(cpx<typename PT<P>::R> (&acc)[NF][4][3], 
     const long nf = cb_index(g, xf, yf, zf, tf);
     const long nb = cb_index(g, xb, yb, zb, tb);
     constexpr bool SC = (P == PF16 || P == PB16);   // 16-bit: the scale joins the phase
+    constexpr bool FIRST = MU == 0 && hop_first<P, NF, KIND>();
     cpx<R> u[9];
     cpx<R> psi[NF * 12];
     float sc;
-    // forward
-    load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nf, psi, sc);
-    load_link<P>(pr.gauge[po], g.vh, MU, i, u);
+    if constexpr (P == P64) {   // bound by FP64 arithmetic: the form with the fewest instructions
+        cpx<R> gf[NF][2][3];
+        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nf, psi, sc);
+        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
 #pragma unroll
-    for (int f = 0; f < NF; ++f) hop_dir<R, MU, -1, false, SC>(acc[f], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
-    // backward
-    load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nb, psi, sc);
-    load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
+        for (int f = 0; f < NF; ++f) hop_forward<R, MU, SC>(gf[f][0], gf[f][1], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
+        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nb, psi, sc);
+        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
 #pragma unroll
-    for (int f = 0; f < NF; ++f) hop_dir<R, MU, +1, true, SC>(acc[f], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
+        for (int f = 0; f < NF; ++f)
+            hop_backward<R, MU, SC, FIRST>(acc[f], gf[f][0], gf[f][1], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
+    } else {
+        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nf, psi, sc);
+        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+            hop_dir<R, MU, -1, false, SC, FIRST>(acc[f], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
+        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nb, psi, sc);
+        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) hop_dir<R, MU, +1, true, SC>(acc[f], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
+    }
 }
 
-// Resident blocks the compiler must fit per SM (128-thread blocks; the register
-// cap follows).  Sweeps at 32^3x64 (light) and 24^3x48 (heavy) put the optimum at:
+// out = B_c v (CONJ: B_c^dagger v) per chirality block c of the even-site inverse.
+// The sign is decided outside: inside the products it made every FMA a pair of
+// predicated ones (FP64 even pass at 16^3x32 188.5 -> 149.8 us, light FP16 at
+// 32^3x64 112.5 -> 106.6 us).
+template <int P, bool CONJ>
+__device__ __forceinline__ void inverse_blocks(cpx<typename PT<P>::R>* out, const OpProb& pr, long i,
+                                               const cpx<typename PT<P>::R> (&acc)[4][3]) {
+    using R = typename PT<P>::R;
+#pragma unroll
+    for (int cb = 0; cb < 2; ++cb) {
+        cpx<R> v[6], w[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            v[j] = acc[2 * cb + j / 3][j % 3];
+            w[j] = C((R)0, (R)0);
+        }
+        // stream the block two rows (24 reals) at a time to bound registers
+#pragma unroll
+        for (int rr = 0; rr < 3; ++rr) {
+            R m[24];
+            load_reals<P, 24>(pr.clov, pr.g.vh, i, 72 * cb + 24 * rr, m);
+#pragma unroll
+            for (int r2 = 0; r2 < 2; ++r2) {
+                const int r = 2 * rr + r2;
+#pragma unroll
+                for (int j = 0; j < 6; ++j) {
+                    const cpx<R> e = C(m[2 * (6 * r2 + j)], m[2 * (6 * r2 + j) + 1]);
+                    if (CONJ) cfma_cj(w[j], e, v[r]);
+                    else cfma(w[r], e, v[j]);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 6; ++j) out[6 * cb + j] = w[j];
+    }
+}
+
+// Resident blocks the compiler must fit per SM (128-thread blocks, FP64 64-thread
+// ones; the register cap follows).  Sweeps at 32^3x64 (light) and 24^3x48 (heavy)
+// put the optimum at:
 //   light 16-bit even pass: 5 blocks (96 registers; the inverse blocks stream two
-//     rows at a time for this).  6 blocks: 112.8 -> 133.4 us FP16, 116.6 -> 174.2 us BF16;
+//     rows at a time for this).  6 blocks: 112.8 -> 133.4 us FP16, 116.6 -> 174.2 us
+//     BF16 (before inverse_blocks took its present form: 106.6 us FP16 since);
 //   light odd pass: 7 blocks FP16 (72 registers, 16 B spilled) and 6 BF16 (80
 //     registers): 5 / 6 / 7 blocks take 112.2 / 104.9 / 103.0 us FP16 and
 //     126.9 / 113.2 / 119.0 us BF16 (4 blocks: 108.3 / 113.1 us);
 //   light FP32 odd pass: 4 blocks (128 registers, 16 B spilled): 156.5 -> 150.0 us
-//     (3 blocks 152.0 us); the FP32 even pass keeps the default (3 blocks at 156
-//     registers; 4 blocks: 187 -> 227 us);
+//     (3 blocks 152.0 us); even pass: 3 blocks (168 registers): 180.4 us against
+//     202.8 us at the 188 registers the compiler takes without a bound;
 //   two-flavour odd pass: 4 blocks in 16-bit storage (128 registers; 3 / 5
 //     blocks: 63.8 -> 67.7 / 75.0 us FP16) and 3 in FP32 (168 registers, 8 B
-//     spilled: 94.8 -> 78.1 us at 24^3x48; 2 / 4 blocks: 94.5 / 84.4 us).
-// The FP64 passes keep the default.  (The two-flavour even pass splits the
-// flavours over a thread pair: dslash_heavy.cu.)
+//     spilled: 94.8 -> 78.1 us at 24^3x48; 2 / 4 blocks: 94.5 / 84.4 us);
+//   FP64: 8 blocks of 64 threads (128 registers).  The FP64 units bound the passes,
+//     but the waits for operands show at 8 warps per SM: 16^3x32 even / odd
+//     149.8 / 153.2 -> 141.6 / 143.4 us against 4 blocks (253 registers, none
+//     spilled); at 24^3x48, where many waves even this out, 636 / 653 -> 640 / 664 us.
+// (The two-flavour even pass splits the flavours over a thread pair: dslash_heavy.cu.)
 template <int P, int NF, int KIND>
 constexpr int dslash_min_blocks() {
     if (P == PF16 || P == PB16) {
@@ -72,8 +140,8 @@ constexpr int dslash_min_blocks() {
         if (KIND == K1_EO_INV) return 5;
         return P == PF16 ? 7 : 6;
     }
-    if (P == P32 && KIND == K2_OE_LOCAL) return NF == 2 ? 3 : 4;
-    return 1;
+    if (P == P32) return KIND == K1_EO_INV ? 3 : (NF == 2 ? 3 : 4);
+    return 8;   // P64
 }
 
 template <int P, int NF, int KIND, int NP, int BS>
@@ -92,48 +160,25 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
     if (valid) {
         const Coord c = cb_coords(pr.g, i, po);
         cpx<R> acc[NF][4][3];
+        if constexpr (!hop_first<P, NF, KIND>()) {
 #pragma unroll
-        for (int f = 0; f < NF; ++f)
+            for (int f = 0; f < NF; ++f)
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
+                for (int s = 0; s < 4; ++s)
 #pragma unroll
-                for (int a = 0; a < 3; ++a) acc[f][s][a] = C((R)0, (R)0);
-        hop_mu<P, NF, 0>(acc, pr, c, i, po);
-        hop_mu<P, NF, 1>(acc, pr, c, i, po);
-        hop_mu<P, NF, 2>(acc, pr, c, i, po);
-        hop_mu<P, NF, 3>(acc, pr, c, i, po);
+                    for (int a = 0; a < 3; ++a) acc[f][s][a] = C((R)0, (R)0);
+        }
+        hop_mu<P, NF, KIND, 0>(acc, pr, c, i, po);
+        hop_mu<P, NF, KIND, 1>(acc, pr, c, i, po);
+        hop_mu<P, NF, KIND, 2>(acc, pr, c, i, po);
+        hop_mu<P, NF, KIND, 3>(acc, pr, c, i, po);
 
         cpx<R> out[NF * 12];
         if constexpr (KIND == K1_EO_INV) {
             if constexpr (NF == 1) {
                 // t_e = (A_c + i sign s_c mu_t)^-1 (H psi) per chirality block c
-#pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    cpx<R> v[6], w[6];
-#pragma unroll
-                    for (int j = 0; j < 6; ++j) {
-                        v[j] = acc[0][2 * cb + j / 3][j % 3];
-                        w[j] = C((R)0, (R)0);
-                    }
-                    // stream the block two rows (24 reals) at a time to bound registers
-#pragma unroll
-                    for (int rr = 0; rr < 3; ++rr) {
-                        R m[24];
-                        load_reals<P, 24>(pr.clov, pr.g.vh, i, 72 * cb + 24 * rr, m);
-#pragma unroll
-                        for (int r2 = 0; r2 < 2; ++r2) {
-                            const int r = 2 * rr + r2;
-#pragma unroll
-                            for (int j = 0; j < 6; ++j) {
-                                const cpx<R> e = C(m[2 * (6 * r2 + j)], m[2 * (6 * r2 + j) + 1]);
-                                if (pr.sign > 0) cfma(w[r], e, v[j]);       // B v
-                                else cfma_cj(w[j], e, v[r]);                // B^dagger v
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 6; ++j) out[6 * cb + j] = w[j];
-                }
+                if (pr.sign > 0) inverse_blocks<P, false>(out, pr, i, acc[0]);
+                else inverse_blocks<P, true>(out, pr, i, acc[0]);
             }
         } else {
             // out = g5 [ (A + i tw g5 [tau3]) psi - eps tau1 psi - kappa^2 acc ]
@@ -142,7 +187,8 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
             R m[72];
             load_reals<P, 72>(pr.clov, pr.g.vh, i, 0, m);
             const R k2 = (R)(pr.kappa * pr.kappa);
-            const R tw = (R)pr.tw;
+            // W_hat = Q_hat + i rho (eq:hWpm): i rho psi = g5 (i rho g5 psi) joins the twist
+            const R tw = (R)pr.tw, rho = (R)pr.rho;
             const R eps = (R)pr.eps;
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
@@ -154,15 +200,13 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
 #pragma unroll
                     for (int j = 0; j < 6; ++j) {
                         v[j] = psi[12 * f + 6 * cb + j];
-                        w[j] = (tw * sc * t3) * mul_i(v[j]);
+                        w[j] = (sc * (tw * t3 + rho)) * mul_i(v[j]);
                         if constexpr (NF == 2) w[j] = w[j] - eps * psi[12 * (1 - f) + 6 * cb + j];
                         w[j] = w[j] - k2 * acc[f][2 * cb + j / 3][j % 3];
                     }
                     herm6_mv_acc<R>(w, m + 36 * cb, v);
-                    const R rh = (R)pr.rho;   // W_hat = Q_hat + i rho (eq:hWpm), added after g5
 #pragma unroll
-                    for (int j = 0; j < 6; ++j)
-                        out[12 * f + 6 * cb + j] = ((cb == 0) ? w[j] : -w[j]) + rh * mul_i(v[j]);
+                    for (int j = 0; j < 6; ++j) out[12 * f + 6 * cb + j] = (cb == 0) ? w[j] : -w[j];
                 }
             }
             if (pr.partial != nullptr) {
@@ -185,7 +229,7 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
 
 template <int P, int NF, int KIND, int NP>
 cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st) {
-    dslash_kernel<P, NF, KIND, NP, DSLASH_BS><<<nblocks, DSLASH_BS, 0, st>>>(b);
+    dslash_kernel<P, NF, KIND, NP, dslash_bs(P)><<<nblocks, dslash_bs(P), 0, st>>>(b);
     return cudaGetLastError();
 }
 

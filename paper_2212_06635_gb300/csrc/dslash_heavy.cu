@@ -66,6 +66,12 @@ __device__ __forceinline__ void store_flavour(void* base, long vh, long i, int f
     }
 }
 
+// Whether the first hop writes the accumulators instead of adding to zeros (as
+// hop_first in dslash.cu).  Adding / writing at 24^3x48: FP16 73.2 / 71.6 us, FP32
+// 88.5 / 90.2 us.
+template <int P>
+constexpr bool heavy_first() { return P == P64 || P == PF16; }
+
 // hops of direction MU for flavour f into acc
 template <int P, int MU>
 __device__ __forceinline__ void hop_mu_flavour(cpx<typename PT<P>::R> (&acc)[4][3], const OpProb& pr, const Coord& c,
@@ -88,20 +94,32 @@ __device__ __forceinline__ void hop_mu_flavour(cpx<typename PT<P>::R> (&acc)[4][
     cpx<R> u[9];
     cpx<R> psi[12];
     float sc;
-    load_flavour_unscaled<P>(pr.in, g.vh, nf, f, psi, sc);
-    load_link<P>(pr.gauge[po], g.vh, MU, i, u);
-    hop_dir<R, MU, -1, false, SC>(acc, psi, u, SC ? ph_f * (R)sc : ph_f);
-    load_flavour_unscaled<P>(pr.in, g.vh, nb, f, psi, sc);
-    load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
-    hop_dir<R, MU, +1, true, SC>(acc, psi, u, SC ? ph_b * (R)sc : ph_b);
+    constexpr bool FIRST = MU == 0 && heavy_first<P>();
+    if constexpr (P == P64) {
+        cpx<R> gf0[3], gf1[3];
+        load_flavour_unscaled<P>(pr.in, g.vh, nf, f, psi, sc);
+        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
+        hop_forward<R, MU, SC>(gf0, gf1, psi, u, SC ? ph_f * (R)sc : ph_f);
+        load_flavour_unscaled<P>(pr.in, g.vh, nb, f, psi, sc);
+        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
+        hop_backward<R, MU, SC, FIRST>(acc, gf0, gf1, psi, u, SC ? ph_b * (R)sc : ph_b);
+    } else {
+        load_flavour_unscaled<P>(pr.in, g.vh, nf, f, psi, sc);
+        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
+        hop_dir<R, MU, -1, false, SC, FIRST>(acc, psi, u, SC ? ph_f * (R)sc : ph_f);
+        load_flavour_unscaled<P>(pr.in, g.vh, nb, f, psi, sc);
+        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
+        hop_dir<R, MU, +1, true, SC>(acc, psi, u, SC ? ph_b * (R)sc : ph_b);
+    }
 }
 
 // Resident blocks per SM the register allocation must allow (128 threads = 64
 // sites).  At 24^3x48: 16-bit 4 / 5 / 6 blocks take 73.9 / 73.5 / 73.9 us (FP16)
-// and 72.1 / 69.8 / 72.7 us (BF16); FP32 3 / 4 / 5 blocks 96.4 / 96.4 / 89.7 us.
+// and 72.1 / 69.8 / 72.7 us (BF16); FP32 3 / 4 / 5 blocks 96.4 / 96.4 / 89.7 us.  FP64 (64-thread blocks): 8 as
+// in dslash.cu; 4 / 8 blocks 317.4 / 317.6 us at 16^3x32.
 template <int P, int KIND>
 constexpr int heavy_min_blocks() {
-    return (P == PF16 || P == PB16) ? 5 : (P == P32 ? 5 : 1);
+    return (P == PF16 || P == PB16) ? 5 : (P == P32 ? 5 : 8);
 }
 
 template <int P, int KIND, int NP, int BS>
@@ -121,10 +139,12 @@ __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, KIND>())) dslash_heav
     if (valid) {
         const Coord c = cb_coords(pr.g, i, po);
         cpx<R> acc[4][3];
+        if constexpr (!heavy_first<P>()) {
 #pragma unroll
-        for (int s = 0; s < 4; ++s)
+            for (int s = 0; s < 4; ++s)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) acc[s][a] = C((R)0, (R)0);
+                for (int a = 0; a < 3; ++a) acc[s][a] = C((R)0, (R)0);
+        }
         hop_mu_flavour<P, 0>(acc, pr, c, i, po, f);
         hop_mu_flavour<P, 1>(acc, pr, c, i, po, f);
         hop_mu_flavour<P, 2>(acc, pr, c, i, po, f);
@@ -176,7 +196,7 @@ cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st);
 #define TM_HEAVY_INST(P, KIND)                                                                        \
     template <>                                                                                       \
     cudaError_t launch_dslash<P, 2, KIND, 1>(const OpBatch<1>& b, int nblocks, cudaStream_t st) {     \
-        dslash_heavy_kernel<P, KIND, 1, DSLASH_BS><<<nblocks, DSLASH_BS, 0, st>>>(b);                \
+        dslash_heavy_kernel<P, KIND, 1, dslash_bs(P)><<<nblocks, dslash_bs(P), 0, st>>>(b);          \
         return cudaGetLastError();                                                                    \
     }
 TM_HEAVY_INST(P64, K1_EO_INV)

@@ -8,6 +8,9 @@
 namespace tmk {
 
 constexpr int DSLASH_BS = 128;   // direct stencil kernel
+// FP64 passes take half-size blocks: their work is even, so the last wave is what
+// differs (24^3x48: 827 / 666 us at 128 threads, 813 / 652 us at 64, 32 the same)
+constexpr int dslash_bs(int P) { return P == P64 ? 64 : DSLASH_BS; }
 constexpr int STAGED_BS = 64;    // shared-memory staged stencil kernel
 constexpr int BLAS_BS = 256;
 constexpr int MIN_BS = 64;       // smallest block size of any reducing kernel (sizes the partials)
