@@ -26,9 +26,9 @@ using namespace tmk;
 
 namespace tmk {
 cudaError_t launch_gauge_import(void* d0, void* d1, const double* src, const Geom& g, cudaStream_t st);
-cudaError_t launch_clover(const Geom& g, const void* g0, const void* g1, int par, double kappa, double csw,
-                          double mu_t, double mubar_t, double epsbar_t, double* outA, double* outB,
-                          double* outH, cudaStream_t st);
+cudaError_t launch_clover(const Geom& g, const void* g0, const void* g1, double kappa, double csw, double mu_t,
+                          double mubar_t, double epsbar_t, double* outA0, double* outA1, double* outB, double* outH,
+                          cudaStream_t st);
 cudaError_t launch_clover_unpack(double* out, const double* A, long vh, cudaStream_t st);
 }  // namespace tmk
 
@@ -265,10 +265,8 @@ extern "C" tm_status tm_clover_compute(tm_ctx* c, const tm_params* prm, void* st
     if (!c->clovB64) CK(cudaMalloc(&c->clovB64, sizeof(double) * CLOV_EVEN_LIGHT_REALS * vh));
     if (heavy && !c->clovH64) CK(cudaMalloc(&c->clovH64, sizeof(double) * CLOV_EVEN_HEAVY_REALS * vh));
     const double k = prm->kappa;
-    CK(launch_clover(c->g, c->gauge64[0], c->gauge64[1], 0, k, prm->csw, 2 * k * prm->mu, 2 * k * prm->mubar,
-                     2 * k * prm->epsbar, c->clovA64[0], c->clovB64, heavy ? c->clovH64 : nullptr, st));
-    CK(launch_clover(c->g, c->gauge64[0], c->gauge64[1], 1, k, prm->csw, 0.0, 0.0, 0.0, c->clovA64[1], nullptr,
-                     nullptr, st));
+    CK(launch_clover(c->g, c->gauge64[0], c->gauge64[1], k, prm->csw, 2 * k * prm->mu, 2 * k * prm->mubar,
+                     2 * k * prm->epsbar, c->clovA64[0], c->clovA64[1], c->clovB64, heavy ? c->clovH64 : nullptr, st));
     c->params = *prm;
     c->have_heavy = heavy;
     c->clover_gauge_gen = c->gauge_gen;

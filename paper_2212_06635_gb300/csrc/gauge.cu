@@ -70,11 +70,29 @@ __global__ void k_clover_from64(void* dst, const double* __restrict__ src, long 
 // ---------------------------------------------------------------------------
 using cd = cpx<double>;
 
+// The clover term in three steps, all FP64 and all bound by the FP64 units (about
+// 2 lanes per cycle and SM), so the split is the one with the fewest products:
+//   k_leaves   one thread per site and plane: the plaquette based at x, once, and
+//              its four rotations, which are the leaves of its four corners.  With
+//              e = b c^+, f = d^+ a they are  a (e d^+), e f, c^+ (f b), f e:
+//              eight 3x3 products, the last of each leaf restricted to the part
+//              that survives Q - Q^+ (792 FMAs instead of the 1296 of a site that
+//              multiplies out its own four leaves);
+//   k_field    one thread per site and plane: sums the corners' contributions,
+//              removes the trace: F_munu, 9 reals;
+//   k_clover   one thread per site and chirality: A and, on even sites, its inverses.
+// The leaves pass through memory: 576 B a site and plane, at 24^3x48 about 0.4 ms
+// of the whole.  Two planes at a time fit the (not yet written) array of the light
+// even inverse, and F fits the array of A, so nothing is allocated.
+// 24^3x48 with both inverses: 16.8 ms as one kernel per parity, each site multiplying out its
+// own leaves -> 8.1 ms.
 struct M3 {
     cd m[9];
 };
 
-__device__ __forceinline__ M3 mm(const M3& a, const M3& b) {   // a b
+// a b, a b^+, a^+ b
+template <bool DA, bool DB>
+__device__ __forceinline__ M3 mul3(const M3& a, const M3& b) {
     M3 c;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -82,209 +100,319 @@ __device__ __forceinline__ M3 mm(const M3& a, const M3& b) {   // a b
         for (int j = 0; j < 3; ++j) {
             cd s = C(0.0, 0.0);
 #pragma unroll
-            for (int k = 0; k < 3; ++k) cfma(s, a.m[3 * i + k], b.m[3 * k + j]);
-            c.m[3 * i + j] = s;
-        }
-    return c;
-}
-__device__ __forceinline__ M3 mmd(const M3& a, const M3& b) {  // a b^+
-    M3 c;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cd s = C(0.0, 0.0);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) s = s + a.m[3 * i + k] * cj(b.m[3 * j + k]);
-            c.m[3 * i + j] = s;
-        }
-    return c;
-}
-__device__ __forceinline__ M3 mdm(const M3& a, const M3& b) {  // a^+ b
-    M3 c;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cd s = C(0.0, 0.0);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) cfma_cj(s, a.m[3 * k + i], b.m[3 * k + j]);
+            for (int k = 0; k < 3; ++k) {
+                const cd x = DA ? a.m[3 * k + i] : a.m[3 * i + k];
+                const cd y = DB ? b.m[3 * j + k] : b.m[3 * k + j];
+                if (DA) cfma_cj(s, x, y);
+                else if (DB) cfma_cj(s, y, x);
+                else cfma(s, x, y);
+            }
             c.m[3 * i + j] = s;
         }
     return c;
 }
 
-__device__ __forceinline__ M3 link_at(const Geom& g, const void* const* gauge, int mu,
-                                      int x, int y, int z, int t) {
-    x = (x + g.X) % g.X; y = (y + g.Y) % g.Y; z = (z + g.Z) % g.Z; t = (t + g.T) % g.T;
-    const int par = (x + y + z + t) & 1;
-    M3 u;
-    load_link<P64>(gauge[par], g.vh, mu, cb_index(g, x, y, z, t), u.m);
-    return u;
-}
-
-// F_munu(x) = (1/8)(Q - Q^+) - (1/3) tr, Q = sum of the four leaves in the (mu,nu) plane
-__device__ M3 clover_leaf(const Geom& g, const void* const* gauge, int mu, int nu, const int* xc) {
-    int e_mu[4] = {0, 0, 0, 0}, e_nu[4] = {0, 0, 0, 0};
-    e_mu[mu] = 1;
-    e_nu[nu] = 1;
-    auto L = [&](int d, int dm, int dn) {   // U_d(x + dm mu + dn nu)
-        return link_at(g, gauge, d, xc[0] + dm * e_mu[0] + dn * e_nu[0], xc[1] + dm * e_mu[1] + dn * e_nu[1],
-                       xc[2] + dm * e_mu[2] + dn * e_nu[2], xc[3] + dm * e_mu[3] + dn * e_nu[3]);
-    };
-    // leaf 1: U_mu(x) U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
-    M3 q = mmd(mmd(mm(L(mu, 0, 0), L(nu, 1, 0)), L(mu, 0, 1)), L(nu, 0, 0));
-    // leaf 2: U_nu(x) U_mu(x-mu+nu)^+ U_nu(x-mu)^+ U_mu(x-mu)
-    M3 l2 = mm(mmd(mmd(L(nu, 0, 0), L(mu, -1, 1)), L(nu, -1, 0)), L(mu, -1, 0));
-    // leaf 3: U_mu(x-mu)^+ U_nu(x-mu-nu)^+ U_mu(x-mu-nu) U_nu(x-nu) = (b a)^+ c d
-    M3 l3;
-    {
-        const M3 a = L(mu, -1, 0), b = L(nu, -1, -1), c = L(mu, -1, -1), d = L(nu, 0, -1);
-        l3 = mm(mdm(mm(b, a), c), d);
+// The anti-hermitian part M - M^+ of M = a b (DA: a^+ b) as 9 reals, one store each
+// stride apart: the three diagonal entries' imaginary parts / 2, then the entries
+// (1,0), (2,0), (2,1) as (re, im)
+template <bool DA>
+__device__ __forceinline__ void store_antiherm(double* out, long stride, const M3& a, const M3& b) {
+    auto at = [&](int i, int k) { return DA ? a.m[3 * k + i] : a.m[3 * i + k]; };
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const cd x = at(i, k), y = b.m[3 * k + i];
+            t = fma(x.re, y.im, t);
+            t = DA ? fma(-x.im, y.re, t) : fma(x.im, y.re, t);
+        }
+        out[i * stride] = t;
     }
-    // leaf 4: U_nu(x-nu)^+ U_mu(x-nu) U_nu(x-nu+mu) U_mu(x)^+
-    M3 l4 = mmd(mm(mdm(L(nu, 0, -1), L(mu, 0, -1)), L(nu, 1, -1)), L(mu, 0, 0));
 #pragma unroll
-    for (int k = 0; k < 9; ++k) q.m[k] = q.m[k] + l2.m[k] + l3.m[k] + l4.m[k];
-    M3 f;
+    for (int i = 1; i < 3; ++i)
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) f.m[3 * i + j] = 0.125 * (q.m[3 * i + j] - cj(q.m[3 * j + i]));
-    const double tr_im = (f.m[0].im + f.m[4].im + f.m[8].im) / 3.0;   // trace is imaginary
-#pragma unroll
-    for (int i = 0; i < 3; ++i) f.m[4 * i].im -= tr_im;
-    return f;
-}
-
-// inverse of a 6x6 hermitian positive definite matrix (Cholesky), in place
-__device__ void hpd6_inverse(cd (&h)[36]) {
-    cd L[36];
-#pragma unroll
-    for (int k = 0; k < 36; ++k) L[k] = C(0.0, 0.0);
-    for (int j = 0; j < 6; ++j) {
-        double d = h[6 * j + j].re;
-        for (int k = 0; k < j; ++k) d -= norm2(L[6 * j + k]);
-        const double ljj = sqrt(d);
-        L[6 * j + j] = C(ljj, 0.0);
-        for (int i = j + 1; i < 6; ++i) {
-            cd s = h[6 * i + j];
-            for (int k = 0; k < j; ++k) s = s - L[6 * i + k] * cj(L[6 * j + k]);
-            L[6 * i + j] = (1.0 / ljj) * s;
-        }
-    }
-    cd Li[36];
-#pragma unroll
-    for (int k = 0; k < 36; ++k) Li[k] = C(0.0, 0.0);
-    for (int i = 0; i < 6; ++i) {
-        Li[6 * i + i] = C(1.0 / L[6 * i + i].re, 0.0);
         for (int j = 0; j < i; ++j) {
-            cd s = C(0.0, 0.0);
-            for (int k = j; k < i; ++k) s = s + L[6 * i + k] * Li[6 * k + j];
-            Li[6 * i + j] = (-1.0 / L[6 * i + i].re) * s;
+            cd s = C(0.0, 0.0), t = C(0.0, 0.0);   // M_ij, M_ji
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (DA) {
+                    cfma_cj(s, at(i, k), b.m[3 * k + j]);
+                    cfma_cj(t, at(j, k), b.m[3 * k + i]);
+                } else {
+                    cfma(s, at(i, k), b.m[3 * k + j]);
+                    cfma(t, at(j, k), b.m[3 * k + i]);
+                }
+            }
+            const int e = 3 + 2 * (i * (i - 1) / 2 + j);
+            out[e * stride] = s.re - t.re;
+            out[(e + 1) * stride] = s.im + t.im;
+        }
+}
+
+struct CloverArgs {
+    Geom g;
+    const void* gauge[2];
+    int plane0;          // k_leaves, k_field: planes plane0, plane0 + 1
+    double* leaf;        // [parity][plane of the two][corner][9][vh]
+    double* F[2];        // per parity [plane][5][vh] pairs (9 reals and one unused); the array of
+                         // A, whose pairs of a site k_clover writes over the same site's F
+    double kc;           // kappa csw
+    double mu_t, mubar_t, epsbar_t;
+    double* outB;        // even inverse blocks (may be null)
+    double* outH;        // heavy even inverse blocks (may be null)
+};
+
+// planes 0 xy, 1 xz, 2 xt, 3 yz, 4 yt, 5 zt
+__device__ __forceinline__ void plane_dirs(int plane, int& mu, int& nu) {
+    mu = plane < 3 ? 0 : (plane < 5 ? 1 : 2);
+    nu = plane < 3 ? plane + 1 : (plane < 5 ? plane - 1 : 3);
+}
+
+// checkerboard index of the neighbour d (-1, 0, +1) steps along mu and e along nu
+__device__ __forceinline__ long shifted(const Geom& g, const Coord& c, int mu, int d, int nu, int e) {
+    int x[4] = {c.x, c.y, c.z, c.t};
+    const int L[4] = {g.X, g.Y, g.Z, g.T};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        x[k] += (k == mu ? d : 0) + (k == nu ? e : 0);
+        if (x[k] < 0) x[k] += L[k];
+        if (x[k] >= L[k]) x[k] -= L[k];
+    }
+    return cb_index(g, x[0], x[1], x[2], x[3]);
+}
+
+// blockIdx.y = 2 * (plane of the two) + parity
+__global__ void __launch_bounds__(64) k_leaves(const __grid_constant__ CloverArgs p) {
+    const long vh = p.g.vh, i = (long)blockIdx.x * 64 + threadIdx.x;
+    if (i >= vh) return;
+    const int par = blockIdx.y & 1, pl = blockIdx.y >> 1;
+    int mu, nu;
+    plane_dirs(p.plane0 + pl, mu, nu);
+    const Coord x = cb_coords(p.g, i, par);
+    const long xm = shifted(p.g, x, mu, 1, nu, 0), xn = shifted(p.g, x, mu, 0, nu, 1);
+    M3 a, b, c, d;
+    load_link<P64>(p.gauge[1 - par], vh, nu, xm, b.m);
+    load_link<P64>(p.gauge[1 - par], vh, mu, xn, c.m);
+    load_link<P64>(p.gauge[par], vh, mu, i, a.m);
+    load_link<P64>(p.gauge[par], vh, nu, i, d.m);
+    double* out = p.leaf + (long)(par * 2 + pl) * 36 * vh + i;
+    const M3 e = mul3<false, true>(b, c), f = mul3<true, false>(d, a);
+    store_antiherm<false>(out + 9 * vh, vh, e, f);                             // corner x + mu
+    store_antiherm<false>(out + 27 * vh, vh, f, e);                            // corner x + nu
+    store_antiherm<false>(out, vh, a, mul3<false, true>(e, d));                // corner x
+    store_antiherm<true>(out + 18 * vh, vh, c, mul3<false, false>(f, b));      // corner x + mu + nu
+}
+
+__global__ void __launch_bounds__(128) k_field(const __grid_constant__ CloverArgs p) {
+    const long vh = p.g.vh, i = (long)blockIdx.x * 128 + threadIdx.x;
+    if (i >= vh) return;
+    const int par = blockIdx.y & 1, pl = blockIdx.y >> 1;
+    int mu, nu;
+    plane_dirs(p.plane0 + pl, mu, nu);
+    const Coord x = cb_coords(p.g, i, par);
+    const double* same = p.leaf + (long)(par * 2 + pl) * 36 * vh;
+    const double* other = p.leaf + (long)((1 - par) * 2 + pl) * 36 * vh;
+    const double* src[4] = {same + i, other + 9 * vh + shifted(p.g, x, mu, -1, nu, 0),
+                            same + 18 * vh + shifted(p.g, x, mu, -1, nu, -1),
+                            other + 27 * vh + shifted(p.g, x, mu, 0, nu, -1)};
+    double q[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) q[k] = ((src[0][k * vh] + src[1][k * vh]) + src[2][k * vh]) + src[3][k * vh];
+    // F = (Q - Q^+) / 8 less its trace (imaginary; the leaves' diagonal holds half of Q - Q^+)
+    const double tr = (q[0] + q[1] + q[2]) * (1.0 / 3.0);
+    double2* out = reinterpret_cast<double2*>(p.F[par]) + (long)(p.plane0 + pl) * 5 * vh + i;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) q[k] = k < 3 ? 0.25 * (q[k] - tr) : 0.125 * q[k];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) out[k * vh] = make_double2(q[2 * k], k < 4 ? q[2 * k + 1] : 0.0);
+}
+
+// hermitian 6x6: real diagonal, strictly lower entries row by row
+struct H6 {
+    double d[6];
+    cd l[15];
+    __device__ __forceinline__ cd at(int r, int j) const {   // r != j
+        return r > j ? l[r * (r - 1) / 2 + j] : cj(l[j * (j - 1) / 2 + r]);
+    }
+};
+
+// the product of two hermitian matrices that commute (hermitian again)
+__device__ __forceinline__ H6 mul_commuting(const H6& a, const H6& b) {
+    H6 c;
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+        double t = a.d[r] * b.d[r];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            if (k == r) continue;
+            const cd x = a.at(r, k), y = b.at(r, k);   // b_kr = conj(b_rk)
+            t = fma(x.re, y.re, t);
+            t = fma(x.im, y.im, t);
+        }
+        c.d[r] = t;
+#pragma unroll
+        for (int j = 0; j < r; ++j) {
+            cd s = a.d[r] * b.at(r, j);
+            const cd x = a.at(r, j);
+            s.re = fma(x.re, b.d[j], s.re);
+            s.im = fma(x.im, b.d[j], s.im);
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                if (k != r && k != j) cfma(s, a.at(r, k), b.at(k, j));
+            c.l[r * (r - 1) / 2 + j] = s;
         }
     }
-    for (int i = 0; i < 6; ++i)
-        for (int j = 0; j < 6; ++j) {
-            cd s = C(0.0, 0.0);
-            const int k0 = i > j ? i : j;
-            for (int k = k0; k < 6; ++k) cfma_cj(s, Li[6 * k + i], Li[6 * k + j]);
-            h[6 * i + j] = s;
+    return c;
+}
+
+// (a + shift)^-1 of a hermitian positive definite a + shift, by Cholesky: L, then
+// L^-1, then L^-+ L^-1
+__device__ __forceinline__ H6 hpd6_inverse(const H6& a, double shift) {
+    H6 L;   // L.d: 1 / L_jj
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        double t = a.d[j] + shift;
+#pragma unroll
+        for (int k = 0; k < j; ++k) {
+            const cd x = L.l[j * (j - 1) / 2 + k];
+            t = fma(-x.re, x.re, t);
+            t = fma(-x.im, x.im, t);
         }
+        L.d[j] = rsqrt(t);
+#pragma unroll
+        for (int i = j + 1; i < 6; ++i) {
+            cd s = -a.l[i * (i - 1) / 2 + j];
+#pragma unroll
+            for (int k = 0; k < j; ++k) cfma_cj(s, L.l[j * (j - 1) / 2 + k], L.l[i * (i - 1) / 2 + k]);
+            L.l[i * (i - 1) / 2 + j] = -L.d[j] * s;
+        }
+    }
+    // in place, column by column from the right: Li_ij = -Li_ii sum_{j <= k < i} L_ik Li_kj
+    H6 D;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        D.d[j] = L.d[j];
+#pragma unroll
+        for (int i = j + 1; i < 6; ++i) {
+            const cd x = L.l[i * (i - 1) / 2 + j];
+            cd s = L.d[j] * x;
+#pragma unroll
+            for (int k = j + 1; k < i; ++k) cfma(s, L.l[i * (i - 1) / 2 + k], D.l[k * (k - 1) / 2 + j]);
+            D.l[i * (i - 1) / 2 + j] = -L.d[i] * s;
+        }
+    }
+    H6 out;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        double t = D.d[j] * D.d[j];
+#pragma unroll
+        for (int k = j + 1; k < 6; ++k) {
+            const cd x = D.l[k * (k - 1) / 2 + j];
+            t = fma(x.re, x.re, t);
+            t = fma(x.im, x.im, t);
+        }
+        out.d[j] = t;
+#pragma unroll
+        for (int i = j + 1; i < 6; ++i) {
+            cd s = D.d[i] * D.l[i * (i - 1) / 2 + j];
+#pragma unroll
+            for (int k = i + 1; k < 6; ++k) cfma_cj(s, D.l[k * (k - 1) / 2 + i], D.l[k * (k - 1) / 2 + j]);
+            out.l[i * (i - 1) / 2 + j] = s;
+        }
+    }
+    return out;
 }
 
-__device__ __forceinline__ void put_real(double* base, long vh, long i, int r, double v) {
-    base[((long)(r >> 1) * vh + i) * 2 + (r & 1)] = v;
+// 36 reals of a packed hermitian block at real offset off, less `one` on the diagonal
+__device__ __forceinline__ void store_h6(double* base, long vh, long i, int off, const H6& h, double one) {
+    double r[36];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) r[k] = h.d[k] - one;
+#pragma unroll
+    for (int k = 0; k < 15; ++k) {
+        r[6 + 2 * k] = h.l[k].re;
+        r[7 + 2 * k] = h.l[k].im;
+    }
+    store_reals<P64, 36>(base, vh, i, off, r);
 }
 
-// One thread per site of parity `par`:
+// One thread per site of parity PAR and chirality (threadIdx.y):
 //   A_c = 1 - kappa csw [ i s1 (x) a1 + i s2 (x) a2 + i s3 (x) a3 ],
 //   a1 = F_yz + s F_xt,  a2 = -F_xz + s F_yt,  a3 = F_xy + s F_zt  (s = +1 / -1 per chirality),
-// which is the chirality-block form of 1 - kappa csw sum_{mu<nu} g_mu g_nu F_munu.
-// Writes A (packed hermitian, 72 reals/site); on even sites also the light inverse
-// blocks B_c = (A_c + i s mu_t)^-1 (144 reals) and/or the heavy A_c, D_c (144).
-__global__ void k_clover(Geom g, const void* g0, const void* g1, int par, double kappa, double csw,
-                         double mu_t, double mubar_t, double epsbar_t, double* outA,
-                         double* outB, double* outH) {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.vh) return;
-    const void* gauge[2] = {g0, g1};
-    const Coord c = cb_coords(g, i, par);
-    const int xc[4] = {c.x, c.y, c.z, c.t};
-    const double kc = kappa * csw;
-    M3 F[6];
-    int n = 0;
-    for (int mu = 0; mu < 4; ++mu)
-        for (int nu = mu + 1; nu < 4; ++nu) F[n++] = clover_leaf(g, gauge, mu, nu, xc);
-    // plane order: 0 xy, 1 xz, 2 xt, 3 yz, 4 yt, 5 zt
-    for (int cb = 0; cb < 2; ++cb) {
-        const double s = cb == 0 ? 1.0 : -1.0;
-        cd A[36];
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) {
-                const cd a1 = F[3].m[3 * a + b] + s * F[2].m[3 * a + b];
-                const cd a2 = s * F[4].m[3 * a + b] - F[1].m[3 * a + b];
-                const cd a3 = F[0].m[3 * a + b] + s * F[5].m[3 * a + b];
-                const double id = (a == b) ? 1.0 : 0.0;
-                // S = [[ i a3, i a1 + a2 ], [ i a1 - a2, -i a3 ]]
-                A[6 * (0 + a) + (0 + b)] = C(id, 0.0) - kc * mul_i(a3);
-                A[6 * (0 + a) + (3 + b)] = -kc * (mul_i(a1) + a2);
-                A[6 * (3 + a) + (0 + b)] = -kc * (mul_i(a1) - a2);
-                A[6 * (3 + a) + (3 + b)] = C(id, 0.0) + kc * mul_i(a3);
+// which is the chirality-block form of 1 - kappa csw sum_{mu<nu} g_mu g_nu F_munu:
+//   [[ 1 - kc i a3, -kc (i a1 + a2) ], [ -kc (i a1 - a2), 1 + kc i a3 ]].
+// Writes A (packed hermitian, 72 reals/site) over F, which both threads of a site
+// have read by then; on even sites also the light inverse blocks
+// B_c = (A_c + i s mu_t)^-1 = A D - i s mu_t D, D = (A^2 + mu_t^2)^-1 (144 reals),
+// and/or the heavy A_c - 1, D_c - 1 (144; the deviation from the identity keeps
+// 16-bit rounding relative to it).  A commutes with D, so A D is hermitian and half
+// of it is computed.
+template <int PAR>
+__global__ void __launch_bounds__(128) k_clover(const __grid_constant__ CloverArgs p) {
+    const long vh = p.g.vh, i = (long)blockIdx.x * 64 + threadIdx.x;
+    const int cb = threadIdx.y;
+    const double s = cb == 0 ? 1.0 : -1.0;
+    H6 A;
+    if (i < vh) {
+        auto F = [&](int plane, int k) { return p.F[PAR][2 * ((plane * 5 + (k >> 1)) * vh + i) + (k & 1)]; };
+        // per combination: imaginary diagonal, then entries (1,0), (2,0), (2,1)
+        double a1[9], a2[9], a3[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            a1[k] = F(3, k) + s * F(2, k);
+            a2[k] = s * F(4, k) - F(1, k);
+            a3[k] = F(0, k) + s * F(5, k);
+        }
+        const double kc = p.kc;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            A.d[r] = 1.0 + kc * a3[r];
+            A.d[3 + r] = 1.0 - kc * a3[r];
+        }
+        auto full = [](const double (&v)[9], int r, int j) {   // entry (r, j) of an antihermitian matrix
+            if (r == j) return C(0.0, v[r]);
+            const int e = 3 + 2 * (r > j ? r * (r - 1) / 2 + j : j * (j - 1) / 2 + r);
+            return r > j ? C(v[e], v[e + 1]) : C(-v[e], v[e + 1]);
+        };
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                if (j < r) {
+                    const cd z = full(a3, r, j);
+                    A.l[r * (r - 1) / 2 + j] = C(kc * z.im, -kc * z.re);             // -kc i z
+                    A.l[(r + 3) * (r + 2) / 2 + j + 3] = C(-kc * z.im, kc * z.re);   // +kc i z
+                }
+                const cd u = full(a1, r, j), v = full(a2, r, j);
+                A.l[(r + 3) * (r + 2) / 2 + j] = C(kc * (u.im + v.re), kc * (v.im - u.re));   // -kc (i u - v)
             }
-        // packed hermitian store
-        for (int r = 0; r < 6; ++r) put_real(outA, g.vh, i, 36 * cb + r, A[7 * r].re);
-        for (int r = 1; r < 6; ++r)
+    }
+    __syncthreads();
+    if (i >= vh) return;
+    store_h6(p.F[PAR], vh, i, 36 * cb, A, 0.0);
+    if (PAR != 0) return;
+    const H6 A2 = mul_commuting(A, A);
+    if (p.outB != nullptr) {
+        const H6 D = hpd6_inverse(A2, p.mu_t * p.mu_t);
+        const H6 AD = mul_commuting(A, D);
+        const double m = s * p.mu_t;
+        double2* out = reinterpret_cast<double2*>(p.outB) + (long)(36 * cb) * vh + i;
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+            out[(7 * r) * vh] = make_double2(AD.d[r], -m * D.d[r]);
+#pragma unroll
             for (int j = 0; j < r; ++j) {
-                put_real(outA, g.vh, i, 36 * cb + herm_off(r, j), A[6 * r + j].re);
-                put_real(outA, g.vh, i, 36 * cb + herm_off(r, j) + 1, A[6 * r + j].im);
+                const cd x = AD.l[r * (r - 1) / 2 + j], y = D.l[r * (r - 1) / 2 + j];
+                out[(6 * r + j) * vh] = make_double2(fma(m, y.im, x.re), fma(-m, y.re, x.im));
+                out[(6 * j + r) * vh] = make_double2(fma(-m, y.im, x.re), fma(-m, y.re, -x.im));
             }
-        if (par != 0) continue;
-        // A^2 (hermitian)
-        cd A2[36];
-        for (int r = 0; r < 6; ++r)
-            for (int j = 0; j < 6; ++j) {
-                cd t = C(0.0, 0.0);
-                for (int k = 0; k < 6; ++k) cfma(t, A[6 * r + k], A[6 * k + j]);
-                A2[6 * r + j] = t;
-            }
-        if (outB != nullptr) {
-            cd D[36];
-            for (int k = 0; k < 36; ++k) D[k] = A2[k];
-            for (int r = 0; r < 6; ++r) D[7 * r].re += mu_t * mu_t;
-            hpd6_inverse(D);
-            // B = (A - i s mu_t) D
-            for (int r = 0; r < 6; ++r)
-                for (int j = 0; j < 6; ++j) {
-                    cd t = C(0.0, 0.0);
-                    for (int k = 0; k < 6; ++k) {
-                        cd a = A[6 * r + k];
-                        if (k == r) a.im -= s * mu_t;
-                        cfma(t, a, D[6 * k + j]);
-                    }
-                    put_real(outB, g.vh, i, 72 * cb + 2 * (6 * r + j), t.re);
-                    put_real(outB, g.vh, i, 72 * cb + 2 * (6 * r + j) + 1, t.im);
-                }
         }
-        if (outH != nullptr) {
-            cd D[36];
-            for (int k = 0; k < 36; ++k) D[k] = A2[k];
-            for (int r = 0; r < 6; ++r) D[7 * r].re += mubar_t * mubar_t - epsbar_t * epsbar_t;
-            hpd6_inverse(D);
-            // [A_c - 1 36][D_c - 1 36] per chirality, both packed hermitian (the
-            // deviation from the identity keeps 16-bit rounding relative to it)
-            for (int r = 0; r < 6; ++r) {
-                put_real(outH, g.vh, i, 72 * cb + r, A[7 * r].re - 1.0);
-                put_real(outH, g.vh, i, 72 * cb + 36 + r, D[7 * r].re - 1.0);
-            }
-            for (int r = 1; r < 6; ++r)
-                for (int j = 0; j < r; ++j) {
-                    put_real(outH, g.vh, i, 72 * cb + herm_off(r, j), A[6 * r + j].re);
-                    put_real(outH, g.vh, i, 72 * cb + herm_off(r, j) + 1, A[6 * r + j].im);
-                    put_real(outH, g.vh, i, 72 * cb + 36 + herm_off(r, j), D[6 * r + j].re);
-                    put_real(outH, g.vh, i, 72 * cb + 36 + herm_off(r, j) + 1, D[6 * r + j].im);
-                }
-        }
+    }
+    if (p.outH != nullptr) {
+        const H6 D = hpd6_inverse(A2, p.mubar_t * p.mubar_t - p.epsbar_t * p.epsbar_t);
+        store_h6(p.outH, vh, i, 72 * cb, A, 1.0);
+        store_h6(p.outH, vh, i, 72 * cb + 36, D, 1.0);
     }
 }
 
@@ -327,11 +455,29 @@ cudaError_t launch_clover_from64(void* dst, const double* src, long vh, int nrea
     return cudaGetLastError();
 }
 
-cudaError_t launch_clover(const Geom& g, const void* g0, const void* g1, int par, double kappa, double csw,
-                          double mu_t, double mubar_t, double epsbar_t, double* outA, double* outB,
-                          double* outH, cudaStream_t st) {
-    k_clover<<<(unsigned)((g.vh + 63) / 64), 64, 0, st>>>(g, g0, g1, par, kappa, csw, mu_t, mubar_t,
-                                                          epsbar_t, outA, outB, outH);
+cudaError_t launch_clover(const Geom& g, const void* g0, const void* g1, double kappa, double csw, double mu_t,
+                          double mubar_t, double epsbar_t, double* outA0, double* outA1, double* outB, double* outH,
+                          cudaStream_t st) {
+    CloverArgs p{};
+    p.g = g;
+    p.gauge[0] = g0;
+    p.gauge[1] = g1;
+    p.leaf = outB;
+    p.F[0] = outA0;
+    p.F[1] = outA1;
+    p.kc = kappa * csw;
+    p.mu_t = mu_t;
+    p.mubar_t = mubar_t;
+    p.epsbar_t = epsbar_t;
+    p.outB = outB;
+    p.outH = outH;
+    const unsigned nb64 = (unsigned)((g.vh + 63) / 64), nb128 = (unsigned)((g.vh + 127) / 128);
+    for (p.plane0 = 0; p.plane0 < 6; p.plane0 += 2) {
+        k_leaves<<<dim3(nb64, 4), 64, 0, st>>>(p);
+        k_field<<<dim3(nb128, 4), 128, 0, st>>>(p);
+    }
+    k_clover<0><<<nb64, dim3(64, 2), 0, st>>>(p);
+    k_clover<1><<<nb64, dim3(64, 2), 0, st>>>(p);
     return cudaGetLastError();
 }
 

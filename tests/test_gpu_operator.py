@@ -300,3 +300,34 @@ def test_mass_preconditioned_W_hat(prec):
                 assert rel(lat.apply_dw(tm.TM_WHAT_SQ, psi), wsq) < 2 * DW_TOL
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("heavy", [False, True], ids=["light", "both"])
+@pytest.mark.parametrize("dims", [(2, 6, 10, 18), (12, 10, 6, 22)], ids=lambda d: "x".join(map(str, d)))
+def test_clover_and_inverses_over_many_blocks(dims, heavy):
+    """The clover term (built over F in place), its light and heavy inverses and
+    the double-word passes on lattices of many ragged blocks, an extent of 2 among
+    them, with and without the heavy inverse."""
+    import torch
+    kw = dict(mu=MU, mubar=MUBAR, epsbar=EPSBAR) if heavy else dict(mu=MU)
+    u = F.gauge_field(dims, 1700 + sum(dims))
+    op = D.TwistedMassClover(u, dims, KAPPA, CSW, **kw)
+    lat = Lat(u, dims, KAPPA, CSW, **kw)
+    tm = lat.tm
+    try:
+        for par, sites in ((0, op.geo.even), (1, op.geo.odd)):
+            out = torch.empty(lat.vh * 2 * 36 * 2, dtype=torch.float64, device="cuda:0")
+            tm.tm_clover_export(lat.ctx, par, out)
+            got = out.cpu().numpy().view(np.complex128).reshape(lat.vh, 2, 6, 6)
+            A = op.A[sites]
+            assert rel(got, np.stack([A[:, :6, :6], A[:, 6:, 6:]], axis=1)) < 1e-14
+        psi = F.odd_spinor(dims, 7)
+        cases = [(tm.TM_QHAT_PLUS, op.Qhat(psi, +1), psi), (tm.TM_QHAT_MINUS, op.Qhat(psi, -1), psi)]
+        if heavy:
+            psih = F.odd_spinor(dims, 8, 2)
+            cases += [(tm.TM_QH, op.Qhat_heavy(psih, +1), psih), (tm.TM_QH_DAG, op.Qhat_heavy(psih, -1), psih)]
+        for code, ref, x in cases:
+            assert rel(lat.apply(code, 0, x), ref) < tol(0), code
+            assert rel(lat.apply_dw(code, x), ref) < DW_TOL, code
+    finally:
+        lat.close()
