@@ -367,17 +367,45 @@ static const void* clovH_ptr(const tm_ctx* c, int P) {
 // ---------------------------------------------------------------------------
 // operator application
 // ---------------------------------------------------------------------------
+// Sites per parity up to which the direct passes run as the kernel that splits a site
+// over several warps (dslash_split.cu).  M_hat^dagger M_hat, calls back to back, direct
+// / split, us, at 4,096 / 10,000 / 20,736 sites:
+//   light FP32 20.6 / 16.0, 20.7 / 18.6, 22.7 / 22.7; light FP16 22.7 / 16.7,
+//   22.6 / 20.7, 22.8 / 22.7; light FP64 156 / 62, 161 / 132, 233 / 216 (38,416 sites:
+//   305 / 348); heavy FP32 24.8 / 20.7, 27.7 / 34.9; heavy FP16 26.9 / 22.7,
+//   28.8 / 39.1; heavy FP64 260 / 102, 313 / 294, 487 / 498.
+static long split_limit(int P, int nf) {
+    if (P == P64) return nf == 1 ? 24576 : 12288;
+    return nf == 1 ? 12288 : 6144;
+}
+
+// Kernel of a pass: the tuned choice (0 direct, 1 staged), or the split kernel in place
+// of the direct one on a small lattice.
+enum PassKernel { PK_DIRECT = 0, PK_STAGED = 1, PK_SPLIT = 2 };
+static int pass_kernel(int P, long vh, int nf, int variant) {
+    return variant == PK_DIRECT && P != PDF && vh <= split_limit(P, nf) ? PK_SPLIT : variant;
+}
+template <int P, int NF>
+static int pass_kernel(const tm_ctx* c, int kind) {
+    return P == PDF ? 0 : pass_kernel(P, c->vh, NF, c->variant[P][NF - 1][kind]);
+}
+
 // blocks of a pass: one thread per site, except the direct two-flavour even pass
-// (a thread per site and flavour)
-static int pass_nblk(int P, long vh, int nf, int kind, int staged) {
-    return staged ? nblk(vh, STAGED_BS) : nblk(nf == 2 && kind == K1_EO_INV ? 2 * vh : vh, dslash_bs(P));
+// (a thread per site and flavour) and the double-word passes (likewise)
+static int pass_nblk(int P, long vh, int nf, int kind, int kernel) {
+    if (P == PDF) return nblk((long)nf * vh, DSLASH_BS);
+    if (kernel == PK_SPLIT) return nblk(vh, SPLIT_SITES);
+    return kernel == PK_STAGED ? nblk(vh, STAGED_BS) : nblk(nf == 2 && kind == K1_EO_INV ? 2 * vh : vh, dslash_bs(P));
 }
 
 // launch one pass in the variant the context chose for (P, NF, KIND)
 template <int P, int NF, int KIND, int NP>
-static cudaError_t launch_pass(int variant, const OpBatch<NP>& b, int nb, cudaStream_t st) {
+static cudaError_t launch_pass(int kernel, const OpBatch<NP>& b, int nb, cudaStream_t st) {
     if constexpr (P != P64 && P != PDF) {
-        if (variant) return launch_dslash_staged<P, NF, KIND, NP>(b, nb, st);
+        if (kernel == PK_STAGED) return launch_dslash_staged<P, NF, KIND, NP>(b, nb, st);
+    }
+    if constexpr (NP == 1 && P != PDF) {
+        if (kernel == PK_SPLIT) return launch_dslash_split<P, NF, KIND>(b, nb, st);
     }
     return launch_dslash<P, NF, KIND, NP>(b, nb, st);
 }
@@ -386,8 +414,7 @@ static OpProb make_prob(const tm_ctx* c, int P, int nf, int kind, int sign, void
                         const void* loc, SolverCtl* ctl, bool fuse, double rho = 0.0) {
     OpProb p{};
     p.g = c->g;
-    // (the double-word passes run a thread per site and flavour)
-    p.nblk = P == PDF ? nblk((long)nf * c->vh, DSLASH_BS) : pass_nblk(P, c->vh, nf, kind, c->variant[P][nf - 1][kind]);
+    p.nblk = pass_nblk(P, c->vh, nf, kind, P == PDF ? 0 : pass_kernel(P, c->vh, nf, c->variant[P][nf - 1][kind]));
     p.bc_t = (float)c->params.bc_t;
     p.gauge[0] = gauge_ptr(c, P, 0);
     p.gauge[1] = gauge_ptr(c, P, 1);
@@ -412,17 +439,19 @@ static OpProb make_prob(const tm_ctx* c, int P, int nf, int kind, int sign, void
 // fin != FIN_NONE fuses ||out||^2.
 template <int P, int NF>
 static cudaError_t schur(const tm_ctx* c, int sign, void* out, const void* in, void* te, cudaStream_t st,
-                         SolverCtl* ctl, int fin, double rho = 0.0) {
+                         SolverCtl* ctl, int fin, double rho = 0.0, bool chained = false) {
     OpBatch<1> b{};
     b.n = 1;
+    b.chained = chained;
     b.fin = FIN_NONE;
     b.p[0] = make_prob(c, P, NF, K1_EO_INV, sign, te, in, nullptr, ctl, false);
     b.blk_start[0] = 0;
     b.blk_start[1] = b.p[0].nblk;
-    const int v1 = P == PDF ? 0 : c->variant[P][NF - 1][K1_EO_INV];
-    const int v2 = P == PDF ? 0 : c->variant[P][NF - 1][K2_OE_LOCAL];
+    const int v1 = pass_kernel<P, NF>(c, K1_EO_INV);
+    const int v2 = pass_kernel<P, NF>(c, K2_OE_LOCAL);
     cudaError_t e = launch_pass<P, NF, K1_EO_INV, 1>(v1, b, b.p[0].nblk, st);
     if (e != cudaSuccess) return e;
+    b.chained = true;
     b.fin = fin;
     b.p[0] = make_prob(c, P, NF, K2_OE_LOCAL, sign, out, te, in, ctl, fin != FIN_NONE, rho);
     b.blk_start[1] = b.p[0].nblk;
@@ -445,7 +474,7 @@ static cudaError_t normal_op(const tm_ctx* c, tm_op op, void* out, const void* i
     const double rt = is_what(op) ? 2.0 * c->params.kappa * c->params.rho : 0.0;
     cudaError_t e = schur<P, NF>(c, s1, mid, in, te, st, ctl, fin, s1 * rt);
     if (e != cudaSuccess) return e;
-    return schur<P, NF>(c, s2, out, mid, te, st, ctl, FIN_NONE, s2 * rt);
+    return schur<P, NF>(c, s2, out, mid, te, st, ctl, FIN_NONE, s2 * rt, true);
 }
 
 template <int P, int NF>
@@ -542,7 +571,7 @@ static cudaError_t even_t(const tm_ctx* c, int sign, void* out, const void* in, 
     b.p[0] = make_prob(c, P, NF, K1_EO_INV, sign, out, in, nullptr, nullptr, false);
     b.blk_start[0] = 0;
     b.blk_start[1] = b.p[0].nblk;
-    return launch_pass<P, NF, K1_EO_INV, 1>(c->variant[P][NF - 1][K1_EO_INV], b, b.p[0].nblk, st);
+    return launch_pass<P, NF, K1_EO_INV, 1>(pass_kernel<P, NF>(c, K1_EO_INV), b, b.p[0].nblk, st);
 }
 
 extern "C" tm_status tm_apply_even(tm_ctx* c, tm_op op, tm_prec prec, void* out, const void* in, void* stream) {
@@ -655,6 +684,8 @@ static tm_status kernel_times_t(tm_ctx* c, int sign, const void* in, int reps, d
     void *te = nullptr, *out = nullptr;
     CKS(ws_get(c, WS_APPLY_TE, spinor_bytes(P, 12 * NF, c->vh), &te));
     CKS(ws_get(c, WS_APPLY_MID, spinor_bytes(P, 12 * NF, c->vh), &out));
+    v1 = pass_kernel(P, c->vh, NF, v1);
+    v2 = pass_kernel(P, c->vh, NF, v2);
     OpBatch<1> b{};
     b.n = 1;
     b.fin = FIN_NONE;

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
     __shared__ double sh[BS / 32];
     const int k = find_problem<NP>(b, blockIdx.x);
     const OpProb& pr = b.p[k];
+    pdl_wait();
     if (pr.ctl != nullptr && pr.ctl->flag != CTL_RUN) return;
     const int lb = blockIdx.x - b.blk_start[k];
     const long i = (long)lb * BS + threadIdx.x;
@@ -229,8 +230,7 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
 
 template <int P, int NF, int KIND, int NP>
 cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st) {
-    dslash_kernel<P, NF, KIND, NP, dslash_bs(P)><<<nblocks, dslash_bs(P), 0, st>>>(b);
-    return cudaGetLastError();
+    return launch_chained(dslash_kernel<P, NF, KIND, NP, dslash_bs(P)>, nblocks, dslash_bs(P), 0, st, b.chained, b);
 }
 
 #define TM_INST(P, NF, KIND, NP) \

@@ -244,6 +244,7 @@ template <int NF, int KIND>
 __global__ void __launch_bounds__(DSLASH_BS, 4) dslash_dw_kernel(const __grid_constant__ OpBatch<1> b) {
     extern __shared__ __align__(16) float4 dw_smem[];
     const OpProb& pr = b.p[0];
+    pdl_wait();
     if (pr.ctl != nullptr && pr.ctl->flag != CTL_RUN) return;
     const long gt = (long)blockIdx.x * DSLASH_BS + threadIdx.x;
     const long i = NF == 2 ? gt >> 1 : gt;
@@ -418,8 +419,7 @@ cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st);
         const cudaError_t e = cudaFuncSetAttribute(dslash_dw_kernel<NF, KIND>,                     \
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM); \
         if (e != cudaSuccess) return e;                                                            \
-        dslash_dw_kernel<NF, KIND><<<nblocks, DSLASH_BS, DW_SMEM, st>>>(b);                        \
-        return cudaGetLastError();                                                                 \
+        return launch_chained(dslash_dw_kernel<NF, KIND>, nblocks, DSLASH_BS, DW_SMEM, st, b.chained, b); \
     }
 TM_DW_INST(1, K1_EO_INV)
 TM_DW_INST(1, K2_OE_LOCAL)

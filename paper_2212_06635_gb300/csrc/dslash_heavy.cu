@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, KIND>())) dslash_heav
     using R = typename PT<P>::R;
     const int k = find_problem<NP>(b, blockIdx.x);
     const OpProb& pr = b.p[k];
+    pdl_wait();
     if (pr.ctl != nullptr && pr.ctl->flag != CTL_RUN) return;
     const int lb = blockIdx.x - b.blk_start[k];
     const long gt = (long)lb * BS + threadIdx.x;
@@ -196,8 +197,7 @@ cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st);
 #define TM_HEAVY_INST(P, KIND)                                                                        \
     template <>                                                                                       \
     cudaError_t launch_dslash<P, 2, KIND, 1>(const OpBatch<1>& b, int nblocks, cudaStream_t st) {     \
-        dslash_heavy_kernel<P, KIND, 1, dslash_bs(P)><<<nblocks, dslash_bs(P), 0, st>>>(b);          \
-        return cudaGetLastError();                                                                    \
+        return launch_chained(dslash_heavy_kernel<P, KIND, 1, dslash_bs(P)>, nblocks, dslash_bs(P), 0, st, b.chained, b); \
     }
 TM_HEAVY_INST(P64, K1_EO_INV)
 TM_HEAVY_INST(P32, K1_EO_INV)

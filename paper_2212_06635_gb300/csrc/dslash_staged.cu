@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(BS) dslash_staged_kernel(const __grid_constant
 
     const int k = find_problem<NP>(b, blockIdx.x);
     const OpProb& pr = b.p[k];
+    pdl_wait();
     if (pr.ctl != nullptr && pr.ctl->flag != CTL_RUN) return;
     const int lb = blockIdx.x - b.blk_start[k];
     const int t = threadIdx.x;
@@ -359,8 +360,7 @@ cudaError_t launch_dslash_staged(const OpBatch<NP>& b, int nblocks, cudaStream_t
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    dslash_staged_kernel<P, NF, KIND, NP, BS><<<nblocks, BS, bytes, st>>>(b);
-    return cudaGetLastError();
+    return launch_chained(dslash_staged_kernel<P, NF, KIND, NP, BS>, nblocks, BS, bytes, st, b.chained, b);
 }
 
 #define TM_SINST(P, NF, KIND, NP) \

@@ -360,6 +360,7 @@ struct OpProb {
 template <int NP>
 struct OpBatch {
     int n;
+    bool chained;            // launched as a later kernel of a chain (launch_chained)
     int fin;                 // finalisation of the fused norm (FinOp)
     int blk_start[NP + 1];
     OpProb p[NP];

@@ -13,12 +13,46 @@ constexpr int DSLASH_BS = 128;   // direct stencil kernel
 constexpr int dslash_bs(int P) { return P == P64 ? 64 : DSLASH_BS; }
 constexpr int STAGED_BS = 64;    // shared-memory staged stencil kernel
 constexpr int BLAS_BS = 256;
-constexpr int MIN_BS = 64;       // smallest block size of any reducing kernel (sizes the partials)
+constexpr int SPLIT_SITES = 32;  // sites per block of the small-lattice stencil kernel
+constexpr int MIN_BS = 32;       // fewest sites per block of any reducing kernel (sizes the partials)
 
 enum DslashKind { K1_EO_INV = 0, K2_OE_LOCAL = 1 };
 
 // FinOp codes beyond those in tm_internal.h
 enum { FIN_PP = 4, FIN_CG_UPDATE = 5, FIN_MS_UPDATE = 6 };
+
+// ---------------------------------------------------------------------------
+// Chained launches (programmatic dependent launch).  A kernel launched with
+// `chained` may start while the kernel before it in the stream still runs: until
+// pdl_wait() it reads only data that no kernel of the chain writes (links, clover
+// blocks); pdl_wait() returns when the kernel before has completed and its writes are
+// visible.  The first kernel of a chain is launched without it, so everything
+// before the chain has completed by then.  Only the small-lattice kernel lets the
+// next one start early (pdl_trigger): on larger grids blocks of the next kernel then
+// sit between the last ones of this, and its own blocks end up unevenly spread (heavy
+// FP64 at 12^3x24: 484 -> 666 us).  Without it a chained launch follows as this
+// kernel's blocks end, which still hides the launch: calls back to back, M_hat^dagger
+// M_hat light FP32 at 12^3x24 32.9 -> 20.7 us, light FP16 at 16^3x32 41.2 -> 35.1 us,
+// heavy FP16 at 24^3x48 270.5 -> 257.5 us, light FP16 at 32^3x64 419 -> 409 us.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(Params...), int grid, int block, size_t smem, cudaStream_t st,
+                                  bool chained, const Args&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 // ---------------------------------------------------------------------------
 // solver scalar finalisers (run by one thread of the last block of a reduction)
@@ -174,6 +208,10 @@ cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st);
 // shared-memory staged variant (FP32 / 16-bit storage), STAGED_BS threads per block
 template <int P, int NF, int KIND, int NP>
 cudaError_t launch_dslash_staged(const OpBatch<NP>& b, int nblocks, cudaStream_t st);
+
+// several warps per site, for small lattices (dslash_split.cu), SPLIT_SITES sites per block
+template <int P, int NF, int KIND>
+cudaError_t launch_dslash_split(const OpBatch<1>& b, int nblocks, cudaStream_t st);
 
 // p = r + beta p (+ ||p||^2 when the problem has a shift)       v = {p, r}
 template <int P, int NC, int NP>

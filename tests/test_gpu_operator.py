@@ -331,3 +331,23 @@ def test_clover_and_inverses_over_many_blocks(dims, heavy):
             assert rel(lat.apply_dw(code, x), ref) < DW_TOL, code
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("dims", [(12, 10, 10, 18), (14, 12, 18, 22)], ids=lambda d: "x".join(map(str, d)))
+def test_operators_on_both_sides_of_the_small_lattice_line(dims):
+    """10,800 sites per parity: the light passes split a site over several warps, the
+    heavy FP32 / 16-bit ones take a thread per site; 33,264 sites: all take a thread
+    per site, with a ragged last block."""
+    u = F.gauge_field(dims, 1800 + sum(dims))
+    op = D.TwistedMassClover(u, dims, KAPPA, CSW, mu=MU, mubar=MUBAR, epsbar=EPSBAR)
+    lat = Lat(u, dims, KAPPA, CSW, mu=MU, mubar=MUBAR, epsbar=EPSBAR)
+    tm = lat.tm
+    psi, psih = F.odd_spinor(dims, 7), F.odd_spinor(dims, 8, 2)
+    try:
+        refs = [(tm.TM_QHAT_MINUS, op.Qhat(psi, -1), psi, 1), (tm.TM_MDAGM, op.MdagM(psi), psi, 2),
+                (tm.TM_QH, op.Qhat_heavy(psih, +1), psih, 1), (tm.TM_QH_SQ, op.heavy_sq(psih), psih, 2)]
+        for prec in range(4):
+            for code, ref, x, n in refs:
+                assert rel(lat.apply(code, prec, x), ref) < tol(prec, n), (prec, code)
+    finally:
+        lat.close()
