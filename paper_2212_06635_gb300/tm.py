@@ -153,12 +153,12 @@ def _check(status):
 
 def ptr(x):
     """Address of a tensor / array / ctypes object / int."""
+    if hasattr(x, "data_ptr"):
+        return x.data_ptr()
     if x is None:
         return None
     if isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
-        return x.data_ptr()
     if isinstance(x, np.ndarray):
         if not x.flags["C_CONTIGUOUS"]:
             raise ValueError("array must be C contiguous")
@@ -166,15 +166,34 @@ def ptr(x):
     return ct.addressof(x)
 
 
-def _stream(stream):
-    if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
-        except ImportError:
-            pass
+# torch.cuda once it is known to be usable (looked up on the first call that needs it)
+_cuda = None
+_raw_stream = None
+
+
+def _torch_cuda():
+    global _cuda, _raw_stream
+    try:
+        import torch
+    except ImportError:
         return None
+    if not torch.cuda.is_available():
+        return None
+    _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    _cuda = torch.cuda
+    return _cuda
+
+
+def _stream(stream):
+    # the current stream through is_available() and a Stream object took 3.8 us, a fifth
+    # of an operator call on a small lattice; the raw handle takes 0.3 us
+    if stream is None:
+        cuda = _cuda or _torch_cuda()
+        if cuda is None:
+            return None
+        if _raw_stream is not None:
+            return _raw_stream(cuda.current_device())
+        return cuda.current_stream().cuda_stream
     if hasattr(stream, "cuda_stream"):
         return stream.cuda_stream
     return stream
