@@ -26,11 +26,25 @@
 // Layout and mapping.  Fields are native (structure of arrays over the Vh
 // sites of one parity; 32- or 16-bit storage), math is FP32, the force is the
 // canonical FP64 link layout and is read, added to and written once.  A block of
-// 32 x 4 x 2 threads covers the 64 lexicographic sites [64 b, 64 b + 64): the
-// 32 half-site indices 32 b .. 32 b + 31 of both parities (z), one direction mu
-// per warp (y), so every warp's load of a field vector is one contiguous
-// 512-byte span (16 B per site) and its neighbour loads are the same span
-// shifted.  The four warps of one parity reuse X(x), Y(x) through L1.
+// 32 x 2 x 2 threads covers 64 sites: 32 half-site indices of both parities (z),
+// directions 0, 1 or 2, 3 of a site per thread (y), so every warp's load of a field
+// vector is one contiguous 512-byte span (16 B per site) and its neighbour loads are
+// the same span shifted.  Two directions a thread load the site's own X, Y once for
+// both (36 vectors instead of 48 per pair); 24^3x48, 12 two-flavour pairs: one
+// direction a thread 1609 us FP32 / 1218 us FP16, two 1182 / 981 us, four 1205 / 1178 us.
+//
+// Site order.  A site's spinors are read for its own links and as the forward
+// neighbours of four other sites.  In lexicographic order the +t neighbour is a time
+// slice away, and where a slice of all pairs is a good part of the L2 the blocks that
+// share it run too far apart (DRAM reads 1.8 x the fields at 64 MB a slice).  Such
+// lattices are walked in tiles of up to 8 time slices, t inside z (ForceArgs::tt): 1182 ->
+// 1118 us (tiles of 4 / 16 / 48: 1123 / 1177 / 1279 us).  At 33 MB a slice both orders
+// take the same time, and below the plain one is faster (12 pairs of one flavour,
+// 32 MB: 643 against 670 us), so the line is at 40 MB.
+//
+// Measured and not used: loads issued one or two terms ahead in registers (168, 3
+// blocks: 1144 us), prefetch.global.L2 of the next pair (1117 us), the force added
+// through shared memory in contiguous runs (1188 us).
 //
 // Bytes per launch (algorithmic): each field read once (2 n V spinors), the FP32
 // links once (4 V x 12 reals), the force read and written once (2 x 4 V x 18 x 8).
@@ -90,56 +104,48 @@ __device__ __forceinline__ void force_outer2(cpx<float> (&w)[9], const cpx<float
         }
 }
 
+// Neighbour of site c in direction mu (checkerboard index of the other parity), and
+// whether the hop crosses the lattice's edge
+template <int MU>
+__device__ __forceinline__ long force_neighbour(const Geom& g, const Coord& c, bool& wrap) {
+    const int x = MU == 0 ? c.x : (MU == 1 ? c.y : (MU == 2 ? c.z : c.t));
+    const int L = MU == 0 ? g.X : (MU == 1 ? g.Y : (MU == 2 ? g.Z : g.T));
+    wrap = x + 1 == L;
+    const int n = wrap ? 0 : x + 1;
+    return cb_index(g, MU == 0 ? n : c.x, MU == 1 ? n : c.y, MU == 2 ? n : c.z, MU == 3 ? n : c.t);
+}
+
+// One field pair and flavour f on link (x, MU): w += c_k [ X(x+mu) (x) ((1 - g_mu) Y(x))^*
+// + ((1 + g_mu) Y(x+mu)) (x) X(x)^* ], xs, ys the site's own spinors (scales sx, sy),
+// xn, yn the fields of the other parity, j the neighbour.
 // G5: the Y fields enter as g5 Y.  P_s(g5 B) = B_up - s G B_down = P_-s(B), so
 // g5 only flips the projection sign of the Y spinors.
 template <int P, int NF, int MU, bool G5>
-__device__ __forceinline__ void force_link(const ForceArgs& a, long i, int par, const Coord& c) {
+__device__ __forceinline__ void force_pair(cpx<float> (&w)[9], const void* xn, const void* yn, long vh, long j, int f,
+                                           const cpx<float>* xs, float sx, const cpx<float>* ys, float sy, float ck) {
     constexpr int SY1 = G5 ? +1 : -1;   // sign of Y(x) in the forward term
     constexpr int SY2 = G5 ? -1 : +1;   // sign of Y(x+mu) in the backward term
-    const Geom& g = a.g;
-    int xf = c.x, yf = c.y, zf = c.z, tf = c.t;
-    float ph = 1.f;
-    if (MU == 0) xf = (c.x + 1 == g.X) ? 0 : c.x + 1;
-    if (MU == 1) yf = (c.y + 1 == g.Y) ? 0 : c.y + 1;
-    if (MU == 2) zf = (c.z + 1 == g.Z) ? 0 : c.z + 1;
-    if (MU == 3) {
-        if (c.t + 1 == g.T) { tf = 0; ph = a.bc_t; } else tf = c.t + 1;
-    }
-    const long j = cb_index(g, xf, yf, zf, tf);
-    const long vh = g.vh;
-    cpx<float> w[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) w[e] = C(0.f, 0.f);
+    cpx<float> p[12];
+    cpx<float> hu[2][3], hv[2][3];
+    float sn;
+    // forward hop at x
+    force_load<P, NF>(xn, vh, j, f, p, sn);
+    force_half<MU, -1>(hu, p, 1.f);
+    force_half<MU, SY1>(hv, ys, ck * sn * sy);
+    force_outer2(w, hu, hv);
+    // backward hop at x+mu (through U_mu(x)^dagger)
+    force_load<P, NF>(yn, vh, j, f, p, sn);
+    force_half<MU, SY2>(hu, p, 1.f);
+    force_half<MU, +1>(hv, xs, ck * sn * sx);
+    force_outer2(w, hu, hv);
+}
 
-    for (int k = 0; k < a.n; ++k) {
-        const void* xs = a.x[k][par];
-        const void* ys = a.y[k][par];
-        const void* xn = a.x[k][1 - par];
-        const void* yn = a.y[k][1 - par];
-        const float ck = a.c[k];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            cpx<float> p[12], q[12];
-            cpx<float> hu[2][3], hv[2][3];
-            float s1, s2;
-            // forward hop at x: X(x+mu) (x) ((1 - g_mu) Y(x))^*
-            force_load<P, NF>(xn, vh, j, f, p, s1);
-            force_load<P, NF>(ys, vh, i, f, q, s2);
-            force_half<MU, -1>(hu, p, 1.f);
-            force_half<MU, SY1>(hv, q, ck * s1 * s2);
-            force_outer2(w, hu, hv);
-            // backward hop at x+mu (through U_mu(x)^dagger): ((1 + g_mu) Y(x+mu)) (x) X(x)^*
-            force_load<P, NF>(yn, vh, j, f, p, s1);
-            force_load<P, NF>(xs, vh, i, f, q, s2);
-            force_half<MU, SY2>(hu, p, 1.f);
-            force_half<MU, +1>(hv, q, ck * s1 * s2);
-            force_outer2(w, hu, hv);
-        }
-    }
-
-    // Z = U W, force += T_A[Z] = (Z - Z^+)/2 - i Im(tr Z)/3
+// Z = U W, force += T_A[Z] = (Z - Z^+)/2 - i Im(tr Z)/3 on link (x, MU)
+template <int MU>
+__device__ __forceinline__ void force_project(const ForceArgs& a, const cpx<float> (&w)[9], float ph, long i, int par,
+                                              long lex) {
     cpx<float> u[9];
-    load_link<P32>(a.gauge[par], vh, MU, i, u);
+    load_link<P32>(a.gauge[par], a.g.vh, MU, i, u);
     cpx<float> z[9];
 #pragma unroll
     for (int r = 0; r < 3; ++r)
@@ -151,7 +157,6 @@ __device__ __forceinline__ void force_link(const ForceArgs& a, long i, int par, 
             z[3 * r + s] = ph * acc;
         }
     const float itr = (z[0].im + z[4].im + z[8].im) * (1.f / 3.f);
-    const long lex = 2 * i + (c.x & 1);
     double2* out = reinterpret_cast<double2*>(a.force) + (lex * 4 + MU) * 9;
 #pragma unroll
     for (int r = 0; r < 3; ++r)
@@ -168,35 +173,86 @@ __device__ __forceinline__ void force_link(const ForceArgs& a, long i, int par, 
         }
 }
 
-// 4 resident blocks per SM (64 registers, a few spilled): 1612 -> 1593 us (FP32
-// fields) and 1347 -> 1269 us (FP16) at 24^3x48, 12 two-flavour pairs
-template <int P, int NF, bool G5>
-__global__ void __launch_bounds__(256, 4) force_outer_kernel(const __grid_constant__ ForceArgs a) {
-    const long i = (long)blockIdx.x * 32 + threadIdx.x;
-    if (i >= a.g.vh) return;
-    const int mu = threadIdx.y;
-    const int par = threadIdx.z;
-    const Coord c = cb_coords(a.g, i, par);
-    switch (mu) {   // warp-uniform
-        case 0: force_link<P, NF, 0, G5>(a, i, par, c); break;
-        case 1: force_link<P, NF, 1, G5>(a, i, par, c); break;
-        case 2: force_link<P, NF, 2, G5>(a, i, par, c); break;
-        default: force_link<P, NF, 3, G5>(a, i, par, c); break;
+// directions MU and MU + 1 of one site
+template <int P, int NF, int MU, bool G5>
+__device__ __forceinline__ void force_links(const ForceArgs& a, long i, int par, const Coord& c) {
+    const long vh = a.g.vh;
+    bool wrap0, wrap1;
+    const long j0 = force_neighbour<MU>(a.g, c, wrap0), j1 = force_neighbour<MU + 1>(a.g, c, wrap1);
+    cpx<float> w0[9], w1[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) w0[e] = w1[e] = C(0.f, 0.f);
+    // pairs and flavours as one loop over one copy of the code: unrolled over the
+    // flavours, the variants that share an SM overflow the instruction cache
+#pragma unroll 1
+    for (int q = 0; q < a.n * NF; ++q) {
+        const int k = NF == 2 ? q >> 1 : q, f = NF == 2 ? q & 1 : 0;
+        const void* xn = a.x[k][1 - par];
+        const void* yn = a.y[k][1 - par];
+        const float ck = a.c[k];
+        cpx<float> xs[12], ys[12];
+        float sx, sy;
+        force_load<P, NF>(a.y[k][par], vh, i, f, ys, sy);
+        force_load<P, NF>(a.x[k][par], vh, i, f, xs, sx);
+        force_pair<P, NF, MU, G5>(w0, xn, yn, vh, j0, f, xs, sx, ys, sy, ck);
+        force_pair<P, NF, MU + 1, G5>(w1, xn, yn, vh, j1, f, xs, sx, ys, sy, ck);
     }
+    const long lex = 2 * i + (c.x & 1);
+    force_project<MU>(a, w0, 1.f, i, par, lex);
+    force_project<MU + 1>(a, w1, MU + 1 == 3 && wrap1 ? a.bc_t : 1.f, i, par, lex);
+}
+
+// 4 resident blocks per SM (128 registers): 1182 us at 24^3x48, 12 two-flavour FP32
+// pairs (before the site order of a.tt); 3 / 5 / 6 blocks 1311 / 1301 / 1524 us.
+template <int P, int NF, bool G5>
+__global__ void __launch_bounds__(128, 4) force_outer_kernel(const __grid_constant__ ForceArgs a) {
+    const int v = blockIdx.x * 32 + threadIdx.x;
+    if (v >= a.g.vh) return;
+    const int par = threadIdx.z;
+    Coord c;
+    long i = v;
+    if (a.tt == 0) {
+        c = cb_coords(a.g, i, par);
+    } else {
+        // v counts half-sites along x-lines in the order (t / tt, z, y / 2, t % tt, y % 2),
+        // slowest first; the last tile of t may be shorter
+        const Geom& g = a.g;
+        const int hx = g.X / 2;
+        const int line = v / hx, xi = v - line * hx;
+        const int per = a.tt * g.Z * g.Y, tile = line / per;
+        const int st = min(a.tt, g.T - tile * a.tt);
+        int r = line - tile * per;
+        const int y1 = r & 1;
+        r >>= 1;
+        c.t = tile * a.tt + r % st;
+        r /= st;
+        c.y = 2 * (r % (g.Y / 2)) + y1;
+        c.z = r / (g.Y / 2);
+        c.x = 2 * xi + ((c.y + c.z + c.t + par) & 1);
+        i = (long)((c.t * g.Z + c.z) * g.Y + c.y) * hx + xi;
+    }
+    if (threadIdx.y == 0) force_links<P, NF, 0, G5>(a, i, par, c);   // warp-uniform
+    else force_links<P, NF, 2, G5>(a, i, par, c);
 }
 
 template <int P, int NF>
 static cudaError_t launch_t(const ForceArgs& a, cudaStream_t st) {
     const long nblk = (a.g.vh + 31) / 32;
     if (a.g5y)
-        force_outer_kernel<P, NF, true><<<(unsigned)nblk, dim3(32, 4, 2), 0, st>>>(a);
+        force_outer_kernel<P, NF, true><<<(unsigned)nblk, dim3(32, 2, 2), 0, st>>>(a);
     else
-        force_outer_kernel<P, NF, false><<<(unsigned)nblk, dim3(32, 4, 2), 0, st>>>(a);
+        force_outer_kernel<P, NF, false><<<(unsigned)nblk, dim3(32, 2, 2), 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_force_outer(int prec, int nf, const ForceArgs& a, cudaStream_t st) {
-    if (a.n <= 0 || a.g.vh <= 0) return cudaSuccess;
+cudaError_t launch_force_outer(int prec, int nf, const ForceArgs& a0, cudaStream_t st) {
+    if (a0.n <= 0 || a0.g.vh <= 0) return cudaSuccess;
+    ForceArgs a = a0;
+    // bytes of all pairs on a plane of constant z, t and on a time slice; in the tiled
+    // order the +z neighbour is tt planes away (kept below 24 MB)
+    const double plane = (double)a.g.X * a.g.Y * 2 * a.n * 24 * nf * prec_esz(prec);
+    if (plane * a.g.Z <= 40e6) a.tt = 0;
+    else a.tt = plane * 8 <= 24e6 ? 8 : (plane * 4 <= 24e6 ? 4 : 2);
     switch (prec) {
         case P32: return nf == 1 ? launch_t<P32, 1>(a, st) : launch_t<P32, 2>(a, st);
         case PB16: return nf == 1 ? launch_t<PB16, 1>(a, st) : launch_t<PB16, 2>(a, st);

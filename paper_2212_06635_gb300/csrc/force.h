@@ -11,6 +11,7 @@ struct ForceArgs {
     Geom g;
     float bc_t;                  // phase of the time links crossing t = T-1 -> 0
     int n;                       // field pairs
+    int tt;                      // time slices per tile of the site order; 0: lexicographic (set at launch)
     const void* gauge[2];        // FP32 native links of parity 0 / 1
     const void* x[FORCE_MAXN][2];   // native fields X_k of parity 0 / 1
     const void* y[FORCE_MAXN][2];   // native fields Y_k of parity 0 / 1

@@ -174,6 +174,38 @@ def test_force_outer_full_size_sampled():
         lat.close()
 
 
+@pytest.mark.parametrize("dims,nf,n", [((26, 22, 24, 10), 2, 12), ((48, 40, 8, 6), 1, 32)],
+                         ids=["tiles of 8 and 2", "tiles of 2"])
+def test_force_outer_tiled_site_order(dims, nf, n):
+    """Launches whose time slices exceed the L2 share walk the sites in tiles of
+    time slices (ragged at T = 10); a quarter of the pairs at a time takes the plain
+    order.  The two differ by the FP32 sums over the pairs only: n nf terms of
+    comparable size in each, relative rounding 2^-24 sqrt(n nf) at most."""
+    import torch
+    from paper_2212_06635_gb300 import tm
+    u = F.gauge_field(dims, 1002)
+    lat = Lat(u, dims, KAPPA, CSW, mu=MU)
+    try:
+        gen = torch.Generator(device="cuda:0")
+        gen.manual_seed(7)
+        half = lat.vh * nf * 24
+        fields = [torch.randn(half, generator=gen, device="cuda:0", dtype=torch.float32).view(torch.uint8)
+                  for _ in range(4 * n)]
+        xs = [(fields[4 * k], fields[4 * k + 1]) for k in range(n)]
+        ys = [(fields[4 * k + 2], fields[4 * k + 3]) for k in range(n)]
+        c = [0.5 + 0.1 * k for k in range(n)]
+        one = torch.zeros(2 * lat.vh * 4 * 18, dtype=torch.float64, device="cuda:0")
+        parts = torch.zeros_like(one)
+        tm.tm_force_outer(lat.ctx, 1, nf, c, xs, ys, one, gamma5_y=True)
+        for k in range(0, n, n // 4):
+            e = k + n // 4
+            tm.tm_force_outer(lat.ctx, 1, nf, c[k:e], xs[k:e], ys[k:e], parts, gamma5_y=True)
+        assert float(parts.norm()) > 0.0
+        assert float((one - parts).norm() / parts.norm()) < 2.0 ** -24 * 4 * (n * nf) ** 0.5
+    finally:
+        lat.close()
+
+
 def _schur_codes(tm, heavy, sign):
     if heavy:
         return (tm.TM_QH, tm.TM_QH_DAG) if sign > 0 else (tm.TM_QH_DAG, tm.TM_QH)
