@@ -138,6 +138,7 @@ enum WsId {
     WS_TE_S, WS_MID_S, WS_R_S, WS_P_S, WS_AP_S, WS_X_S,
     WS_STAGE_B, WS_STAGE_X, WS_STAGE_G, WS_APPLY_TE, WS_APPLY_MID, WS_STAGE_IO, WS_TUNE,
     WS_FCG_Z, WS_XDF,
+    WS_RING = 60,   // RING search directions (CG) or residuals (multishift)
     WS_MS_X = 100, WS_MS_P = 200, WS_MS_X64 = 300, WS_RAT = 400
 };
 
@@ -475,6 +476,36 @@ static cudaError_t normal_op(const tm_ctx* c, tm_op op, void* out, const void* i
     cudaError_t e = schur<P, NF>(c, s1, mid, in, te, st, ctl, fin, s1 * rt);
     if (e != cudaSuccess) return e;
     return schur<P, NF>(c, s2, out, mid, te, st, ctl, FIN_NONE, s2 * rt, true);
+}
+
+// r_out = r_in - alpha (A + shift) p with ||r_out||^2 -> fin_update; <p, A p> fused
+// into the first factor (fin_alpha), which gives alpha before the last pass runs.  The
+// solvers' chain: the kernel before is the solver's own.
+template <int P, int NF>
+static cudaError_t normal_update(const tm_ctx* c, tm_op op, void* r_out, const void* r_in, const void* p, void* mid,
+                                 void* te, cudaStream_t st, SolverCtl* ctl, int fin_alpha, int fin_update) {
+    int s1, s2;
+    normal_signs(op, &s1, &s2);
+    const double rt = is_what(op) ? 2.0 * c->params.kappa * c->params.rho : 0.0;
+    cudaError_t e = schur<P, NF>(c, s1, mid, p, te, st, ctl, fin_alpha, s1 * rt, true);
+    if (e != cudaSuccess) return e;
+    OpBatch<1> b{};
+    b.n = 1;
+    b.chained = true;
+    b.fin = FIN_NONE;
+    b.p[0] = make_prob(c, P, NF, K1_EO_INV, s2, te, mid, nullptr, ctl, false);
+    b.blk_start[1] = b.p[0].nblk;
+    e = launch_pass<P, NF, K1_EO_INV, 1>(pass_kernel<P, NF>(c, K1_EO_INV), b, b.p[0].nblk, st);
+    if (e != cudaSuccess) return e;
+    const int kernel = pass_kernel<P, NF>(c, K2_OE_LOCAL) == PK_SPLIT ? PK_SPLIT : PK_DIRECT;   // (no staged form)
+    b.fin = fin_update;
+    b.p[0] = make_prob(c, P, NF, K2_OE_LOCAL, s2, r_out, te, mid, ctl, true, s2 * rt);
+    b.p[0].nblk = pass_nblk(P, c->vh, NF, K2_OE_LOCAL, kernel);
+    b.p[0].r = r_in;
+    b.p[0].p = p;
+    b.blk_start[1] = b.p[0].nblk;
+    if (kernel == PK_SPLIT) return launch_dslash_split<P, NF, K2_UPDATE>(b, b.p[0].nblk, st);
+    return launch_dslash<P, NF, K2_UPDATE, 1>(b, b.p[0].nblk, st);
 }
 
 template <int P, int NF>
@@ -905,6 +936,13 @@ static VecBatch<1> vb1(const tm_ctx* c, void* v0, void* v1 = nullptr, void* v2 =
     return b;
 }
 
+// v = {x, -, ring}
+static VecBatch<1> vb_ring(const tm_ctx* c, void* x, void* const* ring, int m) {
+    VecBatch<1> b = vb1(c, x);
+    for (int k = 0; k < m; ++k) b.p[0].v[2 + k] = ring[k];
+    return b;
+}
+
 template <int P>
 static cudaError_t norm2_t(tm_ctx* c, int nf, const void* f, double* res, cudaStream_t st) {
     VecBatch<1> b = vb1(c, const_cast<void*>(f), nullptr, nullptr, nullptr, res);
@@ -991,18 +1029,38 @@ static tm_status is_zero64(tm_ctx* c, const void* x64, cudaStream_t st, bool* ze
     return TM_OK;
 }
 
-// One CG iteration in storage precision PS (x accumulated in PX):
-//   p = r + beta p;  Ap (fused <p,Ap> -> alpha);  x += alpha p, r -= alpha Ap (fused rr -> beta, flag)
+// Ring of `bytes`-sized fields for a solver that enqueues `chunk` iterations at a time:
+// RING of them if the chunk is a multiple of it and memory allows, else 2 or 1 (the
+// iteration is then the textbook one).
+static tm_status ring_get(tm_ctx* c, size_t bytes, int chunk, void** f, int* m) {
+    int n = chunk % RING == 0 ? RING : (chunk % 2 == 0 ? 2 : 1);
+    for (int k = 0; k < n; ++k) {
+        const tm_status s = ws_get(c, WS_RING + k, bytes, &f[k]);
+        if (s == TM_ERR_OOM && k > 0) {
+            cudaGetLastError();
+            n = 1;
+            break;
+        }
+        CKS(s);
+    }
+    *m = n;
+    return TM_OK;
+}
+
+// Iteration s of a ring of m: p_s = r + beta p_{s-1};  r -= alpha (A + shift) p_s (alpha
+// from the fused <p, A p>; fused rr -> beta, flag);  after the last of the ring
+// x += sum alpha_i p_i (x accumulated in PX).
 template <int PS, int NF>
-static cudaError_t cg_iteration(tm_ctx* c, tm_op op, void* xs, void* p, void* r, void* ap, void* mid, void* te,
-                                cudaStream_t st) {
+static cudaError_t cg_iteration(tm_ctx* c, tm_op op, void* xs, void* const* ps, int m, int s, void* r, void* mid,
+                                void* te, cudaStream_t st) {
     constexpr int PX = PS == P64 ? P64 : P32;
+    constexpr int NC = 12 * NF;
     const int nb = nblk(c->vh, BLAS_BS);
-    cudaError_t e = launch_cg_pupdate<PS, 12 * NF, 1>(vb1(c, p, r), nb, st);
+    cudaError_t e = launch_cg_direction<PS, NC>(vb1(c, ps[s], r, ps[(s + m - 1) % m]), nb, st);
     if (e != cudaSuccess) return e;
-    e = normal_op<PS, NF>(c, op, ap, p, mid, te, st, c->ctl, FIN_CG_ALPHA);
-    if (e != cudaSuccess) return e;
-    return launch_cg_update<PS, PX, 12 * NF, 1>(vb1(c, xs, p, r, ap), nb, st);
+    e = normal_update<PS, NF>(c, op, r, r, ps[s], mid, te, st, c->ctl, FIN_CG_ALPHA, FIN_CG_UPDATE);
+    if (e != cudaSuccess || s + 1 < m) return e;
+    return launch_cg_xupdate<PS, PX, NC>(vb_ring(c, xs, ps, m), m, false, nb, st);
 }
 
 // Solve (A + shift) x = b in place on native FP64 x64, b64.
@@ -1022,15 +1080,11 @@ static tm_status solve_core(tm_ctx* c, tm_op op, double shift, const tm_solve_pa
     CKS(ws_get(c, WS_AX64, b64sz, &ax64));
     CKS(ws_get(c, WS_TE64, b64sz, &te64));
     CKS(ws_get(c, WS_MID64, b64sz, &mid64));
-    void *rs, *ps, *aps, *tes, *mids, *xs;
+    void *rs, *tes, *mids, *xs;
     if (PS == P64) {
         rs = r64; xs = x64; tes = te64; mids = mid64;
-        CKS(ws_get(c, WS_P_S, bssz, &ps));
-        CKS(ws_get(c, WS_AP_S, bssz, &aps));
     } else {
         CKS(ws_get(c, WS_R_S, bssz, &rs));
-        CKS(ws_get(c, WS_P_S, bssz, &ps));
-        CKS(ws_get(c, WS_AP_S, bssz, &aps));
         CKS(ws_get(c, WS_TE_S, bssz, &tes));
         CKS(ws_get(c, WS_MID_S, bssz, &mids));
         CKS(ws_get(c, WS_X_S, spinor_bytes(P32, NC, vh), &xs));
@@ -1040,6 +1094,9 @@ static tm_status solve_core(tm_ctx* c, tm_op op, double shift, const tm_solve_pa
     const double delta = PS == P64 ? 0.0 : (sp->delta > 0 ? sp->delta : default_delta(PS));
     const int chunk = sp->chunk > 0 ? sp->chunk : 16;
     const int nb = nblk(vh, BLAS_BS);
+    void* ps[RING];
+    int m = 1;
+    CKS(ring_get(c, bssz, chunk, ps, &m));
 
     double bb = 0;
     CKS((norm2_dev<P64, NC>(c, b64, st, &bb)));
@@ -1079,14 +1136,16 @@ static tm_status solve_core(tm_ctx* c, tm_op op, double shift, const tm_solve_pa
         h.beta = 0.0;
         h.shift = shift;
         h.maxiter = maxiter;
+        h.ring = m;
         h.stop_rr = std::max(target, delta * delta * rr);
         h.flag = CTL_RUN;
         CKS(put_ctl(c, st));
+        int base = 0;   // iterations done before the current run of chunks
         if (sp->use_graph) {
             cudaGraph_t graph;
             CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
             for (int it = 0; it < chunk; ++it) {
-                cudaError_t e = cg_iteration<PS, NF>(c, op, xs, ps, rs, aps, mids, tes, st);
+                cudaError_t e = cg_iteration<PS, NF>(c, op, xs, ps, m, it % m, rs, mids, tes, st);
                 if (e != cudaSuccess) {
                     cudaStreamEndCapture(st, &graph);
                     return fail(TM_ERR_CUDA, "capture: %s", cudaGetErrorString(e));
@@ -1100,10 +1159,16 @@ static tm_status solve_core(tm_ctx* c, tm_op op, double shift, const tm_solve_pa
             if (gexec) {
                 CK(cudaGraphLaunch(gexec, st));
             } else {
-                for (int it = 0; it < chunk; ++it) CK((cg_iteration<PS, NF>(c, op, xs, ps, rs, aps, mids, tes, st)));
+                for (int it = 0; it < chunk; ++it) CK((cg_iteration<PS, NF>(c, op, xs, ps, m, it % m, rs, mids, tes, st)));
             }
             CKS(get_ctl(c, st));
             if (h.flag == CTL_RUN) continue;
+            // the steps of the ring that x does not hold yet: the iteration that stopped the
+            // run ended before its ring's update, one that broke down does not count
+            const int done = h.iter - base;
+            const int left = h.flag == CTL_BREAKDOWN ? done % m : (done > 0 ? (done - 1) % m + 1 : 0);
+            if (left > 0)
+                CK((launch_cg_xupdate<PS, PS == P64 ? P64 : P32, NC>(vb_ring(c, xs, ps, m), left, true, nb, st)));
             if (h.flag == CTL_BREAKDOWN) { status = TM_ERR_BREAKDOWN; break; }
             // reliable update / convergence check
             if (PS != P64) {
@@ -1122,6 +1187,11 @@ static tm_status solve_core(tm_ctx* c, tm_op op, double shift, const tm_solve_pa
                 break;
             }
             if (PS != P64) CK((launch_convert<PS, P64, NC, 1>(vb1(c, rs, r64), nb, st)));
+            // the next chunk starts at the beginning of the ring: its first iteration takes
+            // the last direction from the end of it
+            if (left > 0 && left != m) CK(cudaMemcpyAsync(ps[m - 1], ps[left - 1], bssz, cudaMemcpyDeviceToDevice, st));
+            base = h.iter;
+            h.slot = 0;
             h.beta = rr / h.rr_old;
             h.rr = rr;
             h.stop_rr = std::max(target, delta * delta * rr);
@@ -1231,10 +1301,11 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
     constexpr int PX = PS == P64 ? P64 : P32;
     const long vh = c->vh;
     const size_t bs = spinor_bytes(PS, NC, vh), bx = spinor_bytes(PX, NC, vh);
-    void *rs, *ps, *aps, *tes, *mids;
-    CKS(ws_get(c, WS_R_S, bs, &rs));
+    const int chunk = sp->chunk > 0 ? sp->chunk : 16;
+    void *ps, *tes, *mids, *rs[RING];
+    int rm = 1;   // residuals kept between two updates of the shifts
+    CKS(ring_get(c, bs, chunk, rs, &rm));
     CKS(ws_get(c, WS_P_S, bs, &ps));
-    CKS(ws_get(c, WS_AP_S, bs, &aps));
     CKS(ws_get(c, WS_TE_S, bs, &tes));
     CKS(ws_get(c, WS_MID_S, bs, &mids));
     MsVecs mv{};
@@ -1253,7 +1324,8 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
     if (!std::isfinite(bb) || !(bb > 0))
         return fail(std::isfinite(bb) ? TM_ERR_ARG : TM_ERR_BREAKDOWN,
                     "multishift: right-hand side must be finite and non-zero");
-    CK((launch_convert<PS, P64, NC, 1>(vb1(c, rs, b64), nb, st)));
+    CK((launch_convert<PS, P64, NC, 1>(vb1(c, rs[rm - 1], b64), nb, st)));
+    for (int k = 0; k < ns; ++k) CK(cudaMemcpyAsync(mv.p[k], rs[rm - 1], bs, cudaMemcpyDeviceToDevice, st));   // p_k = r
     // The sloppy multishift stops each shift when its recursively updated residual
     // falls below floor_tol; the shift-by-shift refinement takes it to sp->tol.
     // Swept on the heavy doublet at 24^3x48 (12 shifts, time of the whole solve
@@ -1283,25 +1355,27 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
     h.rr = bb;
     h.rr_old = bb;
     h.shift = sh_sorted[0];
+    h.ring = rm;
     h.maxiter = sp->maxiter > 0 ? sp->maxiter : 100000;
     h.stop_rr = 0.0;
     h.flag = CTL_RUN;
     CKS(put_ctl(c, st));
-    auto iteration = [&](int first) -> cudaError_t {
-        cudaError_t e = launch_ms_pupdate<PS, PX, NC>(vb1(c, rs, ps), mv, first, nb, st);
+    // iteration s of a ring: p = r + beta p, r_s = r - alpha (A + s0) p; after the last
+    // of the ring all shifts take its iterations at once
+    auto iteration = [&](int s) -> cudaError_t {
+        void* rp = rs[(s + rm - 1) % rm];
+        cudaError_t e = launch_cg_direction<PS, NC>(vb1(c, ps, rp, ps), nb, st);
         if (e != cudaSuccess) return e;
-        e = normal_op<PS, NF>(c, op, aps, ps, mids, tes, st, c->ctl, FIN_MS_ALPHA);
-        if (e != cudaSuccess) return e;
-        return launch_ms_update<PS, NC>(vb1(c, rs, ps, aps), nb, st);
+        e = normal_update<PS, NF>(c, op, rs[s], rp, ps, mids, tes, st, c->ctl, FIN_MS_ALPHA, FIN_MS_UPDATE);
+        if (e != cudaSuccess || s + 1 < rm) return e;
+        return launch_ms_block<PS, PX, NC>(vb_ring(c, nullptr, rs, rm), mv, rm, false, nb, st);
     };
-    CK(iteration(1));
-    const int chunk = sp->chunk > 0 ? sp->chunk : 16;
     cudaGraphExec_t gexec = nullptr;
     if (sp->use_graph) {
         cudaGraph_t graph;
         CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         for (int it = 0; it < chunk; ++it) {
-            cudaError_t e = iteration(0);
+            cudaError_t e = iteration(it % rm);
             if (e != cudaSuccess) {
                 cudaStreamEndCapture(st, &graph);
                 return fail(TM_ERR_CUDA, "capture: %s", cudaGetErrorString(e));
@@ -1318,12 +1392,14 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
         if (gexec) {
             CK(cudaGraphLaunch(gexec, st));
         } else {
-            for (int it = 0; it < chunk; ++it) CK(iteration(0));
+            for (int it = 0; it < chunk; ++it) CK(iteration(it % rm));
         }
     }
     if (gexec) cudaGraphExecDestroy(gexec);
     if (h.flag == CTL_BREAKDOWN) status = fail(TM_ERR_BREAKDOWN, "multishift: breakdown");
-    CK((launch_ms_finish<PS, PX, NC>(vb1(c, rs, ps), mv, nb, st)));
+    // the iterations of the ring that the shifts have not taken yet (as in solve_core)
+    const int left = h.flag == CTL_BREAKDOWN ? h.iter % rm : (h.iter > 0 ? (h.iter - 1) % rm + 1 : 0);
+    if (left > 0) CK((launch_ms_block<PS, PX, NC>(vb_ring(c, nullptr, rs, rm), mv, left, true, nb, st)));
     // hand the sloppy solutions to FP64
     if (PX != P64) {
         for (int k = 0; k < ns; ++k) {

@@ -176,118 +176,155 @@ __global__ void __launch_bounds__(BLAS_BS) k_normalize64(const __grid_constant__
 }
 
 // ---------------------------------------------------------------------------
-// multishift CG vector updates (Sec. 4.2)
+// CG with the residual update in the operator's last pass (K2_UPDATE).  The solution
+// is touched once per RING iterations: x += sum alpha_i p_i from a ring of search
+// directions, so an iteration moves (p, r -> p) here, r once more in the odd pass and
+// a quarter of (RING p, x -> x).  Light FP16: 298 B a site instead of 542 with
+// x, p, r, A p passing through an update kernel every iteration; two-flavour FP32
+// with a shift 1248 instead of 1920 B.
 // ---------------------------------------------------------------------------
-// r_new = r - alpha (Ap + s0 p);  ||r_new||^2 -> FIN_MS_UPDATE
+// p_out = r + beta p_in
 template <int P, int NC>
-__global__ void __launch_bounds__(BLAS_BS) k_ms_update(const __grid_constant__ VecBatch<1> b) {
+__global__ void __launch_bounds__(BLAS_BS) k_cg_direction(const __grid_constant__ VecBatch<1> b) {
     using R = typename PT<P>::R;
+    pdl_wait();
     TM_VEC_PROLOGUE(1)
     if (pr.ctl->flag != CTL_RUN) return;
-    const R alpha = (R)pr.ctl->alpha;
-    const R s0 = (R)pr.ctl->shift;
+    const R beta = (R)pr.ctl->beta;
+    const bool want = pr.ctl->shift != 0.0;
     double s = 0.0;
     if (valid) {
-        cpx<R> r[NC], p[NC], ap[NC];
-        load_spinor<P, NC>(pr.v[0], pr.vh, i, r);
-        load_spinor<P, NC>(pr.v[1], pr.vh, i, p);
-        load_spinor<P, NC>(pr.v[2], pr.vh, i, ap);
-        R t = (R)0;
+        cpx<R> p[NC], r[NC];
+        load_spinor<P, NC>(pr.v[1], pr.vh, i, r);
+        if (beta != (R)0) {
+            load_spinor<P, NC>(pr.v[2], pr.vh, i, p);
 #pragma unroll
-        for (int q = 0; q < NC; ++q) {
-            r[q] = r[q] - alpha * (ap[q] + s0 * p[q]);
-            t += norm2(r[q]);
+            for (int q = 0; q < NC; ++q) p[q] = r[q] + beta * p[q];
+        } else {
+#pragma unroll
+            for (int q = 0; q < NC; ++q) p[q] = r[q];
         }
-        store_spinor<P, NC>(pr.v[0], pr.vh, i, r);
-        s = (double)t;
-    }
-    const double bs = block_sum<BLAS_BS>(s, sh);
-    reduce_finalize<BLAS_BS>(pr.partial, pr.counter, pr.nblk, lb, bs, FIN_MS_UPDATE, pr.ctl, pr.ms,
-                             nullptr, sh);
-}
-
-// Start of a multishift iteration: the x_k update of the previous iteration
-// (x_k += alpha_k p_k, deferred so that p_k is read once) fused with the new
-// directions p_k = zeta_k r + beta_k p_k and p = r + beta p, plus ||p||^2.
-template <int P, int PX, int NC>
-__global__ void __launch_bounds__(BLAS_BS) k_ms_pupdate(const __grid_constant__ VecBatch<1> b,
-                                                        const __grid_constant__ MsVecs mv, int first) {
-    using R = typename PT<P>::R;
-    using RX = typename PT<PX>::R;
-    TM_VEC_PROLOGUE(1)
-    if (pr.ctl->flag != CTL_RUN) return;
-    const MsCtl* ms = pr.ms;
-    const R beta = first ? (R)0 : (R)pr.ctl->beta;
-    double s = 0.0;
-    if (valid) {
-        cpx<R> r[NC];
-        load_spinor<P, NC>(pr.v[0], pr.vh, i, r);
-        {
-            cpx<R> p[NC];
-            if (!first) load_spinor<P, NC>(pr.v[1], pr.vh, i, p);
+        store_spinor<P, NC>(pr.v[0], pr.vh, i, p);
+        if (want) {
             R t = (R)0;
 #pragma unroll
-            for (int q = 0; q < NC; ++q) {
-                p[q] = first ? r[q] : r[q] + beta * p[q];
-                t += norm2(p[q]);
-            }
-            store_spinor<P, NC>(pr.v[1], pr.vh, i, p);
+            for (int q = 0; q < NC; ++q) t += norm2(p[q]);
             s = (double)t;
         }
-#pragma unroll 1
-        for (int kk = 0; kk < ms->nshift; ++kk) {
-            const int act = ms->active[kk];
-            if (act == 0) continue;
-            cpx<R> pk[NC];
-            const R zk = (R)ms->zeta[kk];
-            if (!first) {
-                load_spinor<P, NC>(mv.p[kk], pr.vh, i, pk);
-                const R ak = (R)ms->alpha_s[kk];
-                cpx<RX> xk[NC];
-                load_spinor<PX, NC>(mv.x[kk], pr.vh, i, xk);
-#pragma unroll
-                for (int q = 0; q < NC; ++q) {
-                    xk[q].re += (RX)(ak * pk[q].re);
-                    xk[q].im += (RX)(ak * pk[q].im);
-                }
-                store_spinor<PX, NC>(mv.x[kk], pr.vh, i, xk);
-            }
-            if (act == 1) {
-                const R bk = first ? (R)0 : (R)ms->beta_s[kk];
-#pragma unroll
-                for (int q = 0; q < NC; ++q) pk[q] = first ? zk * r[q] : zk * r[q] + bk * pk[q];
-                store_spinor<P, NC>(mv.p[kk], pr.vh, i, pk);
-            }
-        }
     }
-    const double bs = block_sum<BLAS_BS>(s, sh);
-    reduce_finalize<BLAS_BS>(pr.partial, pr.counter, pr.nblk, lb, bs, FIN_PP, pr.ctl, pr.ms,
-                             nullptr, sh);
+    if (want) {
+        const double bs = block_sum<BLAS_BS>(s, sh);
+        reduce_finalize<BLAS_BS>(pr.partial, pr.counter, pr.nblk, lb, bs, FIN_PP, pr.ctl, pr.ms,
+                                 nullptr, sh);
+    }
 }
 
-// End of a multishift solve: apply the pending x_k += alpha_k p_k.
+// x += sum_{i < n} alpha_i p_i, a vector of reals at a time (one thread per site and vector)
 template <int P, int PX, int NC>
-__global__ void __launch_bounds__(BLAS_BS) k_ms_finish(const __grid_constant__ VecBatch<1> b,
-                                                       const __grid_constant__ MsVecs mv) {
+__global__ void __launch_bounds__(BLAS_BS) k_cg_xupdate(const __grid_constant__ VecBatch<1> b, int n, bool always) {
     using R = typename PT<P>::R;
     using RX = typename PT<PX>::R;
-    TM_VEC_PROLOGUE(1)
-    if (!valid) return;
-    const MsCtl* ms = pr.ms;
-#pragma unroll 1
-    for (int kk = 0; kk < ms->nshift; ++kk) {
-        if (ms->active[kk] == 0) continue;
-        const R ak = (R)ms->alpha_s[kk];
-        cpx<R> pk[NC];
-        cpx<RX> xk[NC];
-        load_spinor<P, NC>(mv.p[kk], pr.vh, i, pk);
-        load_spinor<PX, NC>(mv.x[kk], pr.vh, i, xk);
+    constexpr int W = PT<P>::W;
+    pdl_wait();
+    const VecProb& pr = b.p[0];
+    if (!always && pr.ctl->flag != CTL_RUN) return;
+    const long vh = pr.vh, i = (long)blockIdx.x * BLAS_BS + threadIdx.x;
+    if (i >= vh) return;
+    R alpha[RING];
 #pragma unroll
-        for (int q = 0; q < NC; ++q) {
-            xk[q].re += (RX)(ak * pk[q].re);
-            xk[q].im += (RX)(ak * pk[q].im);
+    for (int k = 0; k < RING; ++k) {
+        alpha[k] = k < n ? (R)pr.ctl->alpha_ring[k] : (R)0;
+        if constexpr (P == PB16 || P == PF16)
+            if (k < n) alpha[k] *= reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.v[2 + k]) + (size_t)vh * NC * 4)[i];
+    }
+    const int v = blockIdx.y;
+    RX x[W];
+    load_reals<PX, W>(pr.v[0], vh, i, W * v, x);
+#pragma unroll
+    for (int k = 0; k < RING; ++k) {
+        if (k < n) {
+            R p[W];
+            load_reals<P, W>(pr.v[2 + k], vh, i, W * v, p);
+#pragma unroll
+            for (int e = 0; e < W; ++e) x[e] += (RX)(alpha[k] * p[e]);
         }
-        store_spinor<PX, NC>(mv.x[kk], pr.vh, i, xk);
+    }
+    store_reals<PX, W>(pr.v[0], vh, i, W * v, x);
+}
+
+// Multishift CG (Sec. 4.2): n iterations of every shift at once.  p_k and x_k pass
+// through memory once per RING iterations instead of every one (12 shifts,
+// two-flavour FP32: 9.2 KB -> 2.5 KB a site and iteration).  One thread per site and
+// vector of reals, with the residuals in registers; 16-bit fields need the maximum
+// over a site for p_k's scale, so there one thread per site reads the residuals (from
+// L2) for each shift.
+template <int P, int PX, int NC>
+__global__ void __launch_bounds__(BLAS_BS) k_ms_block(const __grid_constant__ VecBatch<1> b,
+                                                      const __grid_constant__ MsVecs mv, int n, bool always) {
+    using R = typename PT<P>::R;
+    using RX = typename PT<PX>::R;
+    constexpr bool H = P == PB16 || P == PF16;
+    constexpr int W = H ? 2 * NC : PT<P>::W;   // reals a thread holds
+    pdl_wait();
+    const VecProb& pr = b.p[0];
+    if (!always && pr.ctl->flag != CTL_RUN) return;
+    // the coefficients once per block in the vectors' precision: converted from FP64 by
+    // every thread they took longer than the vectors' traffic (12 shifts at 24^3x48, mean
+    // over a solve: 676 -> 286 us a launch)
+    const MsCtl* ms = pr.ms;
+    const int ns = ms->nshift;
+    __shared__ R coef[MAX_SHIFTS][RING][3];
+    __shared__ int live[MAX_SHIFTS], nlive;
+    for (int e = threadIdx.x; e < ns * RING; e += BLAS_BS) {
+        const int k = e / RING, q = e % RING;
+        coef[k][q][0] = q < n ? (R)ms->alpha_ring[q][k] : (R)0;
+        coef[k][q][1] = q < n ? (R)ms->zeta_ring[q][k] : (R)0;
+        coef[k][q][2] = q < n ? (R)ms->beta_ring[q][k] : (R)0;
+    }
+    if (threadIdx.x == 0) {
+        int m = 0;
+        for (int k = 0; k < ns; ++k) {
+            bool any = false;   // else frozen before this block of iterations
+            for (int q = 0; q < n; ++q) any = any || ms->alpha_ring[q][k] != 0.0;
+            if (any) live[m++] = k;
+        }
+        nlive = m;
+    }
+    __syncthreads();
+    const long vh = pr.vh, i = (long)blockIdx.x * BLAS_BS + threadIdx.x;
+    if (i >= vh) return;
+    const int off = H ? 0 : W * blockIdx.y;
+    R r[H ? 1 : RING][W];
+    if constexpr (!H) {
+#pragma unroll
+        for (int q = 0; q < RING; ++q)
+            if (q < n) load_reals<P, W>(pr.v[2 + q], vh, i, off, r[q]);
+    }
+    const int nl = nlive;
+#pragma unroll (H ? 1 : 2)
+    for (int l = 0; l < nl; ++l) {
+        const int k = live[l];
+        R p[W];
+        RX x[W];
+        if constexpr (H) load_spinor<P, NC>(mv.p[k], vh, i, reinterpret_cast<cpx<R>*>(p));
+        else load_reals<P, W>(mv.p[k], vh, i, off, p);
+        load_reals<PX, W>(mv.x[k], vh, i, off, x);
+#pragma unroll
+        for (int q = 0; q < RING; ++q) {
+            if (q < n) {
+                const R a = coef[k][q][0], z = coef[k][q][1], bt = coef[k][q][2];
+                if constexpr (H) load_spinor<P, NC>(pr.v[2 + q], vh, i, reinterpret_cast<cpx<R>*>(r[0]));
+                const R* rq = r[H ? 0 : q];
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    x[e] += (RX)(a * p[e]);
+                    p[e] = z * rq[e] + bt * p[e];
+                }
+            }
+        }
+        store_reals<PX, W>(mv.x[k], vh, i, off, x);
+        if constexpr (H) store_spinor<P, NC>(mv.p[k], vh, i, reinterpret_cast<const cpx<R>*>(p));
+        else store_reals<P, W>(mv.p[k], vh, i, off, p);
     }
 }
 
@@ -360,18 +397,18 @@ cudaError_t launch_normalize64(const VecBatch<1>& b, int nb, cudaStream_t st) {
     return cudaGetLastError();
 }
 template <int P, int NC>
-cudaError_t launch_ms_update(const VecBatch<1>& b, int nb, cudaStream_t st) {
-    k_ms_update<P, NC><<<nb, BLAS_BS, 0, st>>>(b);
+cudaError_t launch_cg_direction(const VecBatch<1>& b, int nb, cudaStream_t st) {
+    return launch_chained(k_cg_direction<P, NC>, nb, BLAS_BS, 0, st, true, b);
+}
+template <int P, int PX, int NC>
+cudaError_t launch_cg_xupdate(const VecBatch<1>& b, int n, bool always, int nb, cudaStream_t st) {
+    k_cg_xupdate<P, PX, NC><<<dim3(nb, 2 * NC / PT<P>::W), BLAS_BS, 0, st>>>(b, n, always);
     return cudaGetLastError();
 }
 template <int P, int PX, int NC>
-cudaError_t launch_ms_pupdate(const VecBatch<1>& b, const MsVecs& mv, int first, int nb, cudaStream_t st) {
-    k_ms_pupdate<P, PX, NC><<<nb, BLAS_BS, 0, st>>>(b, mv, first);
-    return cudaGetLastError();
-}
-template <int P, int PX, int NC>
-cudaError_t launch_ms_finish(const VecBatch<1>& b, const MsVecs& mv, int nb, cudaStream_t st) {
-    k_ms_finish<P, PX, NC><<<nb, BLAS_BS, 0, st>>>(b, mv);
+cudaError_t launch_ms_block(const VecBatch<1>& b, const MsVecs& mv, int n, bool always, int nb, cudaStream_t st) {
+    const int ny = P == PB16 || P == PF16 ? 1 : 2 * NC / PT<P>::W;
+    k_ms_block<P, PX, NC><<<dim3(nb, ny), BLAS_BS, 0, st>>>(b, mv, n, always);
     return cudaGetLastError();
 }
 template <int P, int NC>
@@ -387,19 +424,18 @@ cudaError_t launch_export(double* dst, const void* src, long vh, cudaStream_t st
 
 // explicit instantiations
 #define TM_PX(P) ((P) == P64 ? P64 : P32)
-#define TM_BLAS_P_NC_NP(P, NC, NP)                                                           \
-    template cudaError_t launch_cg_pupdate<P, NC, NP>(const VecBatch<NP>&, int, cudaStream_t); \
-    template cudaError_t launch_cg_update<P, TM_PX(P), NC, NP>(const VecBatch<NP>&, int, cudaStream_t); \
-    template cudaError_t launch_add_to64<P, NC, NP>(const VecBatch<NP>&, int, cudaStream_t);   \
-    template cudaError_t launch_norm2<P, NC, NP>(const VecBatch<NP>&, int, cudaStream_t);
-#define TM_BLAS_P_NC(P, NC)                                                                  \
-    TM_BLAS_P_NC_NP(P, NC, 1)                                                                \
-    template cudaError_t launch_ms_update<P, NC>(const VecBatch<1>&, int, cudaStream_t);      \
-    template cudaError_t launch_ms_pupdate<P, TM_PX(P), NC>(const VecBatch<1>&, const MsVecs&, int, int, cudaStream_t); \
-    template cudaError_t launch_ms_finish<P, TM_PX(P), NC>(const VecBatch<1>&, const MsVecs&, int, cudaStream_t); \
-    template cudaError_t launch_import<P, NC>(void*, const double*, long, cudaStream_t);      \
+#define TM_BLAS_P_NC(P, NC)                                                                              \
+    template cudaError_t launch_cg_direction<P, NC>(const VecBatch<1>&, int, cudaStream_t);               \
+    template cudaError_t launch_cg_xupdate<P, TM_PX(P), NC>(const VecBatch<1>&, int, bool, int, cudaStream_t); \
+    template cudaError_t launch_ms_block<P, TM_PX(P), NC>(const VecBatch<1>&, const MsVecs&, int, bool, int, cudaStream_t); \
+    template cudaError_t launch_add_to64<P, NC, 1>(const VecBatch<1>&, int, cudaStream_t);               \
+    template cudaError_t launch_norm2<P, NC, 1>(const VecBatch<1>&, int, cudaStream_t);                  \
+    template cudaError_t launch_import<P, NC>(void*, const double*, long, cudaStream_t);                  \
     template cudaError_t launch_export<P, NC>(double*, const void*, long, cudaStream_t);
-#define TM_BLAS_P(P) TM_BLAS_P_NC(P, 12) TM_BLAS_P_NC(P, 24) TM_BLAS_P_NC_NP(P, 12, MAXP)
+#define TM_BLAS_P(P)                                                                                     \
+    TM_BLAS_P_NC(P, 12) TM_BLAS_P_NC(P, 24)                                                              \
+    template cudaError_t launch_cg_pupdate<P, 12, MAXP>(const VecBatch<MAXP>&, int, cudaStream_t);        \
+    template cudaError_t launch_cg_update<P, TM_PX(P), 12, MAXP>(const VecBatch<MAXP>&, int, cudaStream_t);
 
 TM_BLAS_P(P64)
 TM_BLAS_P(P32)

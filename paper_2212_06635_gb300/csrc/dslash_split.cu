@@ -235,6 +235,21 @@ __global__ void __launch_bounds__(128 * NF) dslash_split_kernel(const __grid_con
                 for (int j = 0; j < 6; ++j) cfma(s, m[c][j], v[j]);
                 out[c] = g5 * s;
             }
+            if constexpr (KIND == K2_UPDATE) {   // residual_update of dslash.cu
+                const R alpha = (R)pr.ctl->alpha, shift = (R)pr.ctl->shift;
+                R rs = (R)1, ps = (R)1;
+                if constexpr (P == PF16 || P == PB16) {
+                    const size_t off = (size_t)vh * NF * 12 * 4;
+                    rs = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.r) + off)[i];
+                    ps = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.p) + off) + i);
+                }
+                const int e = 12 * f + 6 * cb + 3 * h;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    if (shift != (R)0) out[c] = out[c] + shift * (ps * load_complex<P>(pr.p, vh, i, e + c));
+                    out[c] = rs * load_complex<P>(pr.r, vh, i, e + c) - alpha * out[c];
+                }
+            }
         }
     }
     const int e0 = 12 * f + 6 * cb + 3 * h;
@@ -259,8 +274,8 @@ __global__ void __launch_bounds__(128 * NF) dslash_split_kernel(const __grid_con
 #pragma unroll
         for (int c = 0; c < 3; ++c) store_complex<P>(pr.out, vh, i, e0 + c, out[c]);
     }
-    if constexpr (KIND == K2_OE_LOCAL) {
-        if (pr.partial != nullptr) {
+    if constexpr (KIND != K1_EO_INV) {
+        if (KIND == K2_UPDATE || pr.partial != nullptr) {
             R s = (R)0;
             if (valid) {
 #pragma unroll
@@ -285,7 +300,8 @@ cudaError_t launch_dslash_split(const OpBatch<1>& b, int nblocks, cudaStream_t s
 
 #define TM_SPLIT_INST(P, NF)                                                                          \
     template cudaError_t launch_dslash_split<P, NF, K1_EO_INV>(const OpBatch<1>&, int, cudaStream_t); \
-    template cudaError_t launch_dslash_split<P, NF, K2_OE_LOCAL>(const OpBatch<1>&, int, cudaStream_t);
+    template cudaError_t launch_dslash_split<P, NF, K2_OE_LOCAL>(const OpBatch<1>&, int, cudaStream_t); \
+    template cudaError_t launch_dslash_split<P, NF, K2_UPDATE>(const OpBatch<1>&, int, cudaStream_t);
 #define TM_SPLIT_P(P) TM_SPLIT_INST(P, 1) TM_SPLIT_INST(P, 2)
 TM_SPLIT_P(P64)
 TM_SPLIT_P(P32)

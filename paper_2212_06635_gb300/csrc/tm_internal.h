@@ -302,7 +302,8 @@ struct SolverCtl {
     int iter;
     int maxiter;
     int flag;
-    int pad;
+    int slot, ring;   // iteration within the current ring of directions, and the ring's length
+    double alpha_ring[4];
 };
 
 // Multishift state (one per multishift solve), up to MAX_SHIFTS shifts.
@@ -316,6 +317,9 @@ struct MsCtl {
     int active[MAX_SHIFTS];
     int nshift;
     int n_active;
+    // of the iterations of the current ring: the steps, and zeta and beta of the
+    // direction that follows
+    double alpha_ring[4][MAX_SHIFTS], zeta_ring[4][MAX_SHIFTS], beta_ring[4][MAX_SHIFTS];
 };
 
 // ---------------------------------------------------------------------------
@@ -345,6 +349,8 @@ struct OpProb {
     const void* clov;        // clover array of the output parity
     const void* in;          // hopping input (other parity)
     const void* loc;         // K2: odd-site input for the local term
+    const void* r;           // K2_UPDATE: residual and search direction
+    const void* p;
     void* out;
     double kappa;
     double tw;               // light: sign*mu_t; heavy: sign*mubar_t (K2 local term)

@@ -16,7 +16,10 @@ constexpr int BLAS_BS = 256;
 constexpr int SPLIT_SITES = 32;  // sites per block of the small-lattice stencil kernel
 constexpr int MIN_BS = 32;       // fewest sites per block of any reducing kernel (sizes the partials)
 
-enum DslashKind { K1_EO_INV = 0, K2_OE_LOCAL = 1 };
+// K2_UPDATE: the odd pass of the second factor of a normal operator with the residual
+// update in its epilogue, r_out = r - alpha (out + shift p), ||r_out||^2
+enum DslashKind { K1_EO_INV = 0, K2_OE_LOCAL = 1, K2_UPDATE = 2 };
+constexpr int RING = 4;   // search directions kept between two updates of the solutions
 
 // FinOp codes beyond those in tm_internal.h
 enum { FIN_PP = 4, FIN_CG_UPDATE = 5, FIN_MS_UPDATE = 6 };
@@ -88,6 +91,7 @@ __device__ inline void finalize_scalar(int fin, double t, SolverCtl* ctl, MsCtl*
                 ctl->flag = CTL_BREAKDOWN;
             } else {
                 ctl->alpha = ctl->rr / pAp;
+                ctl->alpha_ring[ctl->slot] = ctl->alpha;
                 if (fin == FIN_MS_ALPHA) ms_alpha(ms, ctl->alpha);
             }
             break;
@@ -97,6 +101,8 @@ __device__ inline void finalize_scalar(int fin, double t, SolverCtl* ctl, MsCtl*
             ctl->rr_old = ctl->rr;
             ctl->rr = t;
             ctl->beta = t / ctl->rr_old;
+            const int slot = ctl->slot;
+            ctl->slot = slot + 1 < ctl->ring ? slot + 1 : 0;
             ctl->iter += 1;
             if (!isfinite(t)) ctl->flag = CTL_BREAKDOWN;
             else if (t < ctl->stop_rr) ctl->flag = CTL_STOP;
@@ -104,9 +110,12 @@ __device__ inline void finalize_scalar(int fin, double t, SolverCtl* ctl, MsCtl*
             if (fin == FIN_MS_UPDATE) {
                 int na = 0;
                 for (int k = 0; k < ms->nshift; ++k) {
+                    ms->alpha_ring[slot][k] = ms->active[k] ? ms->alpha_s[k] : 0.0;
                     if (!ms->active[k]) continue;
                     const double ratio = ms->beta_s[k];
                     ms->beta_s[k] = ctl->beta * ratio * ratio;
+                    ms->beta_ring[slot][k] = ms->beta_s[k];
+                    ms->zeta_ring[slot][k] = ms->zeta[k];
                     // shifted residual r_k = zeta_k r
                     if (ms->zeta[k] * ms->zeta[k] * t < ms->stop_rr) ms->active[k] = 2;  // converged, last update pending
                     else ++na;
@@ -170,7 +179,7 @@ __device__ __forceinline__ void reduce_finalize(double* partial, unsigned int* c
 struct VecProb {
     long vh;
     int nblk;
-    void* v[6];
+    void* v[2 + RING];
     SolverCtl* ctl;
     MsCtl* ms;
     double* partial;
@@ -213,12 +222,19 @@ cudaError_t launch_dslash_staged(const OpBatch<NP>& b, int nblocks, cudaStream_t
 template <int P, int NF, int KIND>
 cudaError_t launch_dslash_split(const OpBatch<1>& b, int nblocks, cudaStream_t st);
 
-// p = r + beta p (+ ||p||^2 when the problem has a shift)       v = {p, r}
+// batched solves: p = r + beta p (+ ||p||^2 when the problem has a shift)       v = {p, r}
 template <int P, int NC, int NP>
 cudaError_t launch_cg_pupdate(const VecBatch<NP>& b, int nblocks, cudaStream_t st);
-// x += alpha p; r -= alpha (Ap + shift p); ||r||^2 -> FIN_CG_UPDATE   v = {x, p, r, Ap}
+// batched solves: x += alpha p; r -= alpha (Ap + shift p); ||r||^2 -> FIN_CG_UPDATE   v = {x, p, r, Ap}
 template <int P, int PX, int NC, int NP>
 cudaError_t launch_cg_update(const VecBatch<NP>& b, int nblocks, cudaStream_t st);
+// p_out = r + beta p_in (+ ||p_out||^2 when the problem has a shift)           v = {p_out, r, p_in}
+template <int P, int NC>
+cudaError_t launch_cg_direction(const VecBatch<1>& b, int nblocks, cudaStream_t st);
+// x += sum_{i < n} alpha_i p_i, alpha_i = ctl->alpha_ring[i] (n <= RING)         v = {x, -, p_0, ...};
+// only while the problem runs, unless `always`
+template <int P, int PX, int NC>
+cudaError_t launch_cg_xupdate(const VecBatch<1>& b, int n, bool always, int nblocks, cudaStream_t st);
 // dst (precision PD) = src (precision PS)                        v = {dst, src}
 template <int PD, int PS, int NC, int NP>
 cudaError_t launch_convert(const VecBatch<NP>& b, int nblocks, cudaStream_t st);
@@ -235,16 +251,11 @@ cudaError_t launch_norm2(const VecBatch<NP>& b, int nblocks, cudaStream_t st);
 template <int NC>
 cudaError_t launch_normalize64(const VecBatch<1>& b, int nblocks, cudaStream_t st);
 
-// multishift: r_new = r - alpha (Ap + s0 p), ||r||^2 -> FIN_MS_UPDATE    v = {r, p, Ap}
-template <int P, int NC>
-cudaError_t launch_ms_update(const VecBatch<1>& b, int nblocks, cudaStream_t st);
-// multishift: x_k += alpha_k p_k (pending); p_k = zeta_k r + beta_k p_k; p = r + beta p
+// multishift: for each shift n iterations at once (MsCtl's rings),
+//   x_k += alpha_k p_k; p_k = zeta_k r_i + beta_k p_k,  i < n <= RING             v = {-, -, r_1, ...}
+// (r_i the residual after the i-th of them); only while the problem runs, unless `always`
 template <int P, int PX, int NC>
-cudaError_t launch_ms_pupdate(const VecBatch<1>& b, const MsVecs& mv, int first, int nblocks,
-                              cudaStream_t st);
-// multishift tail: x_k += alpha_k p_k for shifts with a pending update
-template <int P, int PX, int NC>
-cudaError_t launch_ms_finish(const VecBatch<1>& b, const MsVecs& mv, int nblocks, cudaStream_t st);
+cudaError_t launch_ms_block(const VecBatch<1>& b, const MsVecs& mv, int n, bool always, int nblocks, cudaStream_t st);
 
 // layout
 template <int P, int NC>

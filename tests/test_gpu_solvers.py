@@ -346,3 +346,51 @@ def test_pinned_host_fields_are_stream_ordered_and_overlap():
             assert np.array_equal(got, ref[k])
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1, 3], ids=["f64", "f32", "f16"])
+@pytest.mark.parametrize("nf", [1, 2])
+def test_rings_of_directions_match_single_steps(prec, nf):
+    """The solution is updated once per ring of search directions (4 where the chunk
+    is a multiple of 4, else 2 or 1).  A ring ends anywhere: after every iteration
+    count the iterate is that of single steps (chunk 1), in FP64 up to the order of a
+    ring's sums; full solves reach the tolerance for every chunk, with and without
+    the graph, with the directions restarted by reliable updates in between."""
+    import torch
+    from paper_2212_06635_gb300 import tm
+    dims = (6, 4, 6, 10)
+    _, lat = _lat(dims, 77, **(dict(mu=0.01) if nf == 1 else dict(mu=0.0, mubar=0.1246, epsbar=0.1350)))
+    op = tm.TM_MDAGM if nf == 1 else tm.TM_QH_SQ
+    try:
+        b = to_dev(F.odd_spinor(dims, 78, nf))
+
+        def solve(chunk, graph, maxiter, tol, sloppy):
+            x = torch.zeros_like(b)
+            sp = tm.solve_params(tol=tol, maxiter=maxiter, sloppy=sloppy, chunk=chunk, use_graph=graph)
+            info = tm.tm_solve_cg(lat.ctx, op, sp, x, b, check=False)
+            torch.cuda.synchronize()
+            return x, info
+
+        if prec == 0:
+            for its in (1, 2, 3, 4, 5, 7, 8):
+                ref, _ = solve(1, 1, its, 1e-30, 0)
+                for chunk in (2, 3, 4, 16):
+                    x, info = solve(chunk, 1, its, 1e-30, 0)
+                    assert info.iters == its
+                    assert float((x - ref).norm() / ref.norm()) < 1e-13, (its, chunk)
+        for chunk, graph in ((1, 1), (2, 0), (3, 1), (4, 0), (16, 1)):
+            x, info = solve(chunk, graph, 2000, 1e-10, prec)
+            assert info.status == 0 and info.true_rel_res <= 1e-10, (chunk, graph)
+        # multishift: every shift's directions and solutions in blocks of a ring
+        shifts = [0.01, 0.05, 0.4, 2.0]
+        for chunk, graph in ((1, 1), (2, 0), (3, 1), (16, 1)):
+            xs = [torch.zeros_like(b) for _ in shifts]
+            sp = tm.solve_params(tol=1e-10, sloppy=prec, chunk=chunk, use_graph=graph)
+            for info in tm.tm_solve_multishift(lat.ctx, op, shifts, xs, b, sp):
+                assert info.status == 0 and info.true_rel_res <= 1e-10, (chunk, graph)
+            if chunk == 1:
+                refs = xs
+            for x, r in zip(xs, refs):
+                assert float((x - r).norm() / r.norm()) < 1e-7
+    finally:
+        lat.close()
