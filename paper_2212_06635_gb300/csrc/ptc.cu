@@ -74,10 +74,12 @@ __device__ __forceinline__ void act_load(const uint4* a, long V, int b, long y, 
 // buffer's "empty" mbarrier, so transport and MMAs overlap.  After a tile's last
 // stage the MMA warp commits to "acc_full"; all 16 warps read the accumulators
 // back with tcgen05.ld (TMEM lane = site, so each thread owns one site and
-// writes its output vectors directly) and arrive on "acc_empty" before the next
-// tile's first MMA overwrites them.  The 9 paths' embedded weights (B) stay
-// resident in shared memory.  15 + 1 warps keep 128 registers per thread (4
-// warps per SM sub-partition), which a 17th warp would cut to 96.
+// writes its output vectors directly) and arrive on "acc_empty".  Two tiles have
+// accumulators in tensor memory, and a tile is read back after the next one's last
+// stage: read back at once, all warps waited for the tile's last MMAs and the
+// transport stood still (network at 24^3x48 1608 -> 1442 us).  The 9 paths' embedded
+// weights (B) stay resident in shared memory.  15 + 1 warps keep 128 registers per
+// thread (4 warps per SM sub-partition), which a 17th warp would cut to 96.
 //
 // Shared-memory operand images are the canonical K-major layout without
 // swizzle: core matrices of 8 rows x 16 bytes (8 BF16 along K) stored as 128
@@ -109,7 +111,8 @@ struct TcShape {
     static constexpr int A_STAGE = NPS * 3 * A_COL;
     static constexpr int W_PATH = NN * 16 * KCH;             // bytes of one path's B image
     static constexpr int W_ALL = NPATH * W_PATH;
-    static constexpr int TMEM_COLS = 3 * NN <= 32 ? 32 : (3 * NN <= 64 ? 64 : (3 * NN <= 128 ? 128 : 256));
+    static constexpr int ACC_COLS = 3 * NN <= 32 ? 32 : (3 * NN <= 64 ? 64 : (3 * NN <= 128 ? 128 : 256));
+    static constexpr int TMEM_COLS = 2 * ACC_COLS;           // accumulators of two tiles
     static constexpr int RAW = CPG * 3 * TC_PT * 16;         // cp.async slots: [channel][vector][thread]
     static constexpr int SMEM = W_ALL + TC_STAGES * A_STAGE + RAW + 128;   // + mbarriers, TMEM address, abort flag
     // kind::f16 instruction descriptor: D F32 (bits 4-5 = 1), A and B BF16 (bits 7-9, 10-12 = 1),
@@ -314,12 +317,16 @@ __device__ __forceinline__ void tc_locate_l(const PtcGeom& g, const TcSite& s, i
         f.flags = 3;
         return;
     }
+    // (selections, not s.c[mu]: a run-time index puts the coordinates in local memory, and
+    // each stage of every thread then waits for it: network at 24^3x48 1710 -> 1608 us)
     const int mu = (p - 1) & 3;
     const int L = mu == 0 ? g.X : (mu == 1 ? g.Y : (mu == 2 ? g.Z : g.T));
     const int st = mu == 0 ? 1 : (mu == 1 ? g.X : (mu == 2 ? g.X * g.Y : g.X * g.Y * g.Z));
-    const int cm = s.c[mu];
-    if (p <= 4) f.y = (cm + 1 == L) ? s.x - (L - 1) * st : s.x + st;
-    else f.y = (cm == 0) ? s.x + (L - 1) * st : s.x - st;
+    const int cm = mu == 0 ? s.c[0] : (mu == 1 ? s.c[1] : (mu == 2 ? s.c[2] : s.c[3]));
+    const bool fwd = p <= 4;
+    const bool wrap = cm == (fwd ? L - 1 : 0);
+    const int step = wrap ? st - L * st : st;   // forward; backward takes its negative
+    f.y = s.x + (fwd ? step : -step);
     const uint32_t* base = g.lp + (long)(p - 1) * 9 * g.V + s.x;
 #pragma unroll
     for (int k = 0; k < 9; ++k) f.lw[k] = __ldg(base + (long)k * g.V);
@@ -356,8 +363,11 @@ __device__ __forceinline__ void tc_link(const TcUnit& f, cpx<float> (&u)[9]) {
 // word 3 s + c) -> one 16-byte chunk per colour of the A images at img (4 spins
 // as BF16 (re, im) pairs): t = M v, M the path's link with its dagger and phase
 // already applied.  Two spins share each paired FMA:
-//   Re t = sum_d Re M Re v + Im M (-Im v),  Im t = sum_d Re M Im v + Im M Re v,
-// each lane in the same order as the scalar form.
+//   Re t = sum_d Re M Re v + (-Im M) Im v,  Im t = sum_d Re M Im v + Im M Re v,
+// each lane in the same order as the scalar form.  The links' imaginary parts are
+// negated, once for a thread's channels, not each channel's activations (network at
+// 24^3x48 1442 -> 1409 us; what is left is issue slots of this arithmetic and of the
+// unpacking, not memory: the layer moves 8 activation channels in and out).
 template <int A_COL>
 __device__ __forceinline__ void tc_transport_channel(const uint4 (&a)[3], const float2 (&mr)[9],
                                                      const float2 (&mi)[9], uint8_t* img) {
@@ -366,14 +376,12 @@ __device__ __forceinline__ void tc_transport_channel(const uint4 (&a)[3], const 
     uint32_t wd[3][4];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {   // spins 2h, 2h + 1
-        float2 vr[3], vi[3], nvi[3];
+        float2 vr[3], vi[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const uint32_t w0 = w[3 * (2 * h) + d], w1 = w[3 * (2 * h + 1) + d];
             vr[d] = make_float2(__uint_as_float(w0 << 16), __uint_as_float(w1 << 16));
             vi[d] = make_float2(__uint_as_float(w0 & 0xffff0000u), __uint_as_float(w1 & 0xffff0000u));
-            nvi[d] = make_float2(__uint_as_float((w0 ^ 0x80000000u) & 0xffff0000u),
-                                 __uint_as_float((w1 ^ 0x80000000u) & 0xffff0000u));
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -381,7 +389,7 @@ __device__ __forceinline__ void tc_transport_channel(const uint4 (&a)[3], const 
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 tr = __ffma2_rn(mr[3 * c + d], vr[d], tr);
-                tr = __ffma2_rn(mi[3 * c + d], nvi[d], tr);
+                tr = __ffma2_rn(make_float2(-mi[3 * c + d].x, -mi[3 * c + d].y), vi[d], tr);
                 ti = __ffma2_rn(mr[3 * c + d], vi[d], ti);
                 ti = __ffma2_rn(mi[3 * c + d], vr[d], ti);
             }
@@ -409,10 +417,11 @@ __device__ __forceinline__ void tc_copy_channel(const uint4 (&a)[3], uint8_t* im
 // sites of the tile) for its output channels, release the accumulators and
 // store the BF16 output vectors.  False if the wait ran out (warp-uniform).
 template <typename S, int COUT>   // COUT = output channels written
-__device__ __forceinline__ bool tc_epilogue(uint32_t tmem, uint64_t* acc_full, uint64_t* acc_empty, uint32_t j,
+__device__ __forceinline__ bool tc_epilogue(uint32_t tmem0, uint64_t* acc_full, uint64_t* acc_empty, uint32_t j,
                                             volatile int* abort_flag, int quarter, int wg, int lane, long tile,
                                             const PtcGeom& g, uint4* __restrict__ out) {
-    const bool w = mbar_wait(acc_full, j & 1, abort_flag);
+    const uint32_t tmem = tmem0 + (j & 1) * S::ACC_COLS;
+    const bool w = mbar_wait(acc_full + (j & 1), (j >> 1) & 1, abort_flag);
     if (!__all_sync(0xffffffffu, w)) return false;
     tc_fence_after();
     const int row = 32 * quarter + lane;
@@ -439,7 +448,7 @@ __device__ __forceinline__ bool tc_epilogue(uint32_t tmem, uint64_t* acc_full, u
         }
     }
     tc_fence_before();
-    mbar_arrive(acc_empty);
+    mbar_arrive(acc_empty + (j & 1));
     if (row < TC_SITES && xo < g.V) {
 #pragma unroll
         for (int k = 0; k < CPO; ++k) {
@@ -467,9 +476,9 @@ __global__ void __launch_bounds__(TC_BS, 1) ptc_layer_tc(PtcGeom g, const uint4*
     uint64_t* bar = reinterpret_cast<uint64_t*>(Raw + S::RAW);
     uint64_t* full = bar;                                  // [TC_STAGES] transport -> MMA
     uint64_t* empty = bar + TC_STAGES;                     // [TC_STAGES] MMA -> transport
-    uint64_t* acc_full = bar + 2 * TC_STAGES;              // accumulators ready
-    uint64_t* acc_empty = acc_full + 1;                    // accumulators read back
-    uint64_t* drain = acc_full + 2;
+    uint64_t* acc_full = bar + 2 * TC_STAGES;              // [2] a tile's accumulators ready
+    uint64_t* acc_empty = acc_full + 2;                    // [2] read back
+    uint64_t* drain = acc_full + 4;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -488,8 +497,10 @@ __global__ void __launch_bounds__(TC_BS, 1) ptc_layer_tc(PtcGeom g, const uint4*
             mbar_init(full + k, TC_PT);
             mbar_init(empty + k, 1);
         }
-        mbar_init(acc_full, 1);
-        mbar_init(acc_empty, TC_BS);
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(acc_full + k, 1);
+            mbar_init(acc_empty + k, TC_BS);
+        }
         mbar_init(drain, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -516,7 +527,8 @@ __global__ void __launch_bounds__(TC_BS, 1) ptc_layer_tc(PtcGeom g, const uint4*
         uint32_t u = 0, j = 0;
         for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++j) {
             if (lane == 0) {
-                if (j > 0 && !mbar_wait(acc_empty, (j - 1) & 1, abort_flag)) ok = false;
+                // (the accumulators that tile j - 2 used)
+                if (j > 1 && !mbar_wait(acc_empty + (j & 1), ((j >> 1) - 1) & 1, abort_flag)) ok = false;
                 for (int stg = 0; stg < S::NSTG && ok; ++stg, ++u) {
                     const int buf = u % TC_STAGES;
                     if (!mbar_wait(full + buf, (u / TC_STAGES) & 1, abort_flag)) { ok = false; break; }
@@ -531,21 +543,25 @@ __global__ void __launch_bounds__(TC_BS, 1) ptc_layer_tc(PtcGeom g, const uint4*
                             for (int kk = 0; kk < S::KCH / 2; ++kk) {
                                 const uint32_t as = a_base + buf * S::A_STAGE + (q * 3 + c) * S::A_COL + kk * 256;
                                 const uint32_t ws = w_base + pp * S::W_PATH + kk * 256;
-                                tc_mma(tmem + c * S::NN, smem_desc(as, 128, SBO), smem_desc(ws, 128, SBO), S::IDESC,
-                                       (pp > 0 || kk > 0) ? 1u : 0u);
+                                tc_mma(tmem + (j & 1) * S::ACC_COLS + c * S::NN, smem_desc(as, 128, SBO),
+                                       smem_desc(ws, 128, SBO), S::IDESC, (pp > 0 || kk > 0) ? 1u : 0u);
                             }
                     }
                     tc_commit(empty + buf);
                 }
-                if (ok) tc_commit(acc_full);
+                if (ok) tc_commit(acc_full + (j & 1));
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
-            if (!tc_epilogue<S, S::NOUT>(tmem, acc_full, acc_empty, j, abort_flag, quarter, wg, lane, tile, g, out)) {
+            if (j > 0 && !tc_epilogue<S, S::NOUT>(tmem, acc_full, acc_empty, j - 1, abort_flag, quarter, wg, lane,
+                                                  tile - gridDim.x, g, out)) {
                 ok = false;
                 break;
             }
         }
+        if (ok && j > 0)
+            ok = tc_epilogue<S, S::NOUT>(tmem, acc_full, acc_empty, j - 1, abort_flag, quarter, wg, lane,
+                                         blockIdx.x + (long)(j - 1) * gridDim.x, g, out);
     } else {
         // ---- transport warps
         const int r = tid % TC_SITES, grp = tid / TC_SITES;   // site r of the tile, site group
@@ -613,11 +629,15 @@ __global__ void __launch_bounds__(TC_BS, 1) ptc_layer_tc(PtcGeom g, const uint4*
                 mbar_arrive(full + buf);
             }
             if (!ok) break;
-            if (!tc_epilogue<S, S::NOUT>(tmem, acc_full, acc_empty, j, abort_flag, quarter, wg, lane, tile, g, out)) {
+            if (j > 0 && !tc_epilogue<S, S::NOUT>(tmem, acc_full, acc_empty, j - 1, abort_flag, quarter, wg, lane,
+                                                  tile - gridDim.x, g, out)) {
                 ok = false;
                 break;
             }
         }
+        if (ok && j > 0)
+            ok = tc_epilogue<S, S::NOUT>(tmem, acc_full, acc_empty, j - 1, abort_flag, quarter, wg, lane,
+                                         blockIdx.x + (long)(j - 1) * gridDim.x, g, out);
     }
 
     // drain: every copy and MMA issued by this block completes (each wait bounded,

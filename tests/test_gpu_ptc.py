@@ -257,3 +257,29 @@ def test_gradients_alternating_between_two_live_contexts():
         tm.tm_ptc_destroy(net)
         la.close()
         lb.close()
+
+
+def test_many_tiles_per_block_repeat_a_periodic_field():
+    """A lattice that repeats an 8^3x16 one twice in every direction (7 tiles per
+    persistent block, so both sets of accumulators are reused several times) gives
+    every copy the values of the small lattice, where each block has one tile."""
+    dims, rep = (8, 8, 8, 16), (2, 2, 2, 2, 1, 1, 1)
+    big = (16, 16, 16, 32)
+    u = F.gauge_field(dims, 31)
+    chans = [1, 8, 8, 8, 1]
+    ws = P.random_weights(chans, 32, scale=1.0)
+    geo, geo2 = D.Geometry(dims), D.Geometry(big)
+    r = F.odd_spinor(dims, 33)
+    shape = (dims[3], dims[2], dims[1], dims[0], 4, 3)
+    r2 = np.tile(geo.embed_odd(r).reshape(shape), rep[:6]).reshape(-1, 4, 3)[geo2.odd]
+    out = []
+    for d, uu, rr in ((dims, u, r), (big, np.ascontiguousarray(np.tile(u, rep)), np.ascontiguousarray(r2))):
+        lat = Lat(uu, d, KAPPA, CSW, mu=MU, bc_t=1)
+        net = _net(lat.tm, chans, ws)
+        try:
+            out.append(_apply(lat.tm, lat, net, rr))
+        finally:
+            lat.tm.tm_ptc_destroy(net)
+            lat.close()
+    ref = np.tile(geo.embed_odd(out[0]).reshape(shape), rep[:6]).reshape(-1, 4, 3)[geo2.odd]
+    assert np.array_equal(out[1], ref)
