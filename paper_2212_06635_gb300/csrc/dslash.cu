@@ -52,7 +52,7 @@ __device__ __forceinline__ void residual_update(cpx<typename PT<P>::R>* out, con
 // measured faster.  Adding / writing, us: light FP16 even 106.6 / 110.6, odd 102.3 /
 // 100.8; FP32 even 198.7 / 180.4 (with the register cap below), odd 152.3 / 149.4;
 // BF16 at 18x22x26x44 30.7 / 31.3 and 28.7 / 29.5; two-flavour odd pass at 24^3x48
-// FP16 61.6 / 61.3, FP32 75.0 / 75.9.
+// FP16 61.6 / 61.3 (59.5 with the factor folded, hop_dir), FP32 75.0 / 75.9.
 template <int P, int NF, int KIND>
 constexpr bool hop_first() {
     if (P == P64) return true;
@@ -99,11 +99,12 @@ __device__ __forceinline__ void hop_mu(cpx<typename PT<P>::R> (&acc)[NF][4][3], 
         load_link<P>(pr.gauge[po], g.vh, MU, i, u);
 #pragma unroll
         for (int f = 0; f < NF; ++f)
-            hop_dir<R, MU, -1, false, SC, FIRST>(acc[f], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
+            hop_dir<R, MU, -1, false, SC, FIRST, NF == 2>(acc[f], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
         load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nb, psi, sc);
         load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
 #pragma unroll
-        for (int f = 0; f < NF; ++f) hop_dir<R, MU, +1, true, SC>(acc[f], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
+        for (int f = 0; f < NF; ++f)
+            hop_dir<R, MU, +1, true, SC, false, NF == 2>(acc[f], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
     }
 }
 

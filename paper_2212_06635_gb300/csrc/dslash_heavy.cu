@@ -106,17 +106,19 @@ __device__ __forceinline__ void hop_mu_flavour(cpx<typename PT<P>::R> (&acc)[4][
     } else {
         load_flavour_unscaled<P>(pr.in, g.vh, nf, f, psi, sc);
         load_link<P>(pr.gauge[po], g.vh, MU, i, u);
-        hop_dir<R, MU, -1, false, SC, FIRST>(acc, psi, u, SC ? ph_f * (R)sc : ph_f);
+        hop_dir<R, MU, -1, false, SC, FIRST, true>(acc, psi, u, SC ? ph_f * (R)sc : ph_f);
         load_flavour_unscaled<P>(pr.in, g.vh, nb, f, psi, sc);
         load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
-        hop_dir<R, MU, +1, true, SC>(acc, psi, u, SC ? ph_b * (R)sc : ph_b);
+        hop_dir<R, MU, +1, true, SC, false, true>(acc, psi, u, SC ? ph_b * (R)sc : ph_b);
     }
 }
 
 // Resident blocks per SM the register allocation must allow (128 threads = 64
 // sites).  At 24^3x48: 16-bit 4 / 5 / 6 blocks take 73.9 / 73.5 / 73.9 us (FP16)
-// and 72.1 / 69.8 / 72.7 us (BF16); FP32 3 / 4 / 5 blocks 96.4 / 96.4 / 89.7 us.  FP64 (64-thread blocks): 8 as
-// in dslash.cu; 4 / 8 blocks 317.4 / 317.6 us at 16^3x32.
+// and 72.1 / 69.8 / 72.7 us (BF16), with the spinor's factor multiplying the half
+// spinors (folded into the FMAs as now, BF16 at 5 blocks: 66.7 us); FP32 3 / 4 / 5
+// blocks 96.4 / 96.4 / 89.7 us.  FP64 (64-thread blocks): 8 as in dslash.cu; 4 / 8
+// blocks 317.4 / 317.6 us at 16^3x32.
 template <int P, int KIND>
 constexpr int heavy_min_blocks() {
     return (P == PF16 || P == PB16) ? 5 : (P == P32 ? 5 : 8);
