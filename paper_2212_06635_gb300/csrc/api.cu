@@ -139,7 +139,8 @@ enum WsId {
     WS_STAGE_B, WS_STAGE_X, WS_STAGE_G, WS_APPLY_TE, WS_APPLY_MID, WS_STAGE_IO, WS_TUNE,
     WS_FCG_Z, WS_XDF,
     WS_RING = 60,   // RING search directions (CG) or residuals (multishift)
-    WS_MS_X = 100, WS_MS_P = 200, WS_MS_X64 = 300, WS_RAT = 400
+    WS_MS_X = 100, WS_MS_P = 200, WS_MS_X64 = 300, WS_RAT = 400,
+    WS_GROUP = 500, WS_GROUP_PARTIAL = 499
 };
 
 // ---------------------------------------------------------------------------
@@ -162,12 +163,12 @@ extern "C" tm_status tm_create(tm_ctx** out, const int dims[4], int device) {
     cudaError_t e = cudaSuccess;
     e = e ? e : cudaStreamCreateWithFlags(&c->sstream, cudaStreamNonBlocking);
     e = e ? e : cudaMalloc(&c->partial, sizeof(double) * c->max_blocks);
-    e = e ? e : cudaMalloc(&c->counter, sizeof(unsigned int) * 4);
-    e = e ? e : cudaMemset(c->counter, 0, sizeof(unsigned int) * 4);
-    e = e ? e : cudaMalloc(&c->ctl, sizeof(SolverCtl));
-    e = e ? e : cudaMemset(c->ctl, 0, sizeof(SolverCtl));
+    e = e ? e : cudaMalloc(&c->counter, sizeof(unsigned int) * GROUP);
+    e = e ? e : cudaMemset(c->counter, 0, sizeof(unsigned int) * GROUP);
+    e = e ? e : cudaMalloc(&c->ctl, sizeof(SolverCtl) * GROUP);
+    e = e ? e : cudaMemset(c->ctl, 0, sizeof(SolverCtl) * GROUP);
     e = e ? e : cudaMalloc(&c->ms, sizeof(MsCtl));
-    e = e ? e : cudaMallocHost(&c->h_ctl, sizeof(SolverCtl));
+    e = e ? e : cudaMallocHost(&c->h_ctl, sizeof(SolverCtl) * GROUP);
     e = e ? e : cudaMallocHost(&c->h_ms, sizeof(MsCtl));
     e = e ? e : cudaMalloc(&c->d_scal, sizeof(double) * 16);
     e = e ? e : cudaMallocHost(&c->h_scal, sizeof(double) * 16);
@@ -402,7 +403,7 @@ static int pass_nblk(int P, long vh, int nf, int kind, int kernel) {
 // launch one pass in the variant the context chose for (P, NF, KIND)
 template <int P, int NF, int KIND, int NP>
 static cudaError_t launch_pass(int kernel, const OpBatch<NP>& b, int nb, cudaStream_t st) {
-    if constexpr (P != P64 && P != PDF) {
+    if constexpr (P != P64 && P != PDF && NP != GROUP) {
         if (kernel == PK_STAGED) return launch_dslash_staged<P, NF, KIND, NP>(b, nb, st);
     }
     if constexpr (NP == 1 && P != PDF) {
@@ -478,34 +479,65 @@ static cudaError_t normal_op(const tm_ctx* c, tm_op op, void* out, const void* i
     return schur<P, NF>(c, s2, out, mid, te, st, ctl, FIN_NONE, s2 * rt, true);
 }
 
+// Reduction scratch of problem q of a group.
+static double* slot_partial(const tm_ctx* c, int q) {
+    if (q == 0) return c->partial;
+    return reinterpret_cast<double*>(c->ws.at(WS_GROUP_PARTIAL).first) + (size_t)(q - 1) * c->max_blocks;
+}
+
 // r_out = r_in - alpha (A + shift) p with ||r_out||^2 -> fin_update; <p, A p> fused
 // into the first factor (fin_alpha), which gives alpha before the last pass runs.  The
-// solvers' chain: the kernel before is the solver's own.
-template <int P, int NF>
-static cudaError_t normal_update(const tm_ctx* c, tm_op op, void* r_out, const void* r_in, const void* p, void* mid,
-                                 void* te, cudaStream_t st, SolverCtl* ctl, int fin_alpha, int fin_update) {
+// solvers' chain: the kernel before is the solver's own.  n problems, each with its own
+// control word; a group (NP == GROUP) takes the direct passes: together its lattices
+// fill the chip, and its blocks share what the staged variant would stage.
+struct UpdVecs {
+    void *r_out, *r_in, *p, *mid, *te;
+};
+template <int P, int NF, int NP>
+static cudaError_t normal_update(const tm_ctx* c, tm_op op, const UpdVecs* w, int n, cudaStream_t st, int fin_alpha,
+                                 int fin_update) {
     int s1, s2;
     normal_signs(op, &s1, &s2);
     const double rt = is_what(op) ? 2.0 * c->params.kappa * c->params.rho : 0.0;
-    cudaError_t e = schur<P, NF>(c, s1, mid, p, te, st, ctl, fin_alpha, s1 * rt, true);
-    if (e != cudaSuccess) return e;
-    OpBatch<1> b{};
-    b.n = 1;
+    const int v1 = NP == 1 ? pass_kernel<P, NF>(c, K1_EO_INV) : PK_DIRECT;
+    const int v2 = NP == 1 ? pass_kernel<P, NF>(c, K2_OE_LOCAL) : PK_DIRECT;
+    const int vu = v2 == PK_SPLIT ? PK_SPLIT : PK_DIRECT;   // (the update has no staged form)
+    OpBatch<NP> b{};
+    b.n = n;
     b.chained = true;
-    b.fin = FIN_NONE;
-    b.p[0] = make_prob(c, P, NF, K1_EO_INV, s2, te, mid, nullptr, ctl, false);
-    b.blk_start[1] = b.p[0].nblk;
-    e = launch_pass<P, NF, K1_EO_INV, 1>(pass_kernel<P, NF>(c, K1_EO_INV), b, b.p[0].nblk, st);
+    auto table = [&](int kind, int kernel, int sign, int fin, double rho, void* UpdVecs::*out, void* UpdVecs::*in,
+                     void* UpdVecs::*loc) {
+        const int nb = pass_nblk(P, c->vh, NF, kind, kernel);
+        b.fin = fin;
+        for (int q = 0; q < n; ++q) {
+            OpProb& p = b.p[q];
+            p = make_prob(c, P, NF, kind, sign, w[q].*out, w[q].*in, loc ? w[q].*loc : nullptr, c->ctl + q,
+                          fin != FIN_NONE, rho);
+            p.nblk = nb;
+            if (fin != FIN_NONE) p.partial = slot_partial(c, q);
+            p.counter = c->counter + q;
+            b.blk_start[q + 1] = nb * (q + 1);
+        }
+        return nb * n;
+    };
+    int nb = table(K1_EO_INV, v1, s1, FIN_NONE, 0.0, &UpdVecs::te, &UpdVecs::p, nullptr);
+    cudaError_t e = launch_pass<P, NF, K1_EO_INV, NP>(v1, b, nb, st);
     if (e != cudaSuccess) return e;
-    const int kernel = pass_kernel<P, NF>(c, K2_OE_LOCAL) == PK_SPLIT ? PK_SPLIT : PK_DIRECT;   // (no staged form)
-    b.fin = fin_update;
-    b.p[0] = make_prob(c, P, NF, K2_OE_LOCAL, s2, r_out, te, mid, ctl, true, s2 * rt);
-    b.p[0].nblk = pass_nblk(P, c->vh, NF, K2_OE_LOCAL, kernel);
-    b.p[0].r = r_in;
-    b.p[0].p = p;
-    b.blk_start[1] = b.p[0].nblk;
-    if (kernel == PK_SPLIT) return launch_dslash_split<P, NF, K2_UPDATE>(b, b.p[0].nblk, st);
-    return launch_dslash<P, NF, K2_UPDATE, 1>(b, b.p[0].nblk, st);
+    nb = table(K2_OE_LOCAL, v2, s1, fin_alpha, s1 * rt, &UpdVecs::mid, &UpdVecs::te, &UpdVecs::p);
+    e = launch_pass<P, NF, K2_OE_LOCAL, NP>(v2, b, nb, st);
+    if (e != cudaSuccess) return e;
+    nb = table(K1_EO_INV, v1, s2, FIN_NONE, 0.0, &UpdVecs::te, &UpdVecs::mid, nullptr);
+    e = launch_pass<P, NF, K1_EO_INV, NP>(v1, b, nb, st);
+    if (e != cudaSuccess) return e;
+    nb = table(K2_OE_LOCAL, vu, s2, fin_update, s2 * rt, &UpdVecs::r_out, &UpdVecs::te, &UpdVecs::mid);
+    for (int q = 0; q < n; ++q) {
+        b.p[q].r = w[q].r_in;
+        b.p[q].p = w[q].p;
+    }
+    if constexpr (NP == 1) {
+        if (vu == PK_SPLIT) return launch_dslash_split<P, NF, K2_UPDATE>(b, nb, st);
+    }
+    return launch_dslash<P, NF, K2_UPDATE, NP>(b, nb, st);
 }
 
 template <int P, int NF>
@@ -930,28 +962,33 @@ extern "C" tm_status tm_autotune(tm_ctx* c, tm_prec prec, int nf, tm_tuning* cho
 // ---------------------------------------------------------------------------
 // solver building blocks (single problem)
 // ---------------------------------------------------------------------------
+static VecProb vec_prob(const tm_ctx* c, int q) {   // problem q of a group, without its vectors
+    VecProb p{};
+    p.vh = c->vh;
+    p.nblk = nblk(c->vh, BLAS_BS);
+    p.ctl = c->ctl + q;
+    p.ms = c->ms;
+    p.partial = slot_partial(c, q);
+    p.counter = c->counter + q;
+    return p;
+}
+
 static VecBatch<1> vb1(const tm_ctx* c, void* v0, void* v1 = nullptr, void* v2 = nullptr, void* v3 = nullptr,
                        double* dst = nullptr) {
     VecBatch<1> b{};
     b.n = 1;
-    const int nb = nblk(c->vh, BLAS_BS);
-    b.blk_start[0] = 0;
-    b.blk_start[1] = nb;
     VecProb& p = b.p[0];
-    p.vh = c->vh;
-    p.nblk = nb;
+    p = vec_prob(c, 0);
+    b.blk_start[1] = p.nblk;
     p.v[0] = v0; p.v[1] = v1; p.v[2] = v2; p.v[3] = v3;
-    p.ctl = c->ctl;
-    p.ms = c->ms;
-    p.partial = c->partial;
-    p.counter = c->counter;
     p.dst = dst;
     return b;
 }
 
-// v = {x, -, ring}
-static VecBatch<1> vb_ring(const tm_ctx* c, void* x, void* const* ring, int m) {
+// v = {x, -, ring}, of problem q of a group
+static VecBatch<1> vb_ring(const tm_ctx* c, void* x, void* const* ring, int m, int q = 0) {
     VecBatch<1> b = vb1(c, x);
+    b.p[0].ctl = c->ctl + q;
     for (int k = 0; k < m; ++k) b.p[0].v[2 + k] = ring[k];
     return b;
 }
@@ -988,12 +1025,12 @@ static tm_status read_scalar(tm_ctx* c, double* dev, double* out, cudaStream_t s
     return TM_OK;
 }
 
-static tm_status put_ctl(tm_ctx* c, cudaStream_t st) {
-    CK(cudaMemcpyAsync(c->ctl, c->h_ctl, sizeof(SolverCtl), cudaMemcpyHostToDevice, st));
+static tm_status put_ctl(tm_ctx* c, cudaStream_t st, int q = 0) {
+    CK(cudaMemcpyAsync(c->ctl + q, c->h_ctl + q, sizeof(SolverCtl), cudaMemcpyHostToDevice, st));
     return TM_OK;
 }
-static tm_status get_ctl(tm_ctx* c, cudaStream_t st) {
-    CK(cudaMemcpyAsync(c->h_ctl, c->ctl, sizeof(SolverCtl), cudaMemcpyDeviceToHost, st));
+static tm_status get_ctl(tm_ctx* c, cudaStream_t st, int n = 1) {
+    CK(cudaMemcpyAsync(c->h_ctl, c->ctl, n * sizeof(SolverCtl), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     return TM_OK;
 }
@@ -1002,11 +1039,12 @@ static tm_status get_ctl(tm_ctx* c, cudaStream_t st) {
 // so A x = 0 without applying the operator (a zero initial guess).  dw: A x in
 // double-word arithmetic (x and the result rounded to a 48-bit significand on the
 // way in and out; mid64, te64 and ax64 serve as double-word scratch), for the
-// reliable updates inside a mixed-precision solve; otherwise native FP64.
+// reliable updates inside a mixed-precision solve; otherwise native FP64.  q: the
+// problem of a group whose control word holds the shift.
 template <int NF>
 static tm_status true_residual(tm_ctx* c, tm_op op, double shift, void* x64, void* b64, void* r64, void* ax64,
                                void* mid64, void* te64, cudaStream_t st, double* rr, bool x_zero = false,
-                               bool dw = false) {
+                               bool dw = false, int q = 0) {
     const long n16 = 12 * NF * c->vh;   // 16-byte elements of a field
     if (x_zero) {
         CK(cudaMemsetAsync(ax64, 0, spinor_bytes(P64, 12 * NF, c->vh), st));
@@ -1020,9 +1058,11 @@ static tm_status true_residual(tm_ctx* c, tm_op op, double shift, void* x64, voi
     } else {
         CK((normal_op<P64, NF>(c, op, ax64, x64, mid64, te64, st, nullptr, FIN_NONE)));
     }
-    c->h_ctl->shift = shift;
-    CK(cudaMemcpyAsync(&c->ctl->shift, &c->h_ctl->shift, sizeof(double), cudaMemcpyHostToDevice, st));
-    CK((launch_residual64<12 * NF, 1>(vb1(c, r64, b64, ax64, x64, c->d_scal), nblk(c->vh, BLAS_BS), st)));
+    c->h_ctl[q].shift = shift;
+    CK(cudaMemcpyAsync(&c->ctl[q].shift, &c->h_ctl[q].shift, sizeof(double), cudaMemcpyHostToDevice, st));
+    VecBatch<1> v = vb1(c, r64, b64, ax64, x64, c->d_scal);
+    v.p[0].ctl = c->ctl + q;
+    CK((launch_residual64<12 * NF, 1>(v, nblk(c->vh, BLAS_BS), st)));
     return read_scalar(c, c->d_scal, rr, st);
 }
 
@@ -1060,179 +1100,308 @@ static tm_status ring_get(tm_ctx* c, size_t bytes, int chunk, void** f, int* m) 
     return TM_OK;
 }
 
-// Iteration s of a ring of m: p_s = r + beta p_{s-1};  r -= alpha (A + shift) p_s (alpha
-// from the fused <p, A p>; fused rr -> beta, flag);  after the last of the ring
-// x += sum alpha_i p_i (x accumulated in PX).
-template <int PS, int NF>
-static cudaError_t cg_iteration(tm_ctx* c, tm_op op, void* xs, void* const* ps, int m, int s, void* r, void* mid,
-                                void* te, cudaStream_t st) {
+// One system (A + shift) x = b of a solve: the solution in native FP64, its working
+// fields in the storage precision (x in FP32; in FP64 the solution itself), and where
+// the iteration stands.
+struct SolveSys {
+    double shift = 0.0;
+    void* x64 = nullptr;
+    tm_solve_info* info = nullptr;
+    void *r = nullptr, *te = nullptr, *mid = nullptr, *x = nullptr, *p[RING] = {};
+    double rr = 0.0;
+    int base = 0;          // iterations done before the current run of chunks
+    bool done = false;
+};
+
+// Iteration s of a ring of m of n systems: p_s = r + beta p_{s-1};  r -= alpha
+// (A + shift) p_s (alpha from the fused <p, A p>; fused rr -> beta, flag);  after the last
+// of the ring x += sum alpha_i p_i (x accumulated in PX).
+template <int PS, int NF, int NP>
+static cudaError_t cg_iteration(tm_ctx* c, tm_op op, const SolveSys* sys, int n, int m, int s, cudaStream_t st) {
     constexpr int PX = PS == P64 ? P64 : P32;
     constexpr int NC = 12 * NF;
     const int nb = nblk(c->vh, BLAS_BS);
-    cudaError_t e = launch_cg_direction<PS, NC>(vb1(c, ps[s], r, ps[(s + m - 1) % m]), nb, st);
+    VecBatch<NP> dir{}, upd{};
+    UpdVecs w[NP];
+    dir.n = upd.n = n;
+    for (int q = 0; q < n; ++q) {
+        const SolveSys& y = sys[q];
+        dir.p[q] = upd.p[q] = vec_prob(c, q);
+        dir.blk_start[q + 1] = upd.blk_start[q + 1] = nb * (q + 1);
+        dir.p[q].v[0] = y.p[s];
+        dir.p[q].v[1] = y.r;
+        dir.p[q].v[2] = y.p[(s + m - 1) % m];
+        upd.p[q].v[0] = y.x;
+        for (int k = 0; k < m; ++k) upd.p[q].v[2 + k] = y.p[k];
+        w[q] = {y.r, y.r, y.p[s], y.mid, y.te};
+    }
+    cudaError_t e = launch_cg_direction<PS, NC, NP>(dir, nb * n, st);
     if (e != cudaSuccess) return e;
-    e = normal_update<PS, NF>(c, op, r, r, ps[s], mid, te, st, c->ctl, FIN_CG_ALPHA, FIN_CG_UPDATE);
+    e = normal_update<PS, NF, NP>(c, op, w, n, st, FIN_CG_ALPHA, FIN_CG_UPDATE);
     if (e != cudaSuccess || s + 1 < m) return e;
-    return launch_cg_xupdate<PS, PX, NC>(vb_ring(c, xs, ps, m), m, false, nb, st);
+    return launch_cg_xupdate<PS, PX, NC, NP>(upd, m, false, nb, st);
 }
 
-// Solve (A + shift) x = b in place on native FP64 x64, b64.
-// PS == P64: plain FP64 CG.  Otherwise mixed precision with reliable updates:
-// the iteration runs in PS storage / FP32 arithmetic with x accumulated in FP32;
-// whenever ||r|| has dropped by delta since the last true residual, x is folded
-// into the FP64 solution and r = b - A x is recomputed in double-word arithmetic
-// (true_residual); a residual below the tolerance is confirmed in FP64.
+// Working fields of the systems, and the ring's length.  The first system takes the
+// single solve's buffers; the others those of a finished multishift solve of ns shifts
+// (its solutions and directions).  Only lattices of up to GROW_SITES sites per parity
+// allocate more (8 fields a system, 6 MB each at most in FP32 with two flavours); a
+// larger one takes no memory that a later allocation could miss.  Where the buffers end
+// there are fewer systems.
+constexpr long GROW_SITES = 32768;
 template <int PS, int NF>
-static tm_status solve_core(tm_ctx* c, tm_op op, double shift, const tm_solve_params* sp, void* x64, void* b64,
-                            tm_solve_info* info, cudaStream_t st) {
+static tm_status solve_fields(tm_ctx* c, const tm_solve_params* sp, std::vector<SolveSys>& sys, int ns, int* m) {
+    const size_t bytes = spinor_bytes(PS, 12 * NF, c->vh);
+    const int chunk = sp->chunk > 0 ? sp->chunk : 16;
+    SolveSys& y = sys[0];
+    if (PS == P64) {
+        CKS(ws_get(c, WS_R64, bytes, &y.r));
+        CKS(ws_get(c, WS_TE64, bytes, &y.te));
+        CKS(ws_get(c, WS_MID64, bytes, &y.mid));
+        y.x = y.x64;
+    } else {
+        CKS(ws_get(c, WS_R_S, bytes, &y.r));
+        CKS(ws_get(c, WS_TE_S, bytes, &y.te));
+        CKS(ws_get(c, WS_MID_S, bytes, &y.mid));
+        CKS(ws_get(c, WS_X_S, spinor_bytes(P32, 12 * NF, c->vh), &y.x));
+    }
+    CKS(ring_get(c, bytes, chunk, y.p, m));
+    const int n = (int)sys.size();
+    if (n > 1) {
+        void* partial = nullptr;
+        const tm_status s = ws_get(c, WS_GROUP_PARTIAL, sizeof(double) * c->max_blocks * (n - 1), &partial);
+        if (s == TM_ERR_OOM) {
+            cudaGetLastError();
+            sys.resize(1);
+            return TM_OK;
+        }
+        CKS(s);
+    }
+    int next = 0;
+    auto field = [&](size_t size, void** out) {
+        for (; next < 2 * ns; ++next) {
+            auto it = c->ws.find(next < ns ? WS_MS_X + next : WS_MS_P + next - ns);
+            if (it == c->ws.end() || it->second.second < size) continue;
+            ++next;
+            *out = it->second.first;
+            return TM_OK;
+        }
+        if (c->vh > GROW_SITES) return TM_ERR_OOM;
+        return ws_get(c, WS_GROUP + next++ - 2 * ns, size, out);
+    };
+    auto fields = [&](SolveSys& z) {
+        CKS(field(spinor_bytes(P32, 12 * NF, c->vh), &z.x));
+        CKS(field(bytes, &z.r));
+        CKS(field(bytes, &z.te));
+        CKS(field(bytes, &z.mid));
+        for (int k = 0; k < *m; ++k) CKS(field(bytes, &z.p[k]));
+        return TM_OK;
+    };
+    for (int q = 1; q < n; ++q) {
+        const tm_status s = fields(sys[q]);
+        if (s == TM_ERR_OOM) {
+            cudaGetLastError();
+            sys.resize(q);
+            break;
+        }
+        CKS(s);
+    }
+    return TM_OK;
+}
+
+// Solve (A + shift) x = b in place on native FP64 x64, b64, for n systems at once.
+// PS == P64 (one system): plain FP64 CG.  Otherwise mixed precision with reliable
+// updates: the iteration runs in PS storage / FP32 arithmetic with x accumulated in
+// FP32; whenever ||r|| has dropped by delta since the last true residual, x is folded
+// into the FP64 solution and r = b - A x is recomputed in double-word arithmetic
+// (true_residual); a residual below the tolerance is confirmed in FP64.  Systems that
+// have stopped skip their blocks until the others have.
+template <int PS, int NF, int NP>
+static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std::vector<SolveSys>& sys, int m,
+                            void* b64, cudaStream_t st) {
+    static_assert(NP == 1 || PS != P64, "FP64 systems are solved one by one");
     constexpr int NC = 12 * NF;
     const long vh = c->vh;
+    const int n = (int)sys.size();
     const size_t b64sz = spinor_bytes(P64, NC, vh), bssz = spinor_bytes(PS, NC, vh);
     void *r64, *ax64, *te64, *mid64;
     CKS(ws_get(c, WS_R64, b64sz, &r64));
     CKS(ws_get(c, WS_AX64, b64sz, &ax64));
     CKS(ws_get(c, WS_TE64, b64sz, &te64));
     CKS(ws_get(c, WS_MID64, b64sz, &mid64));
-    void *rs, *tes, *mids, *xs;
-    if (PS == P64) {
-        rs = r64; xs = x64; tes = te64; mids = mid64;
-    } else {
-        CKS(ws_get(c, WS_R_S, bssz, &rs));
-        CKS(ws_get(c, WS_TE_S, bssz, &tes));
-        CKS(ws_get(c, WS_MID_S, bssz, &mids));
-        CKS(ws_get(c, WS_X_S, spinor_bytes(P32, NC, vh), &xs));
-    }
     const double tol = sp->tol > 0 ? sp->tol : 1e-10;
     const int maxiter = sp->maxiter > 0 ? sp->maxiter : 100000;
     const double delta = PS == P64 ? 0.0 : (sp->delta > 0 ? sp->delta : default_delta(PS));
     const int chunk = sp->chunk > 0 ? sp->chunk : 16;
     const int nb = nblk(vh, BLAS_BS);
-    void* ps[RING];
-    int m = 1;
-    CKS(ring_get(c, bssz, chunk, ps, &m));
+    const bool dw = PS != P64 && !sp->fp64_updates;   // double-word reliable updates
 
     double bb = 0;
     CKS((norm2_dev<P64, NC>(c, b64, st, &bb)));
-    info->iters = 0;
-    info->reliable_updates = 0;
+    for (SolveSys& y : sys) {
+        y.info->iters = 0;
+        y.info->reliable_updates = 0;
+    }
     if (!std::isfinite(bb)) {
-        info->true_rel_res = bb;
-        info->status = TM_ERR_BREAKDOWN;
+        for (SolveSys& y : sys) {
+            y.info->true_rel_res = bb;
+            y.info->status = TM_ERR_BREAKDOWN;
+        }
         return fail(TM_ERR_BREAKDOWN, "solve: right-hand side is not finite");
     }
     if (!(bb > 0)) {
-        CK(cudaMemsetAsync(x64, 0, b64sz, st));
-        info->true_rel_res = 0.0;
-        info->status = TM_OK;
+        for (SolveSys& y : sys) {
+            CK(cudaMemsetAsync(y.x64, 0, b64sz, st));
+            y.info->true_rel_res = 0.0;
+            y.info->status = TM_OK;
+        }
         return TM_OK;
     }
-    double rr = 0;
-    bool x0 = false;
-    CKS(is_zero64<NF>(c, x64, st, &x0));
-    const bool dw = PS != P64 && !sp->fp64_updates;   // double-word reliable updates
-    CKS(true_residual<NF>(c, op, shift, x64, b64, r64, ax64, mid64, te64, st, &rr, x0, dw));
     const double target = tol * tol * bb;
-    // an initial guess already within the tolerance is confirmed in FP64
-    if (dw && !x0 && rr <= target)
-        CKS(true_residual<NF>(c, op, shift, x64, b64, r64, ax64, mid64, te64, st, &rr));
-    tm_status status = TM_OK;
-    cudaGraphExec_t gexec = nullptr;
-    if (rr > target) {
-        if (PS != P64) {
-            CK((launch_convert<PS, P64, NC, 1>(vb1(c, rs, r64), nb, st)));
-            CK(cudaMemsetAsync(xs, 0, spinor_bytes(P32, NC, vh), st));
-        }
-        SolverCtl& h = *c->h_ctl;
+    tm_status worst = TM_OK;
+    int running = n;
+    auto finish = [&](SolveSys& y, int iters, tm_status status) {
+        y.done = true;
+        --running;
+        y.info->iters = iters;
+        y.info->true_rel_res = std::sqrt(y.rr / bb);
+        y.info->status = status;
+        if (status == TM_OK) return;
+        fail(status, "solve: %s after %d iterations, true rel res %.3e",
+             status == TM_ERR_BREAKDOWN ? "breakdown" : "not converged", iters, y.info->true_rel_res);
+        if (worst == TM_OK) worst = status;
+    };
+    for (int q = 0; q < n; ++q) {
+        SolveSys& y = sys[q];
+        bool x0 = false;
+        CKS(is_zero64<NF>(c, y.x64, st, &x0));
+        CKS(true_residual<NF>(c, op, y.shift, y.x64, b64, r64, ax64, mid64, te64, st, &y.rr, x0, dw, q));
+        // an initial guess already within the tolerance is confirmed in FP64
+        if (dw && !x0 && y.rr <= target)
+            CKS(true_residual<NF>(c, op, y.shift, y.x64, b64, r64, ax64, mid64, te64, st, &y.rr, false, false, q));
+        SolverCtl& h = c->h_ctl[q];
         std::memset(&h, 0, sizeof(SolverCtl));
-        h.rr = rr;
-        h.rr_old = rr;
+        h.rr = y.rr;
+        h.rr_old = y.rr;
         h.beta = 0.0;
-        h.shift = shift;
+        h.shift = y.shift;
         h.maxiter = maxiter;
         h.ring = m;
-        h.stop_rr = leg_stop(PS, delta, rr, target);
+        h.stop_rr = leg_stop(PS, delta, y.rr, target);
         h.flag = CTL_RUN;
-        CKS(put_ctl(c, st));
-        int base = 0;   // iterations done before the current run of chunks
-        if (sp->use_graph) {
-            cudaGraph_t graph;
-            CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            for (int it = 0; it < chunk; ++it) {
-                cudaError_t e = cg_iteration<PS, NF>(c, op, xs, ps, m, it % m, rs, mids, tes, st);
-                if (e != cudaSuccess) {
-                    cudaStreamEndCapture(st, &graph);
-                    return fail(TM_ERR_CUDA, "capture: %s", cudaGetErrorString(e));
-                }
-            }
-            CK(cudaStreamEndCapture(st, &graph));
-            CK(cudaGraphInstantiate(&gexec, graph, 0));
-            cudaGraphDestroy(graph);
+        if (!(y.rr > target)) {
+            finish(y, 0, TM_OK);
+            h.flag = CTL_STOP;
+        } else if (PS != P64) {
+            CK((launch_convert<PS, P64, NC, 1>(vb1(c, y.r, r64), nb, st)));
+            CK(cudaMemsetAsync(y.x, 0, spinor_bytes(P32, NC, vh), st));
         }
-        for (;;) {
-            if (gexec) {
-                CK(cudaGraphLaunch(gexec, st));
-            } else {
-                for (int it = 0; it < chunk; ++it) CK((cg_iteration<PS, NF>(c, op, xs, ps, m, it % m, rs, mids, tes, st)));
+        CKS(put_ctl(c, st, q));
+    }
+    cudaGraphExec_t gexec = nullptr;
+    if (running > 0 && sp->use_graph) {
+        cudaGraph_t graph;
+        CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+        for (int it = 0; it < chunk; ++it) {
+            cudaError_t e = cg_iteration<PS, NF, NP>(c, op, sys.data(), n, m, it % m, st);
+            if (e != cudaSuccess) {
+                cudaStreamEndCapture(st, &graph);
+                return fail(TM_ERR_CUDA, "capture: %s", cudaGetErrorString(e));
             }
-            CKS(get_ctl(c, st));
-            if (h.flag == CTL_RUN) continue;
+        }
+        CK(cudaStreamEndCapture(st, &graph));
+        CK(cudaGraphInstantiate(&gexec, graph, 0));
+        cudaGraphDestroy(graph);
+    }
+    while (running > 0) {
+        if (gexec) {
+            CK(cudaGraphLaunch(gexec, st));
+        } else {
+            for (int it = 0; it < chunk; ++it) CK((cg_iteration<PS, NF, NP>(c, op, sys.data(), n, m, it % m, st)));
+        }
+        CKS(get_ctl(c, st, n));
+        for (int q = 0; q < n; ++q) {
+            SolveSys& y = sys[q];
+            SolverCtl& h = c->h_ctl[q];
+            if (y.done || h.flag == CTL_RUN) continue;
             // the steps of the ring that x does not hold yet: the iteration that stopped the
             // run ended before its ring's update, one that broke down does not count
-            const int done = h.iter - base;
+            const int done = h.iter - y.base;
             const int left = h.flag == CTL_BREAKDOWN ? done % m : (done > 0 ? (done - 1) % m + 1 : 0);
             if (left > 0)
-                CK((launch_cg_xupdate<PS, PS == P64 ? P64 : P32, NC>(vb_ring(c, xs, ps, m), left, true, nb, st)));
-            if (h.flag == CTL_BREAKDOWN) { status = TM_ERR_BREAKDOWN; break; }
+                CK((launch_cg_xupdate<PS, PS == P64 ? P64 : P32, NC, 1>(vb_ring(c, y.x, y.p, m, q), left, true, nb, st)));
+            if (h.flag == CTL_BREAKDOWN) {
+                finish(y, h.iter, TM_ERR_BREAKDOWN);
+                continue;
+            }
             // reliable update / convergence check
             if (PS != P64) {
-                CK((launch_add_to64<P32, NC, 1>(vb1(c, x64, xs), nb, st)));
-                CK(cudaMemsetAsync(xs, 0, spinor_bytes(P32, NC, vh), st));
+                CK((launch_add_to64<P32, NC, 1>(vb1(c, y.x64, y.x), nb, st)));
+                CK(cudaMemsetAsync(y.x, 0, spinor_bytes(P32, NC, vh), st));
             }
-            CKS(true_residual<NF>(c, op, shift, x64, b64, r64, ax64, mid64, te64, st, &rr, false, dw));
-            info->reliable_updates += 1;
+            CKS(true_residual<NF>(c, op, y.shift, y.x64, b64, r64, ax64, mid64, te64, st, &y.rr, false, dw, q));
+            y.info->reliable_updates += 1;
             // a double-word residual below the target is confirmed in FP64 (the
             // returned true residual is always an FP64 one)
-            if (dw && rr <= target)
-                CKS(true_residual<NF>(c, op, shift, x64, b64, r64, ax64, mid64, te64, st, &rr));
-            if (rr <= target) break;
-            if (h.flag == CTL_MAXITER || h.iter >= maxiter || !std::isfinite(rr)) {
-                status = std::isfinite(rr) ? TM_ERR_NOT_CONVERGED : TM_ERR_BREAKDOWN;
-                break;
+            if (dw && y.rr <= target)
+                CKS(true_residual<NF>(c, op, y.shift, y.x64, b64, r64, ax64, mid64, te64, st, &y.rr, false, false, q));
+            if (y.rr <= target) {
+                finish(y, h.iter, TM_OK);
+                continue;
             }
-            if (PS != P64) CK((launch_convert<PS, P64, NC, 1>(vb1(c, rs, r64), nb, st)));
+            if (h.flag == CTL_MAXITER || h.iter >= maxiter || !std::isfinite(y.rr)) {
+                finish(y, h.iter, std::isfinite(y.rr) ? TM_ERR_NOT_CONVERGED : TM_ERR_BREAKDOWN);
+                continue;
+            }
+            if (PS != P64) CK((launch_convert<PS, P64, NC, 1>(vb1(c, y.r, r64), nb, st)));
             // the next chunk starts at the beginning of the ring: its first iteration takes
             // the last direction from the end of it
-            if (left > 0 && left != m) CK(cudaMemcpyAsync(ps[m - 1], ps[left - 1], bssz, cudaMemcpyDeviceToDevice, st));
-            base = h.iter;
+            if (left > 0 && left != m) CK(cudaMemcpyAsync(y.p[m - 1], y.p[left - 1], bssz, cudaMemcpyDeviceToDevice, st));
+            y.base = h.iter;
             h.slot = 0;
-            h.beta = rr / h.rr_old;
-            h.rr = rr;
-            h.stop_rr = leg_stop(PS, delta, rr, target);
+            h.beta = y.rr / h.rr_old;
+            h.rr = y.rr;
+            h.stop_rr = leg_stop(PS, delta, y.rr, target);
             h.flag = CTL_RUN;
-            CKS(put_ctl(c, st));
+            CKS(put_ctl(c, st, q));
         }
-        info->iters = h.iter;
-        if (gexec) cudaGraphExecDestroy(gexec);
     }
-    info->true_rel_res = std::sqrt(rr / bb);
-    info->status = status;
-    if (status != TM_OK)
-        fail(status, "solve: %s after %d iterations, true rel res %.3e",
-             status == TM_ERR_BREAKDOWN ? "breakdown" : "not converged", info->iters, info->true_rel_res);
-    return status;
+    if (gexec) cudaGraphExecDestroy(gexec);
+    return worst;
+}
+
+// ns: shifts of the multishift solve whose buffers a group may use
+template <int PS, int NF>
+static tm_status solve_systems(tm_ctx* c, tm_op op, const tm_solve_params* sp, std::vector<SolveSys>& sys, void* b64,
+                               cudaStream_t st, int ns) {
+    int m = 1;
+    CKS((solve_fields<PS, NF>(c, sp, sys, ns, &m)));
+    if constexpr (PS != P64) {
+        if (sys.size() > 1) return solve_core<PS, NF, GROUP>(c, op, sp, sys, m, b64, st);
+    }
+    return solve_core<PS, NF, 1>(c, op, sp, sys, m, b64, st);
 }
 
 template <int NF>
-static tm_status solve_dispatch(tm_ctx* c, tm_op op, double shift, const tm_solve_params* sp, void* x64, void* b64,
-                                tm_solve_info* info, cudaStream_t st) {
+static tm_status solve_dispatch(tm_ctx* c, tm_op op, const tm_solve_params* sp, std::vector<SolveSys>& sys, void* b64,
+                                cudaStream_t st, int ns = 0) {
     switch (sp->sloppy) {
-        case TM_F64: return solve_core<P64, NF>(c, op, shift, sp, x64, b64, info, st);
-        case TM_F32: return solve_core<P32, NF>(c, op, shift, sp, x64, b64, info, st);
-        case TM_BF16: return solve_core<PB16, NF>(c, op, shift, sp, x64, b64, info, st);
-        case TM_F16: return solve_core<PF16, NF>(c, op, shift, sp, x64, b64, info, st);
+        case TM_F64: return solve_systems<P64, NF>(c, op, sp, sys, b64, st, ns);
+        case TM_F32: return solve_systems<P32, NF>(c, op, sp, sys, b64, st, ns);
+        case TM_BF16: return solve_systems<PB16, NF>(c, op, sp, sys, b64, st, ns);
+        case TM_F16: return solve_systems<PF16, NF>(c, op, sp, sys, b64, st, ns);
     }
     return fail(TM_ERR_ARG, "unknown sloppy precision");
 }
+
+// Shifts refined at once: blocks of one place on the lattice then find its links and
+// clover terms in L2 (two-flavour FP32 passes at 24^3x48, per shift: even 89 -> 52 us
+// averaged over an iteration's running and stopped shifts, last 103 -> 60), and a small
+// lattice fills the chip.  Two-flavour multishift solves, ms, one / 2 / 4 / 8 / 12 shifts
+// at once: 24^3x48 12 shifts 674 / 616 / 590 / 590 / 590; 16^3x32 12 shifts 164 / 139 /
+// 129 / 129 / 129; 12^3x24 12 shifts 78.3 / 65.1 / 58.5 / 53.8 / 52.5 (FP16 refinement);
+// 8^2x12x16 10 shifts 39.5 / 29.2 / 24.6 / 21.9 / 21.1.
+static int group_size(long vh) { return vh <= GROW_SITES ? GROUP : 4; }
 
 // canonical (host or device) <-> native FP64 working copies
 static tm_status stage_in(tm_ctx* c, int nf, const double* canon, int stage_id, void* native64, cudaStream_t st) {
@@ -1295,8 +1464,10 @@ extern "C" tm_status tm_solve_cg(tm_ctx* c, tm_op op, const tm_solve_params* sp,
     CKS(ws_get(c, WS_B64, spinor_bytes(P64, 12 * nf, c->vh), &b64));
     CKS(stage_in(c, nf, b, WS_STAGE_B, b64, st));
     CKS(stage_in(c, nf, x, WS_STAGE_X, x64, st));
-    tm_status s = nf == 1 ? solve_dispatch<1>(c, op, 0.0, sp, x64, b64, info, st)
-                          : solve_dispatch<2>(c, op, 0.0, sp, x64, b64, info, st);
+    std::vector<SolveSys> sys(1);
+    sys[0].x64 = x64;
+    sys[0].info = info;
+    tm_status s = nf == 1 ? solve_dispatch<1>(c, op, sp, sys, b64, st) : solve_dispatch<2>(c, op, sp, sys, b64, st);
     CKS(stage_out(c, nf, x, WS_STAGE_X, x64, st));
     CK(cudaStreamSynchronize(st));
     info->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -1377,9 +1548,10 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
     // of the ring all shifts take its iterations at once
     auto iteration = [&](int s) -> cudaError_t {
         void* rp = rs[(s + rm - 1) % rm];
-        cudaError_t e = launch_cg_direction<PS, NC>(vb1(c, ps, rp, ps), nb, st);
+        cudaError_t e = launch_cg_direction<PS, NC, 1>(vb1(c, ps, rp, ps), nb, st);
         if (e != cudaSuccess) return e;
-        e = normal_update<PS, NF>(c, op, rs[s], rp, ps, mids, tes, st, c->ctl, FIN_MS_ALPHA, FIN_MS_UPDATE);
+        const UpdVecs w{rs[s], rp, ps, mids, tes};
+        e = normal_update<PS, NF, 1>(c, op, &w, 1, st, FIN_MS_ALPHA, FIN_MS_UPDATE);
         if (e != cudaSuccess || s + 1 < rm) return e;
         return launch_ms_block<PS, PX, NC>(vb_ring(c, nullptr, rs, rm), mv, rm, false, nb, st);
     };
@@ -1464,12 +1636,21 @@ static tm_status ms_core(tm_ctx* c, tm_op op, int ns, const double* shifts, void
     for (int k = 0; k < ns; ++k) {
         tm_solve_info& inf = infos[order[k]];
         std::memset(&inf, 0, sizeof(inf));
-        if (s != TM_OK) { inf.status = s; continue; }
-        xk[order[k]] = xk64[k];
-        tm_status r = nf == 1 ? solve_dispatch<1>(c, op, sh[k], &rsp, xk64[k], b64, &inf, st)
-                              : solve_dispatch<2>(c, op, sh[k], &rsp, xk64[k], b64, &inf, st);
-        inf.iters += ms_iters;
+        if (s != TM_OK) inf.status = s;
+        else xk[order[k]] = xk64[k];
+    }
+    for (int k = 0; s == TM_OK && k < ns;) {
+        std::vector<SolveSys> sys(std::min(ns - k, rsp.sloppy == TM_F64 ? 1 : group_size(c->vh)));
+        for (size_t q = 0; q < sys.size(); ++q) {
+            sys[q].shift = sh[k + q];
+            sys[q].x64 = xk64[k + q];
+            sys[q].info = &infos[order[k + q]];
+        }
+        const tm_status r = nf == 1 ? solve_dispatch<1>(c, op, &rsp, sys, b64, st, ns)
+                                    : solve_dispatch<2>(c, op, &rsp, sys, b64, st, ns);
+        for (const SolveSys& y : sys) y.info->iters += ms_iters;
         if (r != TM_OK && worst == TM_OK) worst = r;
+        k += (int)sys.size();
     }
     return worst;
 }

@@ -184,11 +184,11 @@ __global__ void __launch_bounds__(BLAS_BS) k_normalize64(const __grid_constant__
 // with a shift 1248 instead of 1920 B.
 // ---------------------------------------------------------------------------
 // p_out = r + beta p_in
-template <int P, int NC>
-__global__ void __launch_bounds__(BLAS_BS) k_cg_direction(const __grid_constant__ VecBatch<1> b) {
+template <int P, int NC, int NP>
+__global__ void __launch_bounds__(BLAS_BS) k_cg_direction(const __grid_constant__ VecBatch<NP> b) {
     using R = typename PT<P>::R;
     pdl_wait();
-    TM_VEC_PROLOGUE(1)
+    TM_VEC_PROLOGUE(NP)
     if (pr.ctl->flag != CTL_RUN) return;
     const R beta = (R)pr.ctl->beta;
     const bool want = pr.ctl->shift != 0.0;
@@ -220,13 +220,13 @@ __global__ void __launch_bounds__(BLAS_BS) k_cg_direction(const __grid_constant_
 }
 
 // x += sum_{i < n} alpha_i p_i, a vector of reals at a time (one thread per site and vector)
-template <int P, int PX, int NC>
-__global__ void __launch_bounds__(BLAS_BS) k_cg_xupdate(const __grid_constant__ VecBatch<1> b, int n, bool always) {
+template <int P, int PX, int NC, int NP>
+__global__ void __launch_bounds__(BLAS_BS) k_cg_xupdate(const __grid_constant__ VecBatch<NP> b, int n, bool always) {
     using R = typename PT<P>::R;
     using RX = typename PT<PX>::R;
     constexpr int W = PT<P>::W;
     pdl_wait();
-    const VecProb& pr = b.p[0];
+    const VecProb& pr = b.p[blockIdx.z];
     if (!always && pr.ctl->flag != CTL_RUN) return;
     const long vh = pr.vh, i = (long)blockIdx.x * BLAS_BS + threadIdx.x;
     if (i >= vh) return;
@@ -396,13 +396,13 @@ cudaError_t launch_normalize64(const VecBatch<1>& b, int nb, cudaStream_t st) {
     k_normalize64<NC><<<nb, BLAS_BS, 0, st>>>(b);
     return cudaGetLastError();
 }
-template <int P, int NC>
-cudaError_t launch_cg_direction(const VecBatch<1>& b, int nb, cudaStream_t st) {
-    return launch_chained(k_cg_direction<P, NC>, nb, BLAS_BS, 0, st, true, b);
+template <int P, int NC, int NP>
+cudaError_t launch_cg_direction(const VecBatch<NP>& b, int nb, cudaStream_t st) {
+    return launch_chained(k_cg_direction<P, NC, NP>, nb, BLAS_BS, 0, st, true, b);
 }
-template <int P, int PX, int NC>
-cudaError_t launch_cg_xupdate(const VecBatch<1>& b, int n, bool always, int nb, cudaStream_t st) {
-    k_cg_xupdate<P, PX, NC><<<dim3(nb, 2 * NC / PT<P>::W), BLAS_BS, 0, st>>>(b, n, always);
+template <int P, int PX, int NC, int NP>
+cudaError_t launch_cg_xupdate(const VecBatch<NP>& b, int n, bool always, int nb, cudaStream_t st) {
+    k_cg_xupdate<P, PX, NC, NP><<<dim3(nb, 2 * NC / PT<P>::W, b.n), BLAS_BS, 0, st>>>(b, n, always);
     return cudaGetLastError();
 }
 template <int P, int PX, int NC>
@@ -425,8 +425,8 @@ cudaError_t launch_export(double* dst, const void* src, long vh, cudaStream_t st
 // explicit instantiations
 #define TM_PX(P) ((P) == P64 ? P64 : P32)
 #define TM_BLAS_P_NC(P, NC)                                                                              \
-    template cudaError_t launch_cg_direction<P, NC>(const VecBatch<1>&, int, cudaStream_t);               \
-    template cudaError_t launch_cg_xupdate<P, TM_PX(P), NC>(const VecBatch<1>&, int, bool, int, cudaStream_t); \
+    template cudaError_t launch_cg_direction<P, NC, 1>(const VecBatch<1>&, int, cudaStream_t);            \
+    template cudaError_t launch_cg_xupdate<P, TM_PX(P), NC, 1>(const VecBatch<1>&, int, bool, int, cudaStream_t); \
     template cudaError_t launch_ms_block<P, TM_PX(P), NC>(const VecBatch<1>&, const MsVecs&, int, bool, int, cudaStream_t); \
     template cudaError_t launch_add_to64<P, NC, 1>(const VecBatch<1>&, int, cudaStream_t);               \
     template cudaError_t launch_norm2<P, NC, 1>(const VecBatch<1>&, int, cudaStream_t);                  \
@@ -441,6 +441,12 @@ TM_BLAS_P(P64)
 TM_BLAS_P(P32)
 TM_BLAS_P(PB16)
 TM_BLAS_P(PF16)
+#define TM_GROUP(P, NC)                                                                                 \
+    template cudaError_t launch_cg_direction<P, NC, GROUP>(const VecBatch<GROUP>&, int, cudaStream_t);   \
+    template cudaError_t launch_cg_xupdate<P, P32, NC, GROUP>(const VecBatch<GROUP>&, int, bool, int, cudaStream_t);
+TM_GROUP(P32, 12) TM_GROUP(P32, 24)
+TM_GROUP(PB16, 12) TM_GROUP(PB16, 24)
+TM_GROUP(PF16, 12) TM_GROUP(PF16, 24)
 #define TM_CONV2(P, NC, NP)                                                                 \
     template cudaError_t launch_convert<P, P64, NC, NP>(const VecBatch<NP>&, int, cudaStream_t); \
     template cudaError_t launch_convert<P64, P, NC, NP>(const VecBatch<NP>&, int, cudaStream_t);

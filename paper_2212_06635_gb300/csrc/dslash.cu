@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
     const OpProb& pr = b.p[k];
     pdl_wait();
     if (pr.ctl != nullptr && pr.ctl->flag != CTL_RUN) return;
-    const int lb = blockIdx.x - b.blk_start[k];
+    const int lb = block_in_problem<NP>(b, blockIdx.x, k);
     const long i = (long)lb * BS + threadIdx.x;
     const bool valid = i < pr.g.vh;
     const int po = (KIND == K1_EO_INV) ? 0 : 1;   // output parity
@@ -277,5 +277,11 @@ TM_INST_P(P64)
 TM_INST_P(P32)
 TM_INST_P(PB16)
 TM_INST_P(PF16)
+#define TM_INST_GROUP(P)                                                                             \
+    TM_INST(P, 1, K1_EO_INV, GROUP) TM_INST(P, 1, K2_OE_LOCAL, GROUP) TM_INST(P, 1, K2_UPDATE, GROUP) \
+    TM_INST(P, 2, K2_OE_LOCAL, GROUP) TM_INST(P, 2, K2_UPDATE, GROUP)
+TM_INST_GROUP(P32)
+TM_INST_GROUP(PB16)
+TM_INST_GROUP(PF16)
 
 }  // namespace tmk

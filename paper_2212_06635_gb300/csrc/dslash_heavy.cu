@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, KIND>())) dslash_heav
     const OpProb& pr = b.p[k];
     pdl_wait();
     if (pr.ctl != nullptr && pr.ctl->flag != CTL_RUN) return;
-    const int lb = blockIdx.x - b.blk_start[k];
+    const int lb = block_in_problem<NP>(b, blockIdx.x, k);
     const long gt = (long)lb * BS + threadIdx.x;
     const long i = gt >> 1;
     const int f = (int)(gt & 1);
@@ -196,14 +196,17 @@ template <int P, int NF, int KIND, int NP>
 cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st);
 
 // the two-flavour even-pass instantiations of launch_dslash: nblocks covers 2 vh threads
-#define TM_HEAVY_INST(P, KIND)                                                                        \
+#define TM_HEAVY_INST(P, KIND, NP)                                                                    \
     template <>                                                                                       \
-    cudaError_t launch_dslash<P, 2, KIND, 1>(const OpBatch<1>& b, int nblocks, cudaStream_t st) {     \
-        return launch_chained(dslash_heavy_kernel<P, KIND, 1, dslash_bs(P)>, nblocks, dslash_bs(P), 0, st, b.chained, b); \
+    cudaError_t launch_dslash<P, 2, KIND, NP>(const OpBatch<NP>& b, int nblocks, cudaStream_t st) {   \
+        return launch_chained(dslash_heavy_kernel<P, KIND, NP, dslash_bs(P)>, nblocks, dslash_bs(P), 0, st, b.chained, b); \
     }
-TM_HEAVY_INST(P64, K1_EO_INV)
-TM_HEAVY_INST(P32, K1_EO_INV)
-TM_HEAVY_INST(PB16, K1_EO_INV)
-TM_HEAVY_INST(PF16, K1_EO_INV)
+TM_HEAVY_INST(P64, K1_EO_INV, 1)
+TM_HEAVY_INST(P32, K1_EO_INV, 1)
+TM_HEAVY_INST(PB16, K1_EO_INV, 1)
+TM_HEAVY_INST(PF16, K1_EO_INV, 1)
+TM_HEAVY_INST(P32, K1_EO_INV, GROUP)
+TM_HEAVY_INST(PB16, K1_EO_INV, GROUP)
+TM_HEAVY_INST(PF16, K1_EO_INV, GROUP)
 
 }  // namespace tmk

@@ -326,6 +326,9 @@ struct MsCtl {
 // problem descriptors for batched kernels (one block belongs to one problem)
 // ---------------------------------------------------------------------------
 constexpr int MAXP = 32;
+// a group: right-hand sides of one operator on one lattice (the shifts of a multishift
+// solve while they are refined)
+constexpr int GROUP = MAX_SHIFTS;
 
 struct Geom {
     int X, Y, Z, T;
@@ -374,12 +377,21 @@ struct OpBatch {
 
 enum FinOp { FIN_NONE = 0, FIN_STORE = 1, FIN_CG_ALPHA = 2, FIN_MS_ALPHA = 3 };
 
+// The problem that a block works on, and the block's index in it.  Batches run problem
+// after problem; the problems of a group block by block, since blocks that read the
+// same links and clover terms then run together and find them in L2.
 template <int NP>
 __device__ __forceinline__ int find_problem(const OpBatch<NP>& b, int blk) {
+    if constexpr (NP == GROUP) return blk % (unsigned)b.n;
     int k = 0;
 #pragma unroll 1
     while (k + 1 < b.n && blk >= b.blk_start[k + 1]) ++k;
     return k;
+}
+template <int NP>
+__device__ __forceinline__ int block_in_problem(const OpBatch<NP>& b, int blk, int k) {
+    if constexpr (NP == GROUP) return blk / (unsigned)b.n;
+    return blk - b.blk_start[k];
 }
 
 // site coordinates of checkerboard index i of parity par

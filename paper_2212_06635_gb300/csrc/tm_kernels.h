@@ -229,12 +229,12 @@ cudaError_t launch_cg_pupdate(const VecBatch<NP>& b, int nblocks, cudaStream_t s
 template <int P, int PX, int NC, int NP>
 cudaError_t launch_cg_update(const VecBatch<NP>& b, int nblocks, cudaStream_t st);
 // p_out = r + beta p_in (+ ||p_out||^2 when the problem has a shift)           v = {p_out, r, p_in}
-template <int P, int NC>
-cudaError_t launch_cg_direction(const VecBatch<1>& b, int nblocks, cudaStream_t st);
+template <int P, int NC, int NP>
+cudaError_t launch_cg_direction(const VecBatch<NP>& b, int nblocks, cudaStream_t st);
 // x += sum_{i < n} alpha_i p_i, alpha_i = ctl->alpha_ring[i] (n <= RING)         v = {x, -, p_0, ...};
-// only while the problem runs, unless `always`
-template <int P, int PX, int NC>
-cudaError_t launch_cg_xupdate(const VecBatch<1>& b, int n, bool always, int nblocks, cudaStream_t st);
+// only while the problem runs, unless `always`; nblocks per problem (all of one size)
+template <int P, int PX, int NC, int NP>
+cudaError_t launch_cg_xupdate(const VecBatch<NP>& b, int n, bool always, int nblocks, cudaStream_t st);
 // dst (precision PD) = src (precision PS)                        v = {dst, src}
 template <int PD, int PS, int NC, int NP>
 cudaError_t launch_convert(const VecBatch<NP>& b, int nblocks, cudaStream_t st);

@@ -394,3 +394,40 @@ def test_rings_of_directions_match_single_steps(prec, nf):
                 assert float((x - r).norm() / r.norm()) < 1e-7
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("dims,ns,nf,sloppy,refine,chunk,graph", [
+    ((4, 4, 4, 4), 16, 2, 1, 1, 16, 1),          # all shifts at once, fewer sites than a block
+    ((6, 4, 6, 10), 3, 1, 1, 3, 3, 0),           # ragged blocks, no ring, no graph
+    ((6, 4, 6, 10), 16, 2, 3, 2, 16, 1),
+    ((16, 16, 16, 18), 9, 2, 1, 1, 16, 1),       # groups limited by the multishift's buffers
+    ((16, 16, 16, 18), 5, 1, 3, 1, 16, 1),       # (whose 16-bit directions are too small for FP32)
+    ((16, 16, 16, 18), 5, 2, 0, 3, 4, 0),        # (and which are absent after an FP64 multishift)
+    ((16, 16, 16, 18), 2, 1, 1, 2, 2, 1),
+])
+def test_shifts_refined_in_groups(dims, ns, nf, sloppy, refine, chunk, graph):
+    """Shifts are refined several at a time, each with its own stopping point: every
+    solution meets the tolerance by the FP64 operator, and a second call, with the
+    buffers of the first, gives the same values."""
+    import torch
+    from paper_2212_06635_gb300 import tm
+    act = dict(mu=0.01) if nf == 1 else dict(mu=0.0, mubar=0.1246, epsbar=0.1350)
+    lat = Lat(F.gauge_field(dims, 91), dims, 0.1394, CSW, **act)
+    op = tm.TM_MDAGM if nf == 1 else tm.TM_QH_SQ
+    shifts = [1e-4 * 3e4 ** (k / (ns - 1)) for k in range(ns)][::-1]
+    try:
+        b = to_dev(F.odd_spinor(dims, 92, nf))
+        sp = tm.solve_params(tol=1e-10, sloppy=sloppy, refine=refine, chunk=chunk, use_graph=graph)
+        runs = []
+        for _ in range(2):
+            xs = [torch.zeros_like(b) for _ in shifts]
+            infos = tm.tm_solve_multishift(lat.ctx, op, shifts, xs, b, sp)
+            assert all(i.status == 0 and i.true_rel_res <= 1e-10 and i.iters > 0 for i in infos)
+            runs.append(xs)
+        for s, x, y in zip(shifts, *runs):
+            assert torch.equal(x, y)
+            shape = F.odd_spinor(dims, 92, nf).shape
+            r = from_dev(b, shape) - lat.apply(op, 0, from_dev(x, shape)) - s * from_dev(x, shape)
+            assert np.linalg.norm(r) <= 1.01e-10 * np.linalg.norm(from_dev(b, shape)), s
+    finally:
+        lat.close()
