@@ -431,3 +431,22 @@ def test_shifts_refined_in_groups(dims, ns, nf, sloppy, refine, chunk, graph):
             assert np.linalg.norm(r) <= 1.01e-10 * np.linalg.norm(from_dev(b, shape)), s
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("sloppy,delta", [(1, 0.0), (3, 0.0), (2, 0.0), (1, 1e-6), (3, 1e-3), (3, 0.3)])
+def test_returned_residual_of_a_mixed_solve_is_the_fp64_one(sloppy, delta):
+    """Legs whose iterated residual has met the target are confirmed in FP64 at once,
+    others after a double-word residual; with a threshold far below what the storage
+    carries the iterated residual says little, and further legs follow."""
+    dims = (6, 4, 6, 10)
+    op, lat = _lat(dims, 1260)
+    tm = lat.tm
+    try:
+        b = F.odd_spinor(dims, 2260)
+        x = to_dev(np.zeros_like(b))
+        info = tm.tm_solve_cg(lat.ctx, tm.TM_MDAGM, tm.solve_params(tol=1e-11, sloppy=sloppy, delta=delta), x, to_dev(b))
+        res = S.rel_residual(op.MdagM, from_dev(x, b.shape), b)
+        assert info.status == 0 and info.true_rel_res <= 1e-11
+        assert abs(info.true_rel_res - res) <= 1e-2 * res
+    finally:
+        lat.close()
