@@ -438,10 +438,10 @@ static OpProb make_prob(const tm_ctx* c, int P, int nf, int kind, int sign, void
 }
 
 // out = Q_hat(sign) in (+ i rho in for W_hat), via the even temporary te.
-// fin != FIN_NONE fuses ||out||^2.
+// fin != FIN_NONE fuses ||out||^2.  out64: a double-word result is stored as FP64.
 template <int P, int NF>
 static cudaError_t schur(const tm_ctx* c, int sign, void* out, const void* in, void* te, cudaStream_t st,
-                         SolverCtl* ctl, int fin, double rho = 0.0, bool chained = false) {
+                         SolverCtl* ctl, int fin, double rho = 0.0, bool chained = false, bool out64 = false) {
     OpBatch<1> b{};
     b.n = 1;
     b.chained = chained;
@@ -457,6 +457,9 @@ static cudaError_t schur(const tm_ctx* c, int sign, void* out, const void* in, v
     b.fin = fin;
     b.p[0] = make_prob(c, P, NF, K2_OE_LOCAL, sign, out, te, in, ctl, fin != FIN_NONE, rho);
     b.blk_start[1] = b.p[0].nblk;
+    if constexpr (P == PDF) {
+        if (out64) return launch_dslash<PDF, NF, K2_OUT64, 1>(b, b.p[0].nblk, st);
+    }
     return launch_pass<P, NF, K2_OE_LOCAL, 1>(v2, b, b.p[0].nblk, st);
 }
 
@@ -467,7 +470,8 @@ static void normal_signs(tm_op op, int* s1, int* s2) {
     else { *s1 = -1; *s2 = +1; }                       // Qh Qh^+
 }
 
-// out = A in for a normal op, fin fused into the first factor (||Q in||^2 = <in, A in>)
+// out = A in for a normal op, fin fused into the first factor (||Q in||^2 = <in, A in>);
+// from a double-word field an FP64 one
 template <int P, int NF>
 static cudaError_t normal_op(const tm_ctx* c, tm_op op, void* out, const void* in, void* mid, void* te,
                              cudaStream_t st, SolverCtl* ctl, int fin) {
@@ -476,7 +480,7 @@ static cudaError_t normal_op(const tm_ctx* c, tm_op op, void* out, const void* i
     const double rt = is_what(op) ? 2.0 * c->params.kappa * c->params.rho : 0.0;
     cudaError_t e = schur<P, NF>(c, s1, mid, in, te, st, ctl, fin, s1 * rt);
     if (e != cudaSuccess) return e;
-    return schur<P, NF>(c, s2, out, mid, te, st, ctl, FIN_NONE, s2 * rt, true);
+    return schur<P, NF>(c, s2, out, mid, te, st, ctl, FIN_NONE, s2 * rt, true, P == PDF);
 }
 
 // Reduction scratch of problem q of a group.
@@ -545,12 +549,13 @@ static tm_status apply_t(tm_ctx* c, tm_op op, void* out, const void* in, cudaStr
     void *te = nullptr, *mid = nullptr;
     CKS(ws_get(c, WS_APPLY_TE, spinor_bytes(P, 12 * NF, c->vh), &te));
     if (op == TM_QHAT_PLUS || op == TM_QH) {
-        CK(schur<P, NF>(c, +1, out, in, te, st, nullptr, FIN_NONE));
+        CK(schur<P, NF>(c, +1, out, in, te, st, nullptr, FIN_NONE, 0.0, false, P == PDF));
     } else if (op == TM_QHAT_MINUS || op == TM_QH_DAG) {
-        CK(schur<P, NF>(c, -1, out, in, te, st, nullptr, FIN_NONE));
+        CK(schur<P, NF>(c, -1, out, in, te, st, nullptr, FIN_NONE, 0.0, false, P == PDF));
     } else if (op == TM_WHAT_PLUS || op == TM_WHAT_MINUS) {
         const int sg = op == TM_WHAT_PLUS ? +1 : -1;
-        CK(schur<P, NF>(c, sg, out, in, te, st, nullptr, FIN_NONE, sg * 2.0 * c->params.kappa * c->params.rho));
+        CK(schur<P, NF>(c, sg, out, in, te, st, nullptr, FIN_NONE, sg * 2.0 * c->params.kappa * c->params.rho, false,
+                        P == PDF));
     } else {
         CKS(ws_get(c, WS_APPLY_MID, spinor_bytes(P, 12 * NF, c->vh), &mid));
         CK(normal_op<P, NF>(c, op, out, in, mid, te, st, nullptr, FIN_NONE));
@@ -621,8 +626,7 @@ extern "C" tm_status tm_apply_Mhat(tm_ctx* c, tm_op op, tm_prec prec, void* out,
     return fail(TM_ERR_ARG, "tm_apply_Mhat: unknown precision");
 }
 
-// op(in) in double-word arithmetic on native FP64 fields (out doubles as the
-// double-word result and is converted in place)
+// op(in) in double-word arithmetic on native FP64 fields
 template <int NF>
 static tm_status apply_dw_t(tm_ctx* c, tm_op op, void* out, const void* in, cudaStream_t st) {
     const long n16 = 12 * NF * c->vh;
@@ -631,7 +635,6 @@ static tm_status apply_dw_t(tm_ctx* c, tm_op op, void* out, const void* in, cuda
     CKS(ws_get(c, WS_XDF, spinor_bytes(PDF, 12 * NF, c->vh), &xdf));
     CK(launch_f64_to_df(xdf, in, n16, st));
     CKS(apply_t<PDF, NF>(c, op, out, xdf, st));
-    CK(launch_df_to_f64(out, out, n16, st));
     return TM_OK;
 }
 
@@ -1047,10 +1050,10 @@ static tm_status get_ctl(tm_ctx* c, cudaStream_t st, int n = 1) {
 
 // r = b - (A + shift) x and rr = ||r||^2 in FP64.  x_zero: x is known to be zero,
 // so A x = 0 without applying the operator (a zero initial guess).  dw: A x in
-// double-word arithmetic (x and the result rounded to a 48-bit significand on the
-// way in and out; mid64, te64 and ax64 serve as double-word scratch), for the
-// reliable updates inside a mixed-precision solve; otherwise native FP64.  q: the
-// problem of a group whose control word holds the shift.
+// double-word arithmetic (x rounded to a 48-bit significand on the way in; mid64 and
+// te64 serve as double-word scratch), for the reliable updates inside a
+// mixed-precision solve; otherwise native FP64.  q: the problem of a group whose
+// control word holds the shift.
 template <int NF>
 static tm_status true_residual(tm_ctx* c, tm_op op, double shift, void* x64, void* b64, void* r64, void* ax64,
                                void* mid64, void* te64, cudaStream_t st, double* rr, bool x_zero = false,
@@ -1064,7 +1067,6 @@ static tm_status true_residual(tm_ctx* c, tm_op op, double shift, void* x64, voi
         CKS(ws_get(c, WS_XDF, spinor_bytes(PDF, 12 * NF, c->vh), &xdf));
         CK(launch_f64_to_df(xdf, x64, n16, st));
         CK((normal_op<PDF, NF>(c, op, ax64, xdf, mid64, te64, st, nullptr, FIN_NONE)));
-        CK(launch_df_to_f64(ax64, ax64, n16, st));
     } else {
         CK((normal_op<P64, NF>(c, op, ax64, x64, mid64, te64, st, nullptr, FIN_NONE)));
     }
@@ -1406,9 +1408,9 @@ static tm_status solve_dispatch(tm_ctx* c, tm_op op, const tm_solve_params* sp, 
 }
 
 // Shifts refined at once: blocks of one place on the lattice then find its links and
-// clover terms in L2 (two-flavour FP32 passes at 24^3x48, per shift: even 89 -> 52 us
-// averaged over an iteration's running and stopped shifts, last 103 -> 60), and a small
-// lattice fills the chip.  Two-flavour multishift solves, ms, one / 2 / 4 / 8 / 12 shifts
+// clover terms in L2 (two-flavour FP32 passes at 24^3x48 inside the solver, per running
+// shift: even 89 -> 71 us, odd 92 -> 68 us, last 103 -> 79 us), and a small lattice fills
+// the chip.  Two-flavour multishift solves, ms, one / 2 / 4 / 8 / 12 shifts
 // at once: 24^3x48 12 shifts 674 / 616 / 590 / 590 / 590; 16^3x32 12 shifts 164 / 139 /
 // 129 / 129 / 129; 12^3x24 12 shifts 78.3 / 65.1 / 58.5 / 53.8 / 52.5 (FP16 refinement);
 // 8^2x12x16 10 shifts 39.5 / 29.2 / 24.6 / 21.9 / 21.1.
@@ -1523,15 +1525,12 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
     for (int k = 0; k < ns; ++k) CK(cudaMemcpyAsync(mv.p[k], rs[rm - 1], bs, cudaMemcpyDeviceToDevice, st));   // p_k = r
     // The sloppy multishift stops each shift when its recursively updated residual
     // falls below floor_tol; the shift-by-shift refinement takes it to sp->tol.
-    // Swept on the heavy doublet at 24^3x48 (12 shifts, time of the whole solve
-    // with refinement): FP32 1e-6 / 1e-7 / 1e-8 / 1e-9 / 1e-10 -> 0.721 / 0.631 /
-    // 0.594 / 0.611 / 0.634 s; 16-bit 2e-4 / 5e-5 / 1e-5 / 1e-6 -> 0.972 / 0.936 /
-    // 0.870 / 0.892 s.  Below the storage's own precision the sloppy solutions
-    // still improve (the reductions are FP64), and a refinement iteration costs
-    // about half a multishift one, until the extra multishift iterations stop
-    // paying.  With the shifts refined in groups: FP32 1e-6 / 1e-7 / 1e-8 / 3e-9 / 1e-9 ->
-    // 0.645 / 0.602 / 0.586 / 0.599 / 0.603 s; 16-bit 2e-4 / 5e-5 / 1e-5 / 3e-6 / 1e-6 ->
-    // 0.925 / 0.926 / 0.822 / 0.839 / 0.850 s (tolerance 1e-12).
+    // Swept on the heavy doublet at 24^3x48 (12 shifts to 1e-12, time of the whole
+    // solve with refinement): FP32 1e-6 / 1e-7 / 1e-8 / 3e-9 / 1e-9 -> 0.645 / 0.602 /
+    // 0.586 / 0.599 / 0.603 s; 16-bit 2e-4 / 5e-5 / 1e-5 / 3e-6 / 1e-6 -> 0.925 / 0.926 /
+    // 0.822 / 0.839 / 0.850 s.  Below the storage's own precision the sloppy solutions
+    // still improve (the reductions are FP64), and one multishift iteration serves all
+    // shifts, until the extra ones stop paying.
     const double floor_tol = PS == P64 ? 0.0 : (PS == P32 ? 1e-8 : 1e-5);
     const double ms_tol = std::max(sp->tol, floor_tol);
     MsCtl& m = *c->h_ms;

@@ -30,6 +30,8 @@
 // operator 3022 -> 2264 us against loads at the point of use, rows unrolled, at the
 // same errors (8.0e-15 / 8.5e-15).  Pairing the two hops of a direction as the FP64
 // passes do (36 compensated additions instead of 48) gives 8.1e-15 and is not used.
+// The operator's last pass stores FP64 itself: its conversions (2 per cycle and SM) hide
+// behind the FP32 work, as a kernel of their own they took 43 us (light, 905 -> 865 us).
 #include "tm_internal.h"
 #include "tm_kernels.h"
 #include "dslash_common.cuh"
@@ -397,7 +399,13 @@ __global__ void __launch_bounds__(DSLASH_BS, 4) dslash_dw_kernel(const __grid_co
                 herm6_row_dw(s, slots, v, r);
                 const cpx<df> w = cc_get(s);
                 const cpx<df> o = C(df(sc * w.re.h, sc * w.re.l), df(sc * w.im.h, sc * w.im.l));
-                store_reals<PDF, 2>(pr.out, vh, i, 24 * f + 2 * (6 * cb + r), reinterpret_cast<const df*>(&o));
+                const int off = 24 * f + 2 * (6 * cb + r);
+                if constexpr (KIND == K2_OUT64) {
+                    const double q[2] = {(double)o.re, (double)o.im};
+                    store_reals<P64, 2>(pr.out, vh, i, off, q);
+                } else {
+                    store_reals<PDF, 2>(pr.out, vh, i, off, reinterpret_cast<const df*>(&o));
+                }
             }
             if (cb == 0) {
                 dw_fetch<18>(slots, 0, pr.clov, vh, 18, i);   // A_1
@@ -425,5 +433,7 @@ TM_DW_INST(1, K1_EO_INV)
 TM_DW_INST(1, K2_OE_LOCAL)
 TM_DW_INST(2, K1_EO_INV)
 TM_DW_INST(2, K2_OE_LOCAL)
+TM_DW_INST(1, K2_OUT64)
+TM_DW_INST(2, K2_OUT64)
 
 }  // namespace tmk

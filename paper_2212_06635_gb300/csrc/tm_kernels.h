@@ -18,7 +18,8 @@ constexpr int MIN_BS = 32;       // fewest sites per block of any reducing kerne
 
 // K2_UPDATE: the odd pass of the second factor of a normal operator with the residual
 // update in its epilogue, r_out = r - alpha (out + shift p), ||r_out||^2
-enum DslashKind { K1_EO_INV = 0, K2_OE_LOCAL = 1, K2_UPDATE = 2 };
+// K2_OUT64 (double-word passes): K2_OE_LOCAL with the result stored as FP64
+enum DslashKind { K1_EO_INV = 0, K2_OE_LOCAL = 1, K2_UPDATE = 2, K2_OUT64 = 3 };
 constexpr int RING = 4;   // search directions kept between two updates of the solutions
 
 // FinOp codes beyond those in tm_internal.h
@@ -267,6 +268,5 @@ cudaError_t launch_links_from64(void* dst, const void* src64, long vh, cudaStrea
 template <int P>
 cudaError_t launch_clover_from64(void* dst, const double* src, long vh, int nreal, cudaStream_t st);
 cudaError_t launch_f64_to_df(void* dst, const void* src, long n, cudaStream_t st);
-cudaError_t launch_df_to_f64(void* dst, const void* src, long n, cudaStream_t st);
 
 }  // namespace tmk
