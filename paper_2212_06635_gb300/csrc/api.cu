@@ -375,9 +375,10 @@ static const void* clovH_ptr(const tm_ctx* c, int P) {
 //   light FP32 20.6 / 16.0, 20.7 / 18.6, 22.7 / 22.7; light FP16 22.7 / 16.7,
 //   22.6 / 20.7, 22.8 / 22.7; light FP64 156 / 62, 161 / 132, 233 / 216 (38,416 sites:
 //   305 / 348); heavy FP32 24.8 / 20.7, 27.7 / 34.9; heavy FP16 26.9 / 22.7,
-//   28.8 / 39.1; heavy FP64 260 / 102, 313 / 294, 487 / 498.
+//   28.8 / 39.1; heavy FP64 178 / 102, 262 / 294, 447 / 498 (6,144 sites: 182 / 198;
+//   4864 are one wave of the split kernel).
 static long split_limit(int P, int nf) {
-    if (P == P64) return nf == 1 ? 24576 : 12288;
+    if (P == P64) return nf == 1 ? 24576 : 4864;
     return nf == 1 ? 12288 : 6144;
 }
 
@@ -392,12 +393,12 @@ static int pass_kernel(const tm_ctx* c, int kind) {
     return P == PDF ? 0 : pass_kernel(P, c->vh, NF, c->variant[P][NF - 1][kind]);
 }
 
-// blocks of a pass: one thread per site, except the direct two-flavour even pass
-// (a thread per site and flavour) and the double-word passes (likewise)
+// blocks of a pass: one thread per site, except the direct two-flavour even pass, the
+// FP64 odd one and the double-word passes (a thread per site and flavour)
 static int pass_nblk(int P, long vh, int nf, int kind, int kernel) {
     if (P == PDF) return nblk((long)nf * vh, DSLASH_BS);
     if (kernel == PK_SPLIT) return nblk(vh, SPLIT_SITES);
-    return kernel == PK_STAGED ? nblk(vh, STAGED_BS) : nblk(nf == 2 && kind == K1_EO_INV ? 2 * vh : vh, dslash_bs(P));
+    return kernel == PK_STAGED ? nblk(vh, STAGED_BS) : nblk(nf == 2 && (kind == K1_EO_INV || P == P64) ? 2 * vh : vh, dslash_bs(P));
 }
 
 // launch one pass in the variant the context chose for (P, NF, KIND)

@@ -16,37 +16,6 @@
 
 namespace tmk {
 
-// out = r - alpha (out + shift p) with the residual and search direction of site i, a
-// vector of reals at a time: the update of CG without a stored A p (alpha is known
-// before the second factor of the operator is applied)
-template <int P, int NC>
-__device__ __forceinline__ void residual_update(cpx<typename PT<P>::R>* out, const OpProb& pr, long i) {
-    using R = typename PT<P>::R;
-    constexpr int W = PT<P>::W;
-    const long vh = pr.g.vh;
-    const R alpha = (R)pr.ctl->alpha, shift = (R)pr.ctl->shift;
-    R* o = reinterpret_cast<R*>(out);
-    R rs = (R)1, ps = (R)1;
-    if constexpr (P == PB16 || P == PF16) {
-        const size_t off = (size_t)vh * NC * 4;
-        rs = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.r) + off)[i];
-        ps = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.p) + off) + i);
-    }
-#pragma unroll
-    for (int v = 0; v < 2 * NC / W; ++v) {
-        if (shift != (R)0) {
-            R p[W];
-            load_reals<P, W>(pr.p, vh, i, W * v, p);
-#pragma unroll
-            for (int e = 0; e < W; ++e) o[W * v + e] += shift * (ps * p[e]);
-        }
-        R r[W];
-        load_reals<P, W>(pr.r, vh, i, W * v, r);
-#pragma unroll
-        for (int e = 0; e < W; ++e) o[W * v + e] = rs * r[e] - alpha * o[W * v + e];
-    }
-}
-
 // Whether the first hop writes the accumulators instead of adding to zeros (which
 // saves 24 additions a flavour, but moves the register allocation): per pass what
 // measured faster.  Adding / writing, us: light FP16 even 106.6 / 110.6, odd 102.3 /
@@ -178,7 +147,7 @@ constexpr int dslash_min_blocks() {
 
 template <int P, int NF, int KIND, int NP, int BS>
 __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash_kernel(const __grid_constant__ OpBatch<NP> b) {
-    static_assert(NF == 1 || KIND != K1_EO_INV, "the two-flavour even pass lives in dslash_heavy.cu");
+    static_assert(NF == 1 || (KIND != K1_EO_INV && P != P64), "two-flavour passes of dslash_heavy.cu");
     using R = typename PT<P>::R;
     __shared__ double sh[BS / 32];
     const int k = find_problem<NP>(b, blockIdx.x);
@@ -269,14 +238,13 @@ cudaError_t launch_dslash(const OpBatch<NP>& b, int nblocks, cudaStream_t st) {
 #define TM_INST(P, NF, KIND, NP) \
     template cudaError_t launch_dslash<P, NF, KIND, NP>(const OpBatch<NP>&, int, cudaStream_t);
 #define TM_INST_P(P)                                                                      \
-    TM_INST(P, 1, K1_EO_INV, 1) TM_INST(P, 1, K2_OE_LOCAL, 1) TM_INST(P, 2, K2_OE_LOCAL, 1) \
-    TM_INST(P, 1, K2_UPDATE, 1) TM_INST(P, 2, K2_UPDATE, 1)                                \
+    TM_INST(P, 1, K1_EO_INV, 1) TM_INST(P, 1, K2_OE_LOCAL, 1) TM_INST(P, 1, K2_UPDATE, 1) \
     TM_INST(P, 1, K1_EO_INV, MAXP) TM_INST(P, 1, K2_OE_LOCAL, MAXP)
-TM_INST_P(P64)
-// (the double-word passes: dslash_dw.cu)
-TM_INST_P(P32)
-TM_INST_P(PB16)
-TM_INST_P(PF16)
+#define TM_INST_TWO(P) TM_INST(P, 2, K2_OE_LOCAL, 1) TM_INST(P, 2, K2_UPDATE, 1)
+TM_INST_P(P64)   // (its two-flavour odd pass: dslash_heavy.cu; the double-word passes: dslash_dw.cu)
+TM_INST_P(P32) TM_INST_TWO(P32)
+TM_INST_P(PB16) TM_INST_TWO(PB16)
+TM_INST_P(PF16) TM_INST_TWO(PF16)
 #define TM_INST_GROUP(P)                                                                             \
     TM_INST(P, 1, K1_EO_INV, GROUP) TM_INST(P, 1, K2_OE_LOCAL, GROUP) TM_INST(P, 1, K2_UPDATE, GROUP) \
     TM_INST(P, 2, K2_OE_LOCAL, GROUP) TM_INST(P, 2, K2_UPDATE, GROUP)

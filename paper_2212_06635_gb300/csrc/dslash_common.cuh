@@ -200,4 +200,36 @@ __device__ __forceinline__ void herm6_mv_acc(cpx<R> (&w)[6], const R* m, const c
         }
 }
 
+// out = r - alpha (out + shift p) with the residual and search direction of site i, a
+// vector of reals at a time: the update of CG without a stored A p (alpha is known
+// before the second factor of the operator is applied).  NR reals from `off` of a site's
+// 2 NC.
+template <int P, int NC, int NR = 2 * NC>
+__device__ __forceinline__ void residual_update(cpx<typename PT<P>::R>* out, const OpProb& pr, long i, int off = 0) {
+    using R = typename PT<P>::R;
+    constexpr int W = PT<P>::W;
+    const long vh = pr.g.vh;
+    const R alpha = (R)pr.ctl->alpha, shift = (R)pr.ctl->shift;
+    R* o = reinterpret_cast<R*>(out);
+    R rs = (R)1, ps = (R)1;
+    if constexpr (P == PB16 || P == PF16) {
+        const size_t scale = (size_t)vh * NC * 4;
+        rs = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.r) + scale)[i];
+        ps = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.p) + scale) + i);
+    }
+#pragma unroll
+    for (int v = 0; v < NR / W; ++v) {
+        if (shift != (R)0) {
+            R p[W];
+            load_reals<P, W>(pr.p, vh, i, off + W * v, p);
+#pragma unroll
+            for (int e = 0; e < W; ++e) o[W * v + e] += shift * (ps * p[e]);
+        }
+        R r[W];
+        load_reals<P, W>(pr.r, vh, i, off + W * v, r);
+#pragma unroll
+        for (int e = 0; e < W; ++e) o[W * v + e] = rs * r[e] - alpha * o[W * v + e];
+    }
+}
+
 }  // namespace tmk

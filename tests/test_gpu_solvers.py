@@ -450,3 +450,26 @@ def test_returned_residual_of_a_mixed_solve_is_the_fp64_one(sloppy, delta):
         assert abs(info.true_rel_res - res) <= 1e-2 * res
     finally:
         lat.close()
+
+
+def test_heavy_fp64_cg_with_the_flavours_over_thread_pairs():
+    """6,000 sites per parity (a ragged last block), above the small-lattice line of the
+    two-flavour FP64 passes: plain FP64 CG and FP64 multishift reach the tolerance."""
+    import torch
+    from paper_2212_06635_gb300 import tm
+    dims = (12, 10, 10, 10)
+    lat = Lat(F.gauge_field(dims, 93), dims, 0.1394, CSW, mubar=0.1246, epsbar=0.1350)
+    try:
+        host = F.odd_spinor(dims, 94, 2)
+        b = to_dev(host)
+        xs = [torch.zeros_like(b) for _ in range(4)]
+        sp = tm.solve_params(tol=1e-12)
+        infos = [tm.tm_solve_cg(lat.ctx, tm.TM_QH_SQ, sp, xs[0], b)]
+        shifts = [0.01, 0.1, 1.0]
+        infos += tm.tm_solve_multishift(lat.ctx, tm.TM_QH_SQ, shifts, xs[1:], b, sp)
+        for i, s, x in zip(infos, [0.0] + shifts, xs):
+            v = from_dev(x, host.shape)
+            r = host - lat.apply(tm.TM_QH_SQ, 0, v) - s * v
+            assert i.status == 0 and np.linalg.norm(r) <= 1.05e-12 * np.linalg.norm(host), s
+    finally:
+        lat.close()
