@@ -59,72 +59,99 @@ inline cudaError_t launch_chained(void (*kernel)(Params...), int grid, int block
 }
 
 // ---------------------------------------------------------------------------
-// solver scalar finalisers (run by one thread of the last block of a reduction)
+// solver scalar finalisers (run by the first warp of the last block of a reduction)
 // ---------------------------------------------------------------------------
-__device__ inline void ms_alpha(MsCtl* ms, double alpha) {
-    // zeta recurrences of multishift CG for the shifts still active
-    for (int k = 0; k < ms->nshift; ++k) {
-        if (ms->active[k] != 1) { ms->active[k] = 0; ms->alpha_s[k] = 0.0; continue; }
-        const double z = ms->zeta[k], zo = ms->zeta_old[k];
-        const double den = alpha * ms->beta_old * (zo - z) + zo * ms->alpha_old * (1.0 + ms->dshift[k] * alpha);
-        const double zn = z * zo * ms->alpha_old / den;
-        ms->alpha_s[k] = alpha * zn / z;
-        ms->beta_s[k] = zn / z;            // ratio kept until beta is known
-        ms->zeta_old[k] = z;
-        ms->zeta[k] = zn;
+// Zeta recurrences of multishift CG for the shifts still active, a lane each: one after
+// another their FP64 divisions held the solver's chain up (multishift solves with
+// refinement, 10 shifts at 8^2x12x16 19.7 -> 18.4 ms, 12 at 24^3x48 553.4 -> 551.1 ms).
+__device__ inline void ms_alpha(MsCtl* ms, double alpha, int k) {
+    const double alpha_old = ms->alpha_old, beta_old = ms->beta_old;
+    if (k < ms->nshift) {
+        if (ms->active[k] != 1) {
+            ms->active[k] = 0;
+            ms->alpha_s[k] = 0.0;
+        } else {
+            const double z = ms->zeta[k], zo = ms->zeta_old[k];
+            const double den = alpha * beta_old * (zo - z) + zo * alpha_old * (1.0 + ms->dshift[k] * alpha);
+            const double zn = z * zo * alpha_old / den;
+            ms->alpha_s[k] = alpha * zn / z;
+            ms->beta_s[k] = zn / z;            // ratio kept until beta is known
+            ms->zeta_old[k] = z;
+            ms->zeta[k] = zn;
+        }
     }
-    ms->alpha_old = alpha;
+    __syncwarp();
+    if (k == 0) ms->alpha_old = alpha;
+}
+
+// After an iteration with ||r||^2 = t: directions and rings of the shifts (a lane each),
+// and the end of the solve once all have converged.
+__device__ inline void ms_update(SolverCtl* ctl, MsCtl* ms, double t, double beta, int slot, int k) {
+    bool running = false;
+    if (k < ms->nshift) {
+        ms->alpha_ring[slot][k] = ms->active[k] ? ms->alpha_s[k] : 0.0;
+        if (ms->active[k]) {
+            const double ratio = ms->beta_s[k];
+            ms->beta_s[k] = beta * ratio * ratio;
+            ms->beta_ring[slot][k] = ms->beta_s[k];
+            ms->zeta_ring[slot][k] = ms->zeta[k];
+            // shifted residual r_k = zeta_k r
+            running = !(ms->zeta[k] * ms->zeta[k] * t < ms->stop_rr);
+            if (!running) ms->active[k] = 2;   // converged, last update pending
+        }
+    }
+    const int na = __popc(__ballot_sync(0xffffffffu, running));
+    if (k == 0) {
+        ms->beta_old = beta;
+        ms->n_active = na;
+        if (na == 0 && ctl->flag == CTL_RUN) ctl->flag = CTL_STOP;
+    }
 }
 
 __device__ inline void finalize_scalar(int fin, double t, SolverCtl* ctl, MsCtl* ms, double* dst) {
+    const int lane = threadIdx.x;
     switch (fin) {
         case FIN_STORE:
-            if (dst) *dst = t; else ctl->result = t;
+            if (lane == 0) {
+                if (dst) *dst = t; else ctl->result = t;
+            }
             break;
         case FIN_PP:
-            ctl->result = t;   // ||p||^2 for shifted systems
+            if (lane == 0) ctl->result = t;   // ||p||^2 for shifted systems
             break;
         case FIN_CG_ALPHA:
         case FIN_MS_ALPHA: {
             const double pAp = t + ctl->shift * ctl->result;
-            ctl->pAp = pAp;
-            if (!(pAp > 0.0) || !isfinite(pAp)) {
-                ctl->flag = CTL_BREAKDOWN;
-            } else {
-                ctl->alpha = ctl->rr / pAp;
-                ctl->alpha_ring[ctl->slot] = ctl->alpha;
-                if (fin == FIN_MS_ALPHA) ms_alpha(ms, ctl->alpha);
+            const bool good = pAp > 0.0 && isfinite(pAp);
+            const double alpha = good ? ctl->rr / pAp : 0.0;
+            if (lane == 0) {
+                ctl->pAp = pAp;
+                if (good) {
+                    ctl->alpha = alpha;
+                    ctl->alpha_ring[ctl->slot] = alpha;
+                } else {
+                    ctl->flag = CTL_BREAKDOWN;
+                }
             }
+            if (good && fin == FIN_MS_ALPHA) ms_alpha(ms, alpha, lane);
             break;
         }
         case FIN_CG_UPDATE:
         case FIN_MS_UPDATE: {
-            ctl->rr_old = ctl->rr;
-            ctl->rr = t;
-            ctl->beta = t / ctl->rr_old;
+            const double beta = t / ctl->rr;
             const int slot = ctl->slot;
-            ctl->slot = slot + 1 < ctl->ring ? slot + 1 : 0;
-            ctl->iter += 1;
-            if (!isfinite(t)) ctl->flag = CTL_BREAKDOWN;
-            else if (t < ctl->stop_rr) ctl->flag = CTL_STOP;
-            else if (ctl->iter >= ctl->maxiter) ctl->flag = CTL_MAXITER;
-            if (fin == FIN_MS_UPDATE) {
-                int na = 0;
-                for (int k = 0; k < ms->nshift; ++k) {
-                    ms->alpha_ring[slot][k] = ms->active[k] ? ms->alpha_s[k] : 0.0;
-                    if (!ms->active[k]) continue;
-                    const double ratio = ms->beta_s[k];
-                    ms->beta_s[k] = ctl->beta * ratio * ratio;
-                    ms->beta_ring[slot][k] = ms->beta_s[k];
-                    ms->zeta_ring[slot][k] = ms->zeta[k];
-                    // shifted residual r_k = zeta_k r
-                    if (ms->zeta[k] * ms->zeta[k] * t < ms->stop_rr) ms->active[k] = 2;  // converged, last update pending
-                    else ++na;
-                }
-                ms->beta_old = ctl->beta;
-                ms->n_active = na;
-                if (na == 0 && ctl->flag == CTL_RUN) ctl->flag = CTL_STOP;
+            __syncwarp();
+            if (lane == 0) {
+                ctl->rr_old = ctl->rr;
+                ctl->rr = t;
+                ctl->beta = beta;
+                ctl->slot = slot + 1 < ctl->ring ? slot + 1 : 0;
+                ctl->iter += 1;
+                if (!isfinite(t)) ctl->flag = CTL_BREAKDOWN;
+                else if (t < ctl->stop_rr) ctl->flag = CTL_STOP;
+                else if (ctl->iter >= ctl->maxiter) ctl->flag = CTL_MAXITER;
             }
+            if (fin == FIN_MS_UPDATE) ms_update(ctl, ms, t, beta, slot, lane);
             break;
         }
         default:
@@ -168,10 +195,8 @@ __device__ __forceinline__ void reduce_finalize(double* partial, unsigned int* c
     double t = 0.0;
     for (int k = threadIdx.x; k < nblk; k += BS) t += ((volatile double*)partial)[k];
     t = block_sum<BS>(t, sh);
-    if (threadIdx.x == 0) {
-        *counter = 0u;
-        finalize_scalar(fin, t, ctl, ms, dst);
-    }
+    if (threadIdx.x == 0) *counter = 0u;
+    if (threadIdx.x < 32) finalize_scalar(fin, t, ctl, ms, dst);
 }
 
 // ---------------------------------------------------------------------------
