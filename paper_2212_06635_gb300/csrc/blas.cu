@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(BLAS_BS) k_convert(const __grid_constant__ Vec
     if (!valid) return;
     cpx<RS> s[NC];
     cpx<RD> d[NC];
-    load_spinor<PS, NC>(pr.v[1], pr.vh, i, s);
+    load_spinor<PS, NC, true>(pr.v[1], pr.vh, i, s);
 #pragma unroll
     for (int q = 0; q < NC; ++q) d[q] = C((RD)s[q].re, (RD)s[q].im);
     store_spinor<PD, NC>(pr.v[0], pr.vh, i, d);
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(BLAS_BS) k_add_to64(const __grid_constant__ Ve
     if (!valid) return;
     cpx<RS> x[NC];
     cpx<double> y[NC];
-    load_spinor<PS, NC>(pr.v[1], pr.vh, i, x);
+    load_spinor<PS, NC, true>(pr.v[1], pr.vh, i, x);
     load_spinor<P64, NC>(pr.v[0], pr.vh, i, y);
 #pragma unroll
     for (int q = 0; q < NC; ++q) y[q] = y[q] + C((double)x[q].re, (double)x[q].im);
@@ -124,9 +124,9 @@ __global__ void __launch_bounds__(BLAS_BS) k_residual64(const __grid_constant__ 
     double s = 0.0;
     if (valid) {
         cpx<double> r[NC], bb[NC], ax[NC], x[NC];
-        load_spinor<P64, NC>(pr.v[1], pr.vh, i, bb);
-        load_spinor<P64, NC>(pr.v[2], pr.vh, i, ax);
-        if (shv != 0.0) load_spinor<P64, NC>(pr.v[3], pr.vh, i, x);
+        load_spinor<P64, NC, true>(pr.v[1], pr.vh, i, bb);
+        load_spinor<P64, NC, true>(pr.v[2], pr.vh, i, ax);
+        if (shv != 0.0) load_spinor<P64, NC, true>(pr.v[3], pr.vh, i, x);
 #pragma unroll
         for (int q = 0; q < NC; ++q) {
             r[q] = bb[q] - ax[q];
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(BLAS_BS) k_norm2(const __grid_constant__ VecBa
     double s = 0.0;
     if (valid) {
         cpx<R> v[NC];
-        load_spinor<P, NC>(pr.v[0], pr.vh, i, v);
+        load_spinor<P, NC, true>(pr.v[0], pr.vh, i, v);
         if constexpr (P == P64) {
 #pragma unroll
             for (int q = 0; q < NC; ++q) s += norm2(v[q]);
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(BLAS_BS) k_cg_xupdate(const __grid_constant__ 
     for (int k = 0; k < RING; ++k) {
         if (k < n) {
             R p[W];
-            load_reals<P, W>(pr.v[2 + k], vh, i, W * v, p);
+            load_readonly<P, W>(pr.v[2 + k], vh, i, W * v, p);
 #pragma unroll
             for (int e = 0; e < W; ++e) x[e] += (RX)(alpha[k] * p[e]);
         }
@@ -298,33 +298,44 @@ __global__ void __launch_bounds__(BLAS_BS) k_ms_block(const __grid_constant__ Ve
     if constexpr (!H) {
 #pragma unroll
         for (int q = 0; q < RING; ++q)
-            if (q < n) load_reals<P, W>(pr.v[2 + q], vh, i, off, r[q]);
+            if (q < n) load_readonly<P, W>(pr.v[2 + q], vh, i, off, r[q]);
     }
+    // shifts a thread has in flight: all loads of a step before its stores
+    constexpr int G = H ? 1 : 2;
     const int nl = nlive;
-#pragma unroll (H ? 1 : 2)
-    for (int l = 0; l < nl; ++l) {
-        const int k = live[l];
-        R p[W];
-        RX x[W];
-        if constexpr (H) load_spinor<P, NC>(mv.p[k], vh, i, reinterpret_cast<cpx<R>*>(p));
-        else load_reals<P, W>(mv.p[k], vh, i, off, p);
-        load_reals<PX, W>(mv.x[k], vh, i, off, x);
+#pragma unroll 1
+    for (int l = 0; l < nl; l += G) {
+        R p[G][W];
+        RX x[G][W];
 #pragma unroll
-        for (int q = 0; q < RING; ++q) {
-            if (q < n) {
-                const R a = coef[k][q][0], z = coef[k][q][1], bt = coef[k][q][2];
-                if constexpr (H) load_spinor<P, NC>(pr.v[2 + q], vh, i, reinterpret_cast<cpx<R>*>(r[0]));
-                const R* rq = r[H ? 0 : q];
+        for (int g = 0; g < G; ++g) {
+            if (l + g >= nl) continue;
+            const int k = live[l + g];
+            if constexpr (H) load_spinor<P, NC>(mv.p[k], vh, i, reinterpret_cast<cpx<R>*>(p[g]));
+            else load_reals<P, W>(mv.p[k], vh, i, off, p[g]);
+            load_reals<PX, W>(mv.x[k], vh, i, off, x[g]);
+        }
 #pragma unroll
-                for (int e = 0; e < W; ++e) {
-                    x[e] += (RX)(a * p[e]);
-                    p[e] = z * rq[e] + bt * p[e];
+        for (int g = 0; g < G; ++g) {
+            if (l + g >= nl) continue;
+            const int k = live[l + g];
+#pragma unroll
+            for (int q = 0; q < RING; ++q) {
+                if (q < n) {
+                    const R a = coef[k][q][0], z = coef[k][q][1], bt = coef[k][q][2];
+                    if constexpr (H) load_spinor<P, NC, true>(pr.v[2 + q], vh, i, reinterpret_cast<cpx<R>*>(r[0]));
+                    const R* rq = r[H ? 0 : q];
+#pragma unroll
+                    for (int e = 0; e < W; ++e) {
+                        x[g][e] += (RX)(a * p[g][e]);
+                        p[g][e] = z * rq[e] + bt * p[g][e];
+                    }
                 }
             }
+            store_reals<PX, W>(mv.x[k], vh, i, off, x[g]);
+            if constexpr (H) store_spinor<P, NC>(mv.p[k], vh, i, reinterpret_cast<const cpx<R>*>(p[g]));
+            else store_reals<P, W>(mv.p[k], vh, i, off, p[g]);
         }
-        store_reals<PX, W>(mv.x[k], vh, i, off, x);
-        if constexpr (H) store_spinor<P, NC>(mv.p[k], vh, i, reinterpret_cast<const cpx<R>*>(p));
-        else store_reals<P, W>(mv.p[k], vh, i, off, p);
     }
 }
 
@@ -352,7 +363,7 @@ __global__ void __launch_bounds__(BLAS_BS) k_export(double* dst, const void* src
     const long i = (long)blockIdx.x * BLAS_BS + threadIdx.x;
     if (i >= vh) return;
     cpx<R> s[NC];
-    load_spinor<P, NC>(src, vh, i, s);
+    load_spinor<P, NC, true>(src, vh, i, s);
     double2* p = reinterpret_cast<double2*>(dst) + i * NC;
 #pragma unroll
     for (int q = 0; q < NC; ++q) p[q] = make_double2((double)s[q].re, (double)s[q].im);

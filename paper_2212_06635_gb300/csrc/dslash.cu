@@ -97,7 +97,7 @@ __device__ __forceinline__ void inverse_blocks(cpx<typename PT<P>::R>* out, cons
 #pragma unroll
         for (int rr = 0; rr < 3; ++rr) {
             R m[24];
-            load_reals<P, 24>(pr.clov, pr.g.vh, i, 72 * cb + 24 * rr, m);
+            load_readonly<P, 24>(pr.clov, pr.g.vh, i, 72 * cb + 24 * rr, m);
 #pragma unroll
             for (int r2 = 0; r2 < 2; ++r2) {
                 const int r = 2 * rr + r2;
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(BS, (dslash_min_blocks<P, NF, KIND>())) dslash
             cpx<R> psi[NF * 12];
             load_spinor<P, NF * 12>(pr.loc, pr.g.vh, i, psi);
             R m[72];
-            load_reals<P, 72>(pr.clov, pr.g.vh, i, 0, m);
+            load_readonly<P, 72>(pr.clov, pr.g.vh, i, 0, m);
             const R k2 = (R)(pr.kappa * pr.kappa);
             // W_hat = Q_hat + i rho (eq:hWpm): i rho psi = g5 (i rho g5 psi) joins the twist
             const R tw = (R)pr.tw, rho = (R)pr.rho;

@@ -215,7 +215,7 @@ __device__ __forceinline__ void residual_update(cpx<typename PT<P>::R>* out, con
     if constexpr (P == PB16 || P == PF16) {
         const size_t scale = (size_t)vh * NC * 4;
         rs = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.r) + scale)[i];
-        ps = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.p) + scale) + i);
+        ps = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.p) + scale)[i];
     }
 #pragma unroll
     for (int v = 0; v < NR / W; ++v) {

@@ -37,7 +37,7 @@ __device__ __forceinline__ void load_flavour_unscaled(const void* base, long vh,
     sc = 1.f;
     if constexpr (P == PB16 || P == PF16) {
         const float* nrm = reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + (size_t)vh * 24 * 2 * 2);
-        sc = __ldg(nrm + i);
+        sc = nrm[i];
     }
 }
 
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, KIND>())) dslash_heav
                 }
                 {   // D_c - 1: 40 reals from 72 cb + 32 (aligned for every storage width), at offset 4
                     R m[40];
-                    load_reals<P, 40>(pr.clov, pr.g.vh, i, 72 * cb + 32, m);
+                    load_readonly<P, 40>(pr.clov, pr.g.vh, i, 72 * cb + 32, m);
                     herm6_mv_acc<R>(dv, m + 4, v);
                 }
 #pragma unroll
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, KIND>())) dslash_heav
                 }
                 {   // A_c - 1: 40 reals from 72 cb, at offset 0
                     R m[40];
-                    load_reals<P, 40>(pr.clov, pr.g.vh, i, 72 * cb, m);
+                    load_readonly<P, 40>(pr.clov, pr.g.vh, i, 72 * cb, m);
                     herm6_mv_acc<R>(w, m, dv);
                 }
                 const R t = tf * (cb == 0 ? tw : -tw);
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, K1_EO_INV>())) dslash
                 w[j] = w[j] - k2 * acc[2 * cb + j / 3][j % 3];
             }
             R m[40];   // 36 reals of the block, from a place aligned for every storage width
-            load_reals<P, 40>(pr.clov, pr.g.vh, i, 32 * cb, m);
+            load_readonly<P, 40>(pr.clov, pr.g.vh, i, 32 * cb, m);
             herm6_mv_acc<R>(w, m + 4 * cb, v);
 #pragma unroll
             for (int j = 0; j < 6; ++j) out[6 * cb + j] = (cb == 0) ? w[j] : -w[j];

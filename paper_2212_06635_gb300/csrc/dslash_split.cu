@@ -23,28 +23,28 @@
 
 namespace tmk {
 
-// complex number e (reals 2e, 2e + 1) and real r of a site's native array
-template <int P>
+// complex number e (reals 2e, 2e + 1) and real r of a site's native array (RO: load_vec)
+template <int P, bool RO>
 __device__ __forceinline__ cpx<typename PT<P>::R> load_complex(const void* base, long vh, long i, int e) {
     if constexpr (P == P64) {
-        const double2 q = __ldg(reinterpret_cast<const double2*>(base) + (long)e * vh + i);
+        const double2 q = load_vec<RO>(reinterpret_cast<const double2*>(base) + (long)e * vh + i);
         return C(q.x, q.y);
     } else if constexpr (P == P32) {
-        const float2 q = __ldg(reinterpret_cast<const float2*>(base) + ((long)(e >> 1) * vh + i) * 2 + (e & 1));
+        const float2 q = load_vec<RO>(reinterpret_cast<const float2*>(base) + ((long)(e >> 1) * vh + i) * 2 + (e & 1));
         return C(q.x, q.y);
     } else {
         const float2 q =
-            h2f2<P>(__ldg(reinterpret_cast<const unsigned int*>(base) + ((long)(e >> 2) * vh + i) * 4 + (e & 3)));
+            h2f2<P>(load_vec<RO>(reinterpret_cast<const unsigned int*>(base) + ((long)(e >> 2) * vh + i) * 4 + (e & 3)));
         return C(q.x, q.y);
     }
 }
-template <int P>
+template <int P, bool RO>
 __device__ __forceinline__ typename PT<P>::R load_real(const void* base, long vh, long i, int r) {
     constexpr int W = PT<P>::W;
     const long e = ((long)(r / W) * vh + i) * W + r % W;
-    if constexpr (P == P64) return __ldg(reinterpret_cast<const double*>(base) + e);
-    else if constexpr (P == P32) return __ldg(reinterpret_cast<const float*>(base) + e);
-    else return h2f<P>(__ldg(reinterpret_cast<const uint16_t*>(base) + e));
+    if constexpr (P == P64) return load_vec<RO>(reinterpret_cast<const double*>(base) + e);
+    else if constexpr (P == P32) return load_vec<RO>(reinterpret_cast<const float*>(base) + e);
+    else return h2f<P>(load_vec<RO>(reinterpret_cast<const uint16_t*>(base) + e));
 }
 template <int P>
 __device__ __forceinline__ void store_complex(void* base, long vh, long i, int e, cpx<typename PT<P>::R> z) {
@@ -54,7 +54,7 @@ __device__ __forceinline__ void store_complex(void* base, long vh, long i, int e
     else reinterpret_cast<unsigned int*>(base)[((long)(e >> 2) * vh + i) * 4 + (e & 3)] = f2h2<P>(z.re, z.im);
 }
 
-// entries (r, j), j = 0 .. 5, of a packed hermitian block at real offset off
+// entries (r, j), j = 0 .. 5, of a packed hermitian block (clover data) at real offset off
 template <int P>
 __device__ __forceinline__ void load_herm_row(cpx<typename PT<P>::R> (&m)[6], const void* base, long vh, long i, int off,
                                               int r) {
@@ -62,9 +62,9 @@ __device__ __forceinline__ void load_herm_row(cpx<typename PT<P>::R> (&m)[6], co
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
         const int hi = r > j ? r : j, lo = r > j ? j : r;
-        if (r == j) m[j] = C(load_real<P>(base, vh, i, off + r), (R)0);
+        if (r == j) m[j] = C(load_real<P, true>(base, vh, i, off + r), (R)0);
         else {
-            m[j] = load_complex<P>(base, vh, i, (off + 6) / 2 + hi * (hi - 1) / 2 + lo);
+            m[j] = load_complex<P, true>(base, vh, i, (off + 6) / 2 + hi * (hi - 1) / 2 + lo);
             if (r < j) m[j].im = -m[j].im;
         }
     }
@@ -92,8 +92,8 @@ __device__ __forceinline__ void split_hops(cpx<typename PT<P>::R> (&acc)[4][3], 
     load_reals<P, 24>(pr.in, g.vh, nb, 24 * f, reinterpret_cast<R*>(pb));
     if constexpr (SC) {
         const float* scale = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.in) + (size_t)g.vh * NF * 12 * 4);
-        ff *= __ldg(scale + nf);
-        fb *= __ldg(scale + nb);
+        ff *= scale[nf];
+        fb *= scale[nb];
     }
     cpx<R> g0[3], g1[3];
     hop_forward<R, MU, SC>(g0, g1, pf, uf, ff);
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(128 * NF) dslash_split_kernel(const __grid_con
 #pragma unroll
                 for (int j = 0; j < 6; ++j) {   // B, or the conjugate of its transpose
                     const int r = 3 * h + c;
-                    m[c][j] = load_complex<P>(pr.clov, vh, i, 36 * cb + (pr.sign > 0 ? 6 * r + j : 6 * j + r));
+                    m[c][j] = load_complex<P, true>(pr.clov, vh, i, 36 * cb + (pr.sign > 0 ? 6 * r + j : 6 * j + r));
                     if (pr.sign < 0) m[c][j].im = -m[c][j].im;
                 }
         } else {
@@ -219,9 +219,9 @@ __global__ void __launch_bounds__(128 * NF) dslash_split_kernel(const __grid_con
         if (valid) {
             R sc = (R)1;
             if constexpr (P == PF16 || P == PB16)
-                sc = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.loc) + (size_t)vh * NF * 12 * 4) + i);
+                sc = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.loc) + (size_t)vh * NF * 12 * 4)[i];
 #pragma unroll
-            for (int j = 0; j < 6; ++j) v[j] = sc * load_complex<P>(pr.loc, vh, i, 12 * f + 6 * cb + j);
+            for (int j = 0; j < 6; ++j) v[j] = sc * load_complex<P, false>(pr.loc, vh, i, 12 * f + 6 * cb + j);
             const R g5 = cb == 0 ? (R)1 : (R)-1, t3 = f == 0 ? (R)1 : (R)-1;
             const R tw = g5 * ((R)pr.tw * t3 + (R)pr.rho), k2 = (R)(pr.kappa * pr.kappa);
 #pragma unroll
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(128 * NF) dslash_split_kernel(const __grid_con
                 const cpx<R> p = h == 0 ? v[c] : v[3 + c];
                 cpx<R> s = tw * mul_i(p);
                 if constexpr (NF == 2)
-                    s = s - (R)pr.eps * (sc * load_complex<P>(pr.loc, vh, i, 12 * (1 - f) + 6 * cb + 3 * h + c));
+                    s = s - (R)pr.eps * (sc * load_complex<P, false>(pr.loc, vh, i, 12 * (1 - f) + 6 * cb + 3 * h + c));
                 s = s - k2 * hops(6 * cb + 3 * h + c);
 #pragma unroll
                 for (int j = 0; j < 6; ++j) cfma(s, m[c][j], v[j]);
@@ -241,13 +241,13 @@ __global__ void __launch_bounds__(128 * NF) dslash_split_kernel(const __grid_con
                 if constexpr (P == PF16 || P == PB16) {
                     const size_t off = (size_t)vh * NF * 12 * 4;
                     rs = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.r) + off)[i];
-                    ps = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.p) + off) + i);
+                    ps = reinterpret_cast<const float*>(reinterpret_cast<const char*>(pr.p) + off)[i];
                 }
                 const int e = 12 * f + 6 * cb + 3 * h;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    if (shift != (R)0) out[c] = out[c] + shift * (ps * load_complex<P>(pr.p, vh, i, e + c));
-                    out[c] = rs * load_complex<P>(pr.r, vh, i, e + c) - alpha * out[c];
+                    if (shift != (R)0) out[c] = out[c] + shift * (ps * load_complex<P, false>(pr.p, vh, i, e + c));
+                    out[c] = rs * load_complex<P, false>(pr.r, vh, i, e + c) - alpha * out[c];
                 }
             }
         }

@@ -83,7 +83,7 @@ __device__ __forceinline__ void force_half(cpx<float> (&h)[2][3], const cpx<floa
 // scale for 16-bit storage (1 for FP32)
 template <int P, int NF>
 __device__ __forceinline__ void force_load(const void* base, long vh, long i, int f, cpx<float>* p, float& sc) {
-    load_reals<P, 24>(base, vh, i, 24 * f, reinterpret_cast<float*>(p));
+    load_readonly<P, 24>(base, vh, i, 24 * f, reinterpret_cast<float*>(p));
     sc = 1.f;
     if constexpr (P == PB16 || P == PF16) {
         const float* nrm = reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) +

@@ -510,7 +510,7 @@ __device__ __forceinline__ void full_op_site(const FullOp& a, long gi, double (&
     cpx<R> psi[12];
     load_spinor<P, 12>(reinterpret_cast<const char*>(a.in) + (size_t)po * a.half, a.g.vh, i, psi);
     R m[72];
-    load_reals<P, 72>(a.A[po], a.g.vh, i, 0, m);
+    load_readonly<P, 72>(a.A[po], a.g.vh, i, 0, m);
     const R kap = (R)a.kappa, tw = (R)a.tw;
     cpx<R> out[12];
 #pragma unroll
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(MG_BS) k_mg_build(const __grid_constant__ Buil
                 cpx<R> v[12];
                 col_at<P>(b, cs, x, v);
                 R mm[72];
-                load_reals<P, 72>(b.A[px], m.g.vh, ix, 0, mm);
+                load_readonly<P, 72>(b.A[px], m.g.vh, ix, 0, mm);
                 cpx<R> lv[6], ww[6];
                 const R sc = hs == 0 ? (R)1 : (R)-1;
 #pragma unroll

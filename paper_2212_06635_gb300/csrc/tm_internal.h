@@ -116,8 +116,20 @@ template <> __device__ __forceinline__ uint32_t f2h2<PB16>(float lo, float hi) {
     return w;
 }
 
+// One vector, through the read-only path (RO) or coherently.  The read-only path needs
+// data that nobody writes while the kernel exists, and the compiler may move its loads
+// across any wait.  A chained kernel (launch_chained) exists while the kernel before it
+// still writes its fields, so it reads spinors and their scales coherently and only links
+// and clover blocks, which no kernel of a chain writes, through it; the same holds for
+// what a kernel updates in place.
+template <bool RO, typename T>
+__device__ __forceinline__ T load_vec(const T* p) {
+    if constexpr (RO) return __ldg(p);
+    else return *p;
+}
+
 // Load NR reals (NR multiple of W) starting at real offset OFF of site i.
-template <int P, int NR>
+template <int P, int NR, bool RO = false>
 __device__ __forceinline__ void load_reals(const void* base, long vh, long i, int off,
                                            typename PT<P>::R* dst) {
     constexpr int W = PT<P>::W;
@@ -126,16 +138,16 @@ __device__ __forceinline__ void load_reals(const void* base, long vh, long i, in
     for (int v = 0; v < NR / W; ++v) {
         const long e = (long)(v0 + v) * vh + i;
         if constexpr (P == P64) {
-            double2 q = __ldg(reinterpret_cast<const double2*>(base) + e);
+            double2 q = load_vec<RO>(reinterpret_cast<const double2*>(base) + e);
             dst[2 * v] = q.x; dst[2 * v + 1] = q.y;
         } else if constexpr (P == PDF) {
-            float4 q = __ldg(reinterpret_cast<const float4*>(base) + e);
+            float4 q = load_vec<RO>(reinterpret_cast<const float4*>(base) + e);
             dst[2 * v] = df(q.x, q.y); dst[2 * v + 1] = df(q.z, q.w);
         } else if constexpr (P == P32) {
-            float4 q = __ldg(reinterpret_cast<const float4*>(base) + e);
+            float4 q = load_vec<RO>(reinterpret_cast<const float4*>(base) + e);
             dst[4 * v] = q.x; dst[4 * v + 1] = q.y; dst[4 * v + 2] = q.z; dst[4 * v + 3] = q.w;
         } else {
-            uint4 q = __ldg(reinterpret_cast<const uint4*>(base) + e);
+            uint4 q = load_vec<RO>(reinterpret_cast<const uint4*>(base) + e);
             const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -145,6 +157,12 @@ __device__ __forceinline__ void load_reals(const void* base, long vh, long i, in
             }
         }
     }
+}
+
+// the same for data that no kernel running at the same time writes
+template <int P, int NR>
+__device__ __forceinline__ void load_readonly(const void* base, long vh, long i, int off, typename PT<P>::R* dst) {
+    load_reals<P, NR, true>(base, vh, i, off, dst);
 }
 
 template <int P, int NR>
@@ -172,16 +190,16 @@ __device__ __forceinline__ void store_reals(void* base, long vh, long i, int off
     }
 }
 
-// Spinor of NC complex components at site i.
-template <int P, int NC>
+// Spinor of NC complex components at site i (RO: load_vec).
+template <int P, int NC, bool RO = false>
 __device__ __forceinline__ void load_spinor(const void* base, long vh, long i,
                                             cpx<typename PT<P>::R>* s) {
     using R = typename PT<P>::R;
-    load_reals<P, 2 * NC>(base, vh, i, 0, reinterpret_cast<R*>(s));
+    load_reals<P, 2 * NC, RO>(base, vh, i, 0, reinterpret_cast<R*>(s));
     if constexpr (P == PB16 || P == PF16) {
         const float* nrm = reinterpret_cast<const float*>(
             reinterpret_cast<const char*>(base) + (size_t)vh * NC * 2 * 2);
-        const float sc = __ldg(nrm + i);
+        const float sc = load_vec<RO>(nrm + i);
 #pragma unroll
         for (int k = 0; k < NC; ++k) { s[k].re *= sc; s[k].im *= sc; }
     }
@@ -198,7 +216,7 @@ __device__ __forceinline__ void load_spinor_unscaled(const void* base, long vh, 
     if constexpr (P == PB16 || P == PF16) {
         const float* nrm = reinterpret_cast<const float*>(
             reinterpret_cast<const char*>(base) + (size_t)vh * NC * 2 * 2);
-        sc = __ldg(nrm + i);
+        sc = nrm[i];
     }
 }
 
@@ -239,6 +257,7 @@ __device__ __forceinline__ void su3_third_row(cpx<R>* u) {
 
 // SU(3) link (9 complex, row major) of direction mu at site i of one parity;
 // element k of direction mu lives at (mu * LinkStore<P>::N + k) * vh + i.
+// (Read-only path: links change between calls only.)
 template <int P>
 __device__ __forceinline__ void load_link(const void* base, long vh, int mu, long i,
                                           cpx<typename PT<P>::R>* u) {
@@ -247,16 +266,16 @@ __device__ __forceinline__ void load_link(const void* base, long vh, int mu, lon
     for (int k = 0; k < N; ++k) {
         const long e = (long)(mu * N + k) * vh + i;
         if constexpr (P == P64) {
-            double2 q = __ldg(reinterpret_cast<const double2*>(base) + e);
+            double2 q = load_vec<true>(reinterpret_cast<const double2*>(base) + e);
             u[k] = C(q.x, q.y);
         } else if constexpr (P == PDF) {
-            float4 q = __ldg(reinterpret_cast<const float4*>(base) + e);
+            float4 q = load_vec<true>(reinterpret_cast<const float4*>(base) + e);
             u[k] = C(df(q.x, q.y), df(q.z, q.w));
         } else if constexpr (P == P32) {
-            float2 q = __ldg(reinterpret_cast<const float2*>(base) + e);
+            float2 q = load_vec<true>(reinterpret_cast<const float2*>(base) + e);
             u[k] = C(q.x, q.y);
         } else {
-            uint32_t q = __ldg(reinterpret_cast<const unsigned int*>(base) + e);
+            uint32_t q = load_vec<true>(reinterpret_cast<const unsigned int*>(base) + e);
             const float2 f = h2f2<P>(q);
             u[k] = C(f.x, f.y);
         }
