@@ -222,7 +222,13 @@ tm_status tm_solve_cg(tm_ctx* ctx, tm_op op, const tm_solve_params* sp, double* 
 /* Solve (A + shifts[k]) x[k] = b for nshift shifts (A = TM_MDAGM or TM_QH_SQ) with
  * one multishift CG in the sloppy precision (Sec. 4.2), then refine each shift
  * by mixed-precision CG to sp->tol ("shift-by-shift refinement").  x[k] canonical
- * FP64 output buffers (host or device); infos has nshift records. */
+ * FP64 output buffers (host or device); infos has nshift records.
+ * Shifts are refined several at a time in the fields the multishift solve has left; on
+ * lattices of up to 32768 sites per parity that takes further fields of the refinement's
+ * precision (8 a shift after the first, less the 2 nshift there are: about 0.5 GB for 16
+ * shifts of a two-flavour FP32 solve at 32768).  They are kept like all workspace until
+ * tm_destroy, taken only if everything else fits, and given back when an allocation for
+ * this context fails (likewise the 3 further directions that a CG solve keeps). */
 tm_status tm_solve_multishift(tm_ctx* ctx, tm_op op, int nshift, const double* shifts,
                               double** x, const double* b, const tm_solve_params* sp,
                               tm_solve_info* infos, void* stream);

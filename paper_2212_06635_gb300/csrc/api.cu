@@ -116,23 +116,7 @@ static tm_status io_slot(tm_ctx::IoRing& r, size_t bytes, cudaStream_t st, int* 
     return TM_OK;
 }
 
-static tm_status ws_get(tm_ctx* c, int id, size_t bytes, void** out) {
-    auto it = c->ws.find(id);
-    if (it != c->ws.end() && it->second.second >= bytes) {
-        *out = it->second.first;
-        return TM_OK;
-    }
-    if (it != c->ws.end()) {
-        cudaFree(it->second.first);
-        c->ws.erase(it);
-    }
-    void* p = nullptr;
-    CK(cudaMalloc(&p, bytes));
-    c->ws[id] = {p, bytes};
-    *out = p;
-    return TM_OK;
-}
-
+// workspace ids (multigrid's: mg.cu, 600 .. 799)
 enum WsId {
     WS_B64 = 1, WS_X64, WS_R64, WS_AX64, WS_TE64, WS_MID64, WS_V64,
     WS_TE_S, WS_MID_S, WS_R_S, WS_P_S, WS_AP_S, WS_X_S,
@@ -140,8 +124,102 @@ enum WsId {
     WS_FCG_Z, WS_XDF,
     WS_RING = 60,   // RING search directions (CG) or residuals (multishift)
     WS_MS_X = 100, WS_MS_P = 200, WS_MS_X64 = 300, WS_RAT = 400,
-    WS_GROUP = 500, WS_GROUP_PARTIAL = 499
+    WS_GROUP_PARTIAL = 999, WS_GROUP = 1000
 };
+
+// Scratch that a call can do without: the ring's fields after the first, and what the
+// further systems of a group take beyond a multishift solve's buffers.  It is taken
+// after everything the call needs (spare_get), kept for the next call, and given back
+// when a needed allocation does not fit, unless the running call works in it.
+static bool is_spare(int id) {
+    return (id > WS_RING && id < WS_RING + RING) || id >= WS_GROUP_PARTIAL;
+}
+
+static void ws_drop(tm_ctx* c, int id) {
+    auto it = c->ws.find(id);
+    if (it == c->ws.end()) return;
+    cudaFree(it->second.first);
+    c->ws_bytes -= it->second.second;
+    c->ws.erase(it);
+}
+
+static bool spare_release(tm_ctx* c) {
+    if (c->spare_busy) return false;
+    std::vector<int> ids;
+    for (auto& kv : c->ws)
+        if (is_spare(kv.first)) ids.push_back(kv.first);
+    if (!ids.empty()) cudaStreamSynchronize(c->sstream);
+    for (int id : ids) ws_drop(c, id);
+    return !ids.empty();
+}
+
+// (an out-of-memory error is returned, not left for the next launch check to find)
+static cudaError_t quiet_malloc(void** p, size_t bytes) {
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
+// device memory of the context outside the workspace
+template <typename T>
+static cudaError_t dev_alloc(tm_ctx* c, T** p, size_t bytes) {
+    cudaError_t e = quiet_malloc(reinterpret_cast<void**>(p), bytes);
+    if (e == cudaErrorMemoryAllocation && spare_release(c)) e = quiet_malloc(reinterpret_cast<void**>(p), bytes);
+    return e;
+}
+
+static cudaError_t ws_alloc(tm_ctx* c, int id, size_t bytes) {
+    if (c->ws_limit > 0 && c->ws_bytes + bytes > c->ws_limit) return cudaErrorMemoryAllocation;
+    void* p = nullptr;
+    const cudaError_t e = quiet_malloc(&p, bytes);
+    if (e != cudaSuccess) return e;
+    c->ws[id] = {p, bytes};
+    c->ws_bytes += bytes;
+    return cudaSuccess;
+}
+
+static void* ws_held(tm_ctx* c, int id, size_t bytes) {   // null: not there, or too small
+    auto it = c->ws.find(id);
+    return it != c->ws.end() && it->second.second >= bytes ? it->second.first : nullptr;
+}
+
+static tm_status ws_get(tm_ctx* c, int id, size_t bytes, void** out) {
+    *out = ws_held(c, id, bytes);
+    if (*out) return TM_OK;
+    ws_drop(c, id);
+    cudaError_t e = ws_alloc(c, id, bytes);
+    if (e == cudaErrorMemoryAllocation && spare_release(c)) e = ws_alloc(c, id, bytes);
+    if (e != cudaSuccess)
+        return fail(e == cudaErrorMemoryAllocation ? TM_ERR_OOM : TM_ERR_CUDA, "workspace of %zu bytes: %s", bytes,
+                    cudaGetErrorString(e));
+    *out = c->ws.at(id).first;
+    return TM_OK;
+}
+
+// spare scratch; false where it does not fit
+static bool spare_get(tm_ctx* c, int id, size_t bytes, void** out) {
+    *out = ws_held(c, id, bytes);
+    if (*out) return true;
+    ws_drop(c, id);
+    if (ws_alloc(c, id, bytes) != cudaSuccess) return false;
+    *out = c->ws.at(id).first;
+    return true;
+}
+
+// the time in which a call works in spare scratch
+struct SpareUse {
+    tm_ctx* c;
+    explicit SpareUse(tm_ctx* ctx) : c(ctx) { c->spare_busy = true; }
+    ~SpareUse() { c->spare_busy = false; }
+    SpareUse(const SpareUse&) = delete;
+};
+
+// Host-side bound on a context's workspace in bytes (0: none), as if the device had no
+// more memory; the bytes held are returned.
+extern "C" size_t tmk_scratch_limit(tm_ctx* c, size_t bytes) {
+    c->ws_limit = bytes;
+    return c->ws_bytes;
+}
 
 // ---------------------------------------------------------------------------
 // context
@@ -217,7 +295,7 @@ extern "C" tm_status tm_gauge_load(tm_ctx* c, const double* links, double gauge_
     const cudaStream_t st = S(stream);
     const size_t canon = (size_t)2 * c->vh * 4 * 18 * sizeof(double);
     for (int p = 0; p < 2; ++p)
-        if (!c->gauge64[p]) CK(cudaMalloc(&c->gauge64[p], link_bytes_parity(P64, c->vh)));
+        if (!c->gauge64[p]) CK(dev_alloc(c, &c->gauge64[p], link_bytes_parity(P64, c->vh)));
     const double* src = links;
     if (!is_device_ptr(links)) {
         void* stage = nullptr;
@@ -228,9 +306,7 @@ extern "C" tm_status tm_gauge_load(tm_ctx* c, const double* links, double gauge_
     CK(launch_gauge_import(c->gauge64[0], c->gauge64[1], src, c->g, st));
     if (src != links) {
         CK(cudaStreamSynchronize(st));
-        auto it = c->ws.find(WS_STAGE_G);
-        cudaFree(it->second.first);
-        c->ws.erase(it);
+        ws_drop(c, WS_STAGE_G);
     }
     c->gauge_id = gauge_id;
     c->gauge_gen += 1;   // every derived object is now stale
@@ -263,9 +339,9 @@ extern "C" tm_status tm_clover_compute(tm_ctx* c, const tm_params* prm, void* st
     const long vh = c->vh;
     const bool heavy = prm->mubar != 0.0 || prm->epsbar != 0.0;
     for (int p = 0; p < 2; ++p)
-        if (!c->clovA64[p]) CK(cudaMalloc(&c->clovA64[p], sizeof(double) * CLOV_ODD_REALS * vh));
-    if (!c->clovB64) CK(cudaMalloc(&c->clovB64, sizeof(double) * CLOV_EVEN_LIGHT_REALS * vh));
-    if (heavy && !c->clovH64) CK(cudaMalloc(&c->clovH64, sizeof(double) * CLOV_EVEN_HEAVY_REALS * vh));
+        if (!c->clovA64[p]) CK(dev_alloc(c, &c->clovA64[p], sizeof(double) * CLOV_ODD_REALS * vh));
+    if (!c->clovB64) CK(dev_alloc(c, &c->clovB64, sizeof(double) * CLOV_EVEN_LIGHT_REALS * vh));
+    if (heavy && !c->clovH64) CK(dev_alloc(c, &c->clovH64, sizeof(double) * CLOV_EVEN_HEAVY_REALS * vh));
     const double k = prm->kappa;
     CK(launch_clover(c->g, c->gauge64[0], c->gauge64[1], k, prm->csw, 2 * k * prm->mu, 2 * k * prm->mubar,
                      2 * k * prm->epsbar, c->clovA64[0], c->clovA64[1], c->clovB64, heavy ? c->clovH64 : nullptr, st));
@@ -286,7 +362,7 @@ extern "C" tm_status tm_clover_export(tm_ctx* c, int parity, double* out, void* 
         CK(launch_clover_unpack(out, c->clovA64[parity], c->vh, st));
     } else {
         void* tmp = nullptr;
-        CK(cudaMalloc(&tmp, bytes));
+        CK(dev_alloc(c, &tmp, bytes));
         CK(launch_clover_unpack(reinterpret_cast<double*>(tmp), c->clovA64[parity], c->vh, st));
         CK(cudaMemcpyAsync(out, tmp, bytes, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
@@ -303,7 +379,7 @@ static tm_status ensure_prec(tm_ctx* c, int P, cudaStream_t st) {
     const long vh = c->vh;
     if (c->gaugeP_gen[P] != c->gauge_gen) {
         for (int p = 0; p < 2; ++p) {
-            if (!c->gaugeP[P][p]) CK(cudaMalloc(&c->gaugeP[P][p], link_bytes_parity(P, vh)));
+            if (!c->gaugeP[P][p]) CK(dev_alloc(c, &c->gaugeP[P][p], link_bytes_parity(P, vh)));
             cudaError_t e = P == P32 ? launch_links_from64<P32>(c->gaugeP[P][p], c->gauge64[p], vh, st)
                           : P == PB16 ? launch_links_from64<PB16>(c->gaugeP[P][p], c->gauge64[p], vh, st)
                                       : launch_links_from64<PF16>(c->gaugeP[P][p], c->gauge64[p], vh, st);
@@ -314,7 +390,7 @@ static tm_status ensure_prec(tm_ctx* c, int P, cudaStream_t st) {
     if (c->clovP_stamp[P] != c->clover_stamp) {
         const size_t esz = prec_esz(P);
         auto conv = [&](void** dst, const double* src, int nreal) -> tm_status {
-            if (!*dst) CK(cudaMalloc(dst, esz * nreal * vh));
+            if (!*dst) CK(dev_alloc(c, dst, esz * nreal * vh));
             cudaError_t e = P == P32 ? launch_clover_from64<P32>(*dst, src, vh, nreal, st)
                           : P == PB16 ? launch_clover_from64<PB16>(*dst, src, vh, nreal, st)
                                       : launch_clover_from64<PF16>(*dst, src, vh, nreal, st);
@@ -329,24 +405,32 @@ static tm_status ensure_prec(tm_ctx* c, int P, cudaStream_t st) {
     return TM_OK;
 }
 
-// double-word copies of the FP64 links and clover arrays (made when stale)
+// memory of the double-word copies of the FP64 links and clover arrays
+static constexpr int DF_CLOV_REALS[3] = {CLOV_ODD_REALS, CLOV_EVEN_LIGHT_REALS, CLOV_EVEN_HEAVY_REALS};
+static tm_status alloc_df(tm_ctx* c) {
+    for (int p = 0; p < 2; ++p)
+        if (!c->gaugeDF[p]) CK(dev_alloc(c, &c->gaugeDF[p], link_bytes_parity(PDF, c->vh)));
+    for (int k = 0; k < 3; ++k) {
+        if (k == 2 && !c->have_heavy) continue;
+        if (!c->clovDF[k]) CK(dev_alloc(c, &c->clovDF[k], (size_t)8 * DF_CLOV_REALS[k] * c->vh));
+    }
+    return TM_OK;
+}
+
+// those copies (made when stale)
 static tm_status ensure_df(tm_ctx* c, cudaStream_t st) {
     CKS(ensure_prec(c, P64, st));
+    CKS(alloc_df(c));
     const long vh = c->vh;
     if (c->gaugeDF_gen != c->gauge_gen) {
-        for (int p = 0; p < 2; ++p) {
-            if (!c->gaugeDF[p]) CK(cudaMalloc(&c->gaugeDF[p], link_bytes_parity(PDF, vh)));
-            CK(launch_f64_to_df(c->gaugeDF[p], c->gauge64[p], 4 * 9 * vh, st));
-        }
+        for (int p = 0; p < 2; ++p) CK(launch_f64_to_df(c->gaugeDF[p], c->gauge64[p], 4 * 9 * vh, st));
         c->gaugeDF_gen = c->gauge_gen;
     }
     if (c->clovDF_stamp != c->clover_stamp) {
         const double* src[3] = {c->clovA64[1], c->clovB64, c->clovH64};
-        const int nreal[3] = {CLOV_ODD_REALS, CLOV_EVEN_LIGHT_REALS, CLOV_EVEN_HEAVY_REALS};
         for (int k = 0; k < 3; ++k) {
             if (k == 2 && !c->have_heavy) continue;
-            if (!c->clovDF[k]) CK(cudaMalloc(&c->clovDF[k], (size_t)8 * nreal[k] * vh));
-            CK(launch_f64_to_df(c->clovDF[k], src[k], (long)nreal[k] / 2 * vh, st));
+            CK(launch_f64_to_df(c->clovDF[k], src[k], (long)DF_CLOV_REALS[k] / 2 * vh, st));
         }
         c->clovDF_stamp = c->clover_stamp;
     }
@@ -1095,22 +1179,15 @@ static tm_status is_zero64(tm_ctx* c, const void* x64, cudaStream_t st, bool* ze
     return TM_OK;
 }
 
-// Ring of `bytes`-sized fields for a solver that enqueues `chunk` iterations at a time:
-// RING of them if the chunk is a multiple of it and memory allows, else 2 or 1 (the
-// iteration is then the textbook one).
-static tm_status ring_get(tm_ctx* c, size_t bytes, int chunk, void** f, int* m) {
-    int n = chunk % RING == 0 ? RING : (chunk % 2 == 0 ? 2 : 1);
-    for (int k = 0; k < n; ++k) {
-        const tm_status s = ws_get(c, WS_RING + k, bytes, &f[k]);
-        if (s == TM_ERR_OOM && k > 0) {
-            cudaGetLastError();
-            n = 1;
-            break;
-        }
-        CKS(s);
-    }
-    *m = n;
-    return TM_OK;
+// The further fields of a ring for a solver that enqueues `chunk` iterations at a time
+// (f[0] is among its needed scratch): RING of them if the chunk is a multiple of it and
+// they fit, else 2 or 1 (the iteration is then the textbook one).
+static void ring_get(tm_ctx* c, size_t bytes, int chunk, void** f, int* m) {
+    const int want = chunk % RING == 0 ? RING : (chunk % 2 == 0 ? 2 : 1);
+    int n = 1;
+    while (n < want && spare_get(c, WS_RING + n, bytes, &f[n])) ++n;
+    *m = n == want ? n : (n >= 2 ? 2 : 1);
+    for (int k = *m; n < want && k < RING; ++k) ws_drop(c, WS_RING + k);
 }
 
 // One system (A + shift) x = b of a solve: the solution in native FP64, its working
@@ -1158,15 +1235,59 @@ static cudaError_t cg_iteration(tm_ctx* c, tm_op op, const SolveSys* sys, int n,
 // Working fields of the systems, and the ring's length.  The first system takes the
 // single solve's buffers; the others those of a finished multishift solve of ns shifts
 // (its solutions and directions).  Only lattices of up to GROW_SITES sites per parity
-// allocate more (8 fields a system, 6 MB each at most in FP32 with two flavours); a
-// larger one takes no memory that a later allocation could miss.  Where the buffers end
-// there are fewer systems.
+// allocate more, as spare scratch (8 fields a system, 6 MB each at most in FP32 with two
+// flavours).  Where the buffers end there are fewer systems.
 constexpr long GROW_SITES = 32768;
 template <int PS, int NF>
-static tm_status solve_fields(tm_ctx* c, const tm_solve_params* sp, std::vector<SolveSys>& sys, int ns, int* m) {
+static void solve_spare(tm_ctx* c, const tm_solve_params* sp, std::vector<SolveSys>& sys, int ns, int* m) {
     const size_t bytes = spinor_bytes(PS, 12 * NF, c->vh);
-    const int chunk = sp->chunk > 0 ? sp->chunk : 16;
-    SolveSys& y = sys[0];
+    ring_get(c, bytes, sp->chunk > 0 ? sp->chunk : 16, sys[0].p, m);
+    const int n = (int)sys.size();
+    if (n > 1) {
+        void* partial = nullptr;
+        if (!spare_get(c, WS_GROUP_PARTIAL, sizeof(double) * c->max_blocks * (n - 1), &partial)) {
+            sys.resize(1);
+            return;
+        }
+    }
+    int next = 0;   // the multishift's 2 ns buffers, then those of WS_GROUP
+    auto field = [&](size_t size, void** out) {
+        for (; next < 2 * ns; ++next) {
+            *out = ws_held(c, next < ns ? WS_MS_X + next : WS_MS_P + next - ns, size);
+            if (!*out) continue;
+            ++next;
+            return true;
+        }
+        if (c->vh > GROW_SITES || !spare_get(c, WS_GROUP + next - 2 * ns, size, out)) return false;
+        ++next;
+        return true;
+    };
+    auto fields = [&](SolveSys& z) {
+        bool ok = field(spinor_bytes(P32, 12 * NF, c->vh), &z.x) && field(bytes, &z.r) && field(bytes, &z.te) &&
+                  field(bytes, &z.mid);
+        for (int k = 0; ok && k < *m; ++k) ok = field(bytes, &z.p[k]);
+        return ok;
+    };
+    for (int q = 1; q < n; ++q) {
+        const int first = std::max(next, 2 * ns);
+        if (fields(sys[q])) continue;
+        for (int k = first; k < next; ++k) ws_drop(c, WS_GROUP + k - 2 * ns);   // of a system that did not fit
+        sys.resize(q);
+        break;
+    }
+}
+
+// All that a solve needs, so that nothing is asked for after the spare fields: the first
+// system's working fields, and what solve_core and true_residual take.
+template <int PS, int NF>
+static tm_status solve_fields(tm_ctx* c, const tm_solve_params* sp, SolveSys& y) {
+    const size_t bytes = spinor_bytes(PS, 12 * NF, c->vh), b64 = spinor_bytes(P64, 12 * NF, c->vh);
+    void* f = nullptr;
+    for (int id : {WS_R64, WS_AX64, WS_TE64, WS_MID64}) CKS(ws_get(c, id, b64, &f));
+    if (PS != P64 && !sp->fp64_updates) {
+        CKS(alloc_df(c));
+        CKS(ws_get(c, WS_XDF, spinor_bytes(PDF, 12 * NF, c->vh), &f));
+    }
     if (PS == P64) {
         CKS(ws_get(c, WS_R64, bytes, &y.r));
         CKS(ws_get(c, WS_TE64, bytes, &y.te));
@@ -1178,47 +1299,7 @@ static tm_status solve_fields(tm_ctx* c, const tm_solve_params* sp, std::vector<
         CKS(ws_get(c, WS_MID_S, bytes, &y.mid));
         CKS(ws_get(c, WS_X_S, spinor_bytes(P32, 12 * NF, c->vh), &y.x));
     }
-    CKS(ring_get(c, bytes, chunk, y.p, m));
-    const int n = (int)sys.size();
-    if (n > 1) {
-        void* partial = nullptr;
-        const tm_status s = ws_get(c, WS_GROUP_PARTIAL, sizeof(double) * c->max_blocks * (n - 1), &partial);
-        if (s == TM_ERR_OOM) {
-            cudaGetLastError();
-            sys.resize(1);
-            return TM_OK;
-        }
-        CKS(s);
-    }
-    int next = 0;
-    auto field = [&](size_t size, void** out) {
-        for (; next < 2 * ns; ++next) {
-            auto it = c->ws.find(next < ns ? WS_MS_X + next : WS_MS_P + next - ns);
-            if (it == c->ws.end() || it->second.second < size) continue;
-            ++next;
-            *out = it->second.first;
-            return TM_OK;
-        }
-        if (c->vh > GROW_SITES) return TM_ERR_OOM;
-        return ws_get(c, WS_GROUP + next++ - 2 * ns, size, out);
-    };
-    auto fields = [&](SolveSys& z) {
-        CKS(field(spinor_bytes(P32, 12 * NF, c->vh), &z.x));
-        CKS(field(bytes, &z.r));
-        CKS(field(bytes, &z.te));
-        CKS(field(bytes, &z.mid));
-        for (int k = 0; k < *m; ++k) CKS(field(bytes, &z.p[k]));
-        return TM_OK;
-    };
-    for (int q = 1; q < n; ++q) {
-        const tm_status s = fields(sys[q]);
-        if (s == TM_ERR_OOM) {
-            cudaGetLastError();
-            sys.resize(q);
-            break;
-        }
-        CKS(s);
-    }
+    CKS(ws_get(c, WS_RING, bytes, &y.p[0]));
     return TM_OK;
 }
 
@@ -1231,7 +1312,7 @@ static tm_status solve_fields(tm_ctx* c, const tm_solve_params* sp, std::vector<
 // have stopped skip their blocks until the others have.
 template <int PS, int NF, int NP>
 static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std::vector<SolveSys>& sys, int m,
-                            void* b64, cudaStream_t st) {
+                            void* b64, double bb, cudaStream_t st) {
     static_assert(NP == 1 || PS != P64, "FP64 systems are solved one by one");
     constexpr int NC = 12 * NF;
     const long vh = c->vh;
@@ -1249,27 +1330,6 @@ static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std:
     const int nb = nblk(vh, BLAS_BS);
     const bool dw = PS != P64 && !sp->fp64_updates;   // double-word reliable updates
 
-    double bb = 0;
-    CKS((norm2_dev<P64, NC>(c, b64, st, &bb)));
-    for (SolveSys& y : sys) {
-        y.info->iters = 0;
-        y.info->reliable_updates = 0;
-    }
-    if (!std::isfinite(bb)) {
-        for (SolveSys& y : sys) {
-            y.info->true_rel_res = bb;
-            y.info->status = TM_ERR_BREAKDOWN;
-        }
-        return fail(TM_ERR_BREAKDOWN, "solve: right-hand side is not finite");
-    }
-    if (!(bb > 0)) {
-        for (SolveSys& y : sys) {
-            CK(cudaMemsetAsync(y.x64, 0, b64sz, st));
-            y.info->true_rel_res = 0.0;
-            y.info->status = TM_OK;
-        }
-        return TM_OK;
-    }
     const double target = tol * tol * bb;
     tm_status worst = TM_OK;
     int running = n;
@@ -1388,12 +1448,37 @@ static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std:
 template <int PS, int NF>
 static tm_status solve_systems(tm_ctx* c, tm_op op, const tm_solve_params* sp, std::vector<SolveSys>& sys, void* b64,
                                cudaStream_t st, int ns) {
-    int m = 1;
-    CKS((solve_fields<PS, NF>(c, sp, sys, ns, &m)));
-    if constexpr (PS != P64) {
-        if (sys.size() > 1) return solve_core<PS, NF, GROUP>(c, op, sp, sys, m, b64, st);
+    constexpr int NC = 12 * NF;
+    const size_t b64sz = spinor_bytes(P64, NC, c->vh);
+    double bb = 0;
+    CKS((norm2_dev<P64, NC>(c, b64, st, &bb)));
+    for (SolveSys& y : sys) {
+        y.info->iters = 0;
+        y.info->reliable_updates = 0;
     }
-    return solve_core<PS, NF, 1>(c, op, sp, sys, m, b64, st);
+    if (!std::isfinite(bb)) {
+        for (SolveSys& y : sys) {
+            y.info->true_rel_res = bb;
+            y.info->status = TM_ERR_BREAKDOWN;
+        }
+        return fail(TM_ERR_BREAKDOWN, "solve: right-hand side is not finite");
+    }
+    if (!(bb > 0)) {
+        for (SolveSys& y : sys) {
+            CK(cudaMemsetAsync(y.x64, 0, b64sz, st));
+            y.info->true_rel_res = 0.0;
+            y.info->status = TM_OK;
+        }
+        return TM_OK;
+    }
+    CKS((solve_fields<PS, NF>(c, sp, sys[0])));
+    int m = 1;
+    const SpareUse use(c);
+    solve_spare<PS, NF>(c, sp, sys, ns, &m);
+    if constexpr (PS != P64) {
+        if (sys.size() > 1) return solve_core<PS, NF, GROUP>(c, op, sp, sys, m, b64, bb, st);
+    }
+    return solve_core<PS, NF, 1>(c, op, sp, sys, m, b64, bb, st);
 }
 
 template <int NF>
@@ -1501,8 +1586,7 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
     const size_t bs = spinor_bytes(PS, NC, vh), bx = spinor_bytes(PX, NC, vh);
     const int chunk = sp->chunk > 0 ? sp->chunk : 16;
     void *ps, *tes, *mids, *rs[RING];
-    int rm = 1;   // residuals kept between two updates of the shifts
-    CKS(ring_get(c, bs, chunk, rs, &rm));
+    CKS(ws_get(c, WS_RING, bs, &rs[0]));
     CKS(ws_get(c, WS_P_S, bs, &ps));
     CKS(ws_get(c, WS_TE_S, bs, &tes));
     CKS(ws_get(c, WS_MID_S, bs, &mids));
@@ -1516,6 +1600,9 @@ static tm_status multishift_core(tm_ctx* c, tm_op op, int ns, const double* sh_s
         }
         CK(cudaMemsetAsync(mv.x[k], 0, bx, st));
     }
+    int rm = 1;   // residuals kept between two updates of the shifts
+    const SpareUse use(c);
+    ring_get(c, bs, chunk, rs, &rm);
     const int nb = nblk(vh, BLAS_BS);
     double bb;
     CKS((norm2_dev<P64, NC>(c, b64, st, &bb)));
@@ -2315,20 +2402,20 @@ extern "C" tm_status tm_ptc_destroy(tm_ptc* n) {
     return TM_OK;
 }
 
-static tm_status ptc_buffers(tm_ptc* n, const tm_ctx* c) {
+static tm_status ptc_buffers(tm_ptc* n, tm_ctx* c) {
     const long V = 2 * c->vh;
     if (n->V == V) return TM_OK;
     ptc_free_acts(n);
-    for (int l = 0; l <= n->L; ++l) CK(cudaMalloc(&n->act[l], (size_t)n->ch[l] * 3 * 16 * V));
-    for (auto& d : n->del) CK(cudaMalloc(&d, (size_t)PTC_MAXC * 3 * 16 * V));
-    CK(cudaMalloc(&n->dpart, sizeof(double) * ((V + 255) / 256)));
-    CK(cudaMalloc(&n->zmix, (size_t)9 * 3 * 16 * V));
-    CK(cudaMalloc(&n->lp, (size_t)8 * 9 * 4 * V));
+    for (int l = 0; l <= n->L; ++l) CK(dev_alloc(c, &n->act[l], (size_t)n->ch[l] * 3 * 16 * V));
+    for (auto& d : n->del) CK(dev_alloc(c, &d, (size_t)PTC_MAXC * 3 * 16 * V));
+    CK(dev_alloc(c, &n->dpart, sizeof(double) * ((V + 255) / 256)));
+    CK(dev_alloc(c, &n->zmix, (size_t)9 * 3 * 16 * V));
+    CK(dev_alloc(c, &n->lp, (size_t)8 * 9 * 4 * V));
     const size_t s32 = spinor_bytes(P32, 12, c->vh);
-    CK(cudaMalloc(&n->e32, s32));
-    CK(cudaMalloc(&n->r32, s32));
-    CK(cudaMalloc(&n->tmp32[0], s32));
-    CK(cudaMalloc(&n->tmp32[1], s32));
+    CK(dev_alloc(c, &n->e32, s32));
+    CK(dev_alloc(c, &n->r32, s32));
+    CK(dev_alloc(c, &n->tmp32[0], s32));
+    CK(dev_alloc(c, &n->tmp32[1], s32));
     n->V = V;
     return TM_OK;
 }
@@ -2784,4 +2871,5 @@ tm_status tmk_failf(tm_status s, const char* fmt, ...) {
 }
 tm_status tmk_ensure_prec(tm_ctx* c, int P, cudaStream_t st) { return ensure_prec(c, P, st); }
 tm_status tmk_ws_get(tm_ctx* c, int id, size_t bytes, void** out) { return ws_get(c, id, bytes, out); }
+bool tmk_spare_release(tm_ctx* c) { return spare_release(c); }
 }  // namespace tmk

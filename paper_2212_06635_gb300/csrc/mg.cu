@@ -44,6 +44,7 @@ namespace tmk {
 tm_status tmk_failf(tm_status s, const char* fmt, ...);
 tm_status tmk_ensure_prec(tm_ctx* c, int P, cudaStream_t st);
 tm_status tmk_ws_get(tm_ctx* c, int id, size_t bytes, void** out);
+bool tmk_spare_release(tm_ctx* c);
 }  // namespace tmk
 
 using namespace tmk;
@@ -979,12 +980,24 @@ bool dev_ptr(const void* p) {
 
 size_t full_bytes(int P, long vh) { return 2 * spinor_bytes(P, 12, vh); }
 
+// device memory; the context's spare scratch makes room for it
+template <typename T>
+cudaError_t dev_alloc(tm_ctx* c, T** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    if (!tmk_spare_release(c)) return e;
+    e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
 // even-site A in storage precision P (lazily; odd A comes with tmk_ensure_prec)
 tm_status ensure_full(tm_ctx* c, int P, cudaStream_t st) {
     MCKS(tmk_ensure_prec(c, P, st));
     if (P == P64) return TM_OK;
     if (c->clovAeP_stamp[P] != c->clover_stamp) {
-        if (!c->clovAeP[P]) MCK(cudaMalloc(&c->clovAeP[P], (size_t)prec_esz(P) * CLOV_ODD_REALS * c->vh));
+        if (!c->clovAeP[P]) MCK(dev_alloc(c, &c->clovAeP[P], (size_t)prec_esz(P) * CLOV_ODD_REALS * c->vh));
         MCK(launch_clover_from64<P32>(c->clovAeP[P], c->clovA64[0], c->vh, CLOV_ODD_REALS, st));
         c->clovAeP_stamp[P] = c->clover_stamp;
     }
@@ -1416,19 +1429,19 @@ extern "C" tm_status tm_mg_create(tm_mg** out, tm_ctx* c, const tm_mg_params* p)
     g->fbytes = full_bytes(g->P, c->vh);
     const size_t ce = g->P == P64 ? 16 : 8;
     cudaError_t e = cudaSuccess;
-    e = e ? e : cudaMalloc(&g->Pm, ce * (size_t)g->nfine * p->nvec);   // 12 V nvec complex
-    e = e ? e : cudaMalloc(&g->Mc, ce * (size_t)g->m.Nb * MG_NSLOT * 4 * p->nvec * p->nvec);
-    e = e ? e : cudaMalloc(&g->vecs, g->fbytes * p->nvec);
+    e = e ? e : dev_alloc(c, &g->Pm, ce * (size_t)g->nfine * p->nvec);   // 12 V nvec complex
+    e = e ? e : dev_alloc(c, &g->Mc, ce * (size_t)g->m.Nb * MG_NSLOT * 4 * p->nvec * p->nvec);
+    e = e ? e : dev_alloc(c, &g->vecs, g->fbytes * p->nvec);
     g->cvec.assign(4 + 2 * p->coarse_restart, nullptr);
-    for (auto& v : g->cvec) e = e ? e : cudaMalloc(&v, ce * g->ncoarse);
-    e = e ? e : cudaMalloc(&g->fz, g->fbytes);
-    e = e ? e : cudaMalloc(&g->frs, g->fbytes);
-    e = e ? e : cudaMalloc(&g->fmr, g->fbytes);
-    e = e ? e : cudaMalloc(&g->ctl, 3 * sizeof(MgCtl));
+    for (auto& v : g->cvec) e = e ? e : dev_alloc(c, &v, ce * g->ncoarse);
+    e = e ? e : dev_alloc(c, &g->fz, g->fbytes);
+    e = e ? e : dev_alloc(c, &g->frs, g->fbytes);
+    e = e ? e : dev_alloc(c, &g->fmr, g->fbytes);
+    e = e ? e : dev_alloc(c, &g->ctl, 3 * sizeof(MgCtl));
     e = e ? e : cudaMallocHost(&g->h_ctl, 3 * sizeof(MgCtl));
-    e = e ? e : cudaMalloc(&g->partial, sizeof(double) * MG_GRID_CAP * MG_PART_W);
-    e = e ? e : cudaMalloc(&g->op_partial, sizeof(double) * 3 * full_op_blocks(c));
-    e = e ? e : cudaMalloc(&g->counter, sizeof(unsigned int));
+    e = e ? e : dev_alloc(c, &g->partial, sizeof(double) * MG_GRID_CAP * MG_PART_W);
+    e = e ? e : dev_alloc(c, &g->op_partial, sizeof(double) * 3 * full_op_blocks(c));
+    e = e ? e : dev_alloc(c, &g->counter, sizeof(unsigned int));
     e = e ? e : cudaMemset(g->counter, 0, sizeof(unsigned int));
     e = e ? e : cudaMemset(g->ctl, 0, 3 * sizeof(MgCtl));
     e = e ? e : cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking);

@@ -59,6 +59,8 @@ struct tm_ctx {
     double* h_scal = nullptr;
 
     std::map<int, std::pair<void*, size_t>> ws;   // workspace buffers by id
+    size_t ws_bytes = 0, ws_limit = 0;            // held, and a bound on it (0: none; tests)
+    bool spare_busy = false;                      // a running solve works in its spare buffers
 
     // host-buffer staging of tm_field_import / tm_field_export: a ring of device
     // buffers per direction, each released by an event recorded after its last use,
