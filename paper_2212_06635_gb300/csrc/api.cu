@@ -1723,16 +1723,18 @@ static tm_status ms_core(tm_ctx* c, tm_op op, int ns, const double* shifts, void
     std::vector<double> sh(ns);
     for (int k = 0; k < ns; ++k) sh[k] = shifts[order[k]];
     std::vector<void*> xk64(ns);
-    for (int k = 0; k < ns; ++k) CKS(ws_get(c, WS_MS_X64 + k, b64sz, &xk64[k]));
+    xk.assign(ns, nullptr);
+    tm_status s = TM_OK;
+    for (int k = 0; s == TM_OK && k < ns; ++k) s = ws_get(c, WS_MS_X64 + k, b64sz, &xk64[k]);
     int ms_iters = 0;
-    tm_status s = nf == 1 ? multishift_dispatch<1>(c, op, ns, sh.data(), b64, sp, xk64, &ms_iters, st)
-                          : multishift_dispatch<2>(c, op, ns, sh.data(), b64, sp, xk64, &ms_iters, st);
+    if (s == TM_OK)
+        s = nf == 1 ? multishift_dispatch<1>(c, op, ns, sh.data(), b64, sp, xk64, &ms_iters, st)
+                    : multishift_dispatch<2>(c, op, ns, sh.data(), b64, sp, xk64, &ms_iters, st);
     tm_status worst = s;
     // shift-by-shift refinement with mixed-precision CG, in its own storage
     // precision when sp->refine names one
     tm_solve_params rsp = *sp;
     if (sp->refine != TM_F64) rsp.sloppy = sp->refine;
-    xk.assign(ns, nullptr);
     for (int k = 0; k < ns; ++k) {
         tm_solve_info& inf = infos[order[k]];
         std::memset(&inf, 0, sizeof(inf));
@@ -1748,7 +1750,10 @@ static tm_status ms_core(tm_ctx* c, tm_op op, int ns, const double* shifts, void
         }
         const tm_status r = nf == 1 ? solve_dispatch<1>(c, op, &rsp, sys, b64, st, ns)
                                     : solve_dispatch<2>(c, op, &rsp, sys, b64, st, ns);
-        for (const SolveSys& y : sys) y.info->iters += ms_iters;
+        for (const SolveSys& y : sys) {
+            y.info->iters += ms_iters;
+            if (r != TM_OK && !y.done) y.info->status = r;   // ended before it was solved
+        }
         if (r != TM_OK && worst == TM_OK) worst = r;
         k += (int)sys.size();
     }

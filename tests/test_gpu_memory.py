@@ -118,3 +118,32 @@ def test_spare_fields_are_given_back_for_a_needed_one():
         assert _bound(lat, held) < held
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("room", [1, 3, 8, 12, 20], ids=lambda r: f"{r} fields")
+def test_multishift_without_room_returns_an_error(room):
+    """A multishift or rational call whose fields do not fit says so, in the records too,
+    and the context goes on working."""
+    op, lat = _lat(1)
+    tm = lat.tm
+    try:
+        b = F.odd_spinor(DIMS, 1504)
+        shifts = [0.01, 0.02, 0.04, 0.08]
+        _bound(lat, room * _field(0, 1))
+        xs = [to_dev(np.zeros_like(b)) for _ in shifts]
+        sp = tm.solve_params(tol=1e-9, sloppy=1)
+        infos = tm.tm_solve_multishift(lat.ctx, tm.TM_MDAGM, shifts, xs, to_dev(b), sp, check=False)
+        fits = room == 20
+        assert all(i.status == (0 if fits else tm.TM_ERR_OOM) for i in infos)
+        assert all((float(x.norm()) > 0) == (room >= 12) for x in xs)   # (12: the refinement had no room)
+        if not fits:
+            with pytest.raises(tm.TMError) as e:
+                tm.tm_solve_multishift(lat.ctx, tm.TM_MDAGM, shifts, xs, to_dev(b), sp)
+            assert e.value.status == tm.TM_ERR_OOM
+            with pytest.raises(tm.TMError):
+                tm.tm_rational_apply(lat.ctx, tm.TM_MDAGM, (1.0, [0.5] * 4, shifts), to_dev(b), to_dev(b), sp)
+        _bound(lat, 0)
+        infos = tm.tm_solve_multishift(lat.ctx, tm.TM_MDAGM, shifts, xs, to_dev(b), sp)
+        assert all(i.status == 0 and i.true_rel_res <= 1e-9 for i in infos)
+    finally:
+        lat.close()
