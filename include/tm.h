@@ -93,7 +93,9 @@ typedef struct {
     tm_prec sloppy;      /* storage precision of the inner iteration; TM_F64 = plain FP64 CG */
     double delta;        /* reliable-update trigger: ||r_sloppy|| < delta * ||r_true_last||;
                             <= 0 selects a default of about sqrt(unit roundoff) of the
-                            sloppy storage: FP16 0.02, BF16 0.06, FP32 0.002 */
+                            sloppy storage: FP16 0.02, BF16 0.06, FP32 0.002, past which
+                            the iteration goes on to a target that is less than a
+                            factor 2.5 (FP32: 10) away */
     int chunk;           /* iterations enqueued between two host checks (0 = default 16) */
     int use_graph;       /* capture the chunk in a CUDA graph and replay it */
     tm_prec refine;      /* tm_solve_multishift only: storage precision of the

@@ -663,17 +663,23 @@ static double default_delta(int sloppy) {
 }
 
 // ||r||^2 at which the sloppy iteration stops for a reliable update: delta^2 of the last
-// true residual, or the solve's target where that is near enough to be reached in one
-// leg, since an update just above the target costs as much as any other.  How far is
-// what the recursion carries: at the default thresholds the iterated residual of FP32
-// differs from the true one by less than 1e-3 after a drop of 500, that of FP16 by 5-20 %
-// after a drop of 50 (heavy multishift and light CG, tolerance 1e-12); so up to 10
-// times delta for FP32 and 2.5 times for the 16-bit formats.  A leg that ends above the
-// target is followed by another.
-static double leg_stop(int sloppy, double delta, double rr, double target) {
-    const double t = delta * delta * rr, reach = sloppy == TM_F32 ? 10.0 : 2.5;
-    return t > reach * reach * target ? t : target;
-}
+// true residual.  Where the caller leaves delta to the library, the solve's target
+// instead if that is near enough to be reached in one leg, since an update just above
+// the target costs as much as any other.  How far is what the recursion carries: at the
+// default thresholds the iterated residual of FP32 differs from the true one by less
+// than 1e-3 after a drop of 500, that of FP16 by 5-20 % after a drop of 50 (heavy
+// multishift and light CG, tolerance 1e-12); so up to 10 times delta for FP32 and 2.5
+// times for the 16-bit formats.  A leg that ends above the target is followed by another.
+struct LegRule {
+    double delta, reach;
+    LegRule(int sloppy, double chosen)   // chosen: tm_solve_params.delta
+        : delta(sloppy == P64 ? 0.0 : (chosen > 0 ? chosen : default_delta(sloppy))),
+          reach(chosen > 0 ? 1.0 : (sloppy == P32 ? 10.0 : 2.5)) {}
+    double stop(double rr, double target) const {
+        const double t = delta * delta * rr;
+        return t > reach * reach * target ? t : target;
+    }
+};
 
 // Whether a leg that took ||r||^2 from rr0 to the iterated rr is sure enough to have met
 // the target that its residual is confirmed in FP64 at once, without a double-word one
@@ -1325,7 +1331,7 @@ static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std:
     CKS(ws_get(c, WS_MID64, b64sz, &mid64));
     const double tol = sp->tol > 0 ? sp->tol : 1e-10;
     const int maxiter = sp->maxiter > 0 ? sp->maxiter : 100000;
-    const double delta = PS == P64 ? 0.0 : (sp->delta > 0 ? sp->delta : default_delta(PS));
+    const LegRule leg(PS, sp->delta);
     const int chunk = sp->chunk > 0 ? sp->chunk : 16;
     const int nb = nblk(vh, BLAS_BS);
     const bool dw = PS != P64 && !sp->fp64_updates;   // double-word reliable updates
@@ -1360,7 +1366,7 @@ static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std:
         h.shift = y.shift;
         h.maxiter = maxiter;
         h.ring = m;
-        h.stop_rr = leg_stop(PS, delta, y.rr, target);
+        h.stop_rr = leg.stop(y.rr, target);
         h.flag = CTL_RUN;
         if (!(y.rr > target)) {
             finish(y, 0, TM_OK);
@@ -1435,7 +1441,7 @@ static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std:
             h.slot = 0;
             h.beta = y.rr / h.rr_old;
             h.rr = y.rr;
-            h.stop_rr = leg_stop(PS, delta, y.rr, target);
+            h.stop_rr = leg.stop(y.rr, target);
             h.flag = CTL_RUN;
             CKS(put_ctl(c, st, q));
         }
@@ -2024,7 +2030,7 @@ static tm_status batch_core(tm_ctx** cs, int n, tm_op op, const tm_solve_params*
     constexpr int PX = PS == P64 ? P64 : P32;
     const double tol = sp->tol > 0 ? sp->tol : 1e-10;
     const int maxiter = sp->maxiter > 0 ? sp->maxiter : 100000;
-    const double delta = PS == P64 ? 0.0 : (sp->delta > 0 ? sp->delta : default_delta(PS));
+    const LegRule leg(PS, sp->delta);
     const int chunk = sp->chunk > 0 ? sp->chunk : 16;
     std::vector<double> bb(n), rr(n);
     std::vector<int> done(n, 0);
@@ -2055,7 +2061,7 @@ static tm_status batch_core(tm_ctx** cs, int n, tm_op op, const tm_solve_params*
         std::memset(&h, 0, sizeof(SolverCtl));
         h.rr = h.rr_old = rr[q];
         h.maxiter = maxiter;
-        h.stop_rr = leg_stop(PS, delta, rr[q], tol * tol * bb[q]);
+        h.stop_rr = leg.stop(rr[q], tol * tol * bb[q]);
         h.flag = CTL_RUN;
         CKS(put_ctl(c, st));
     }
@@ -2227,7 +2233,7 @@ static tm_status batch_core(tm_ctx** cs, int n, tm_op op, const tm_solve_params*
             h.rr = rr[q];
             h.iter = iters;
             h.shift = 0.0;
-            h.stop_rr = leg_stop(PS, delta, rr[q], tol * tol * bb[q]);
+            h.stop_rr = leg.stop(rr[q], tol * tol * bb[q]);
             h.flag = CTL_RUN;
             CKS(put_ctl(c, st));
         }

@@ -452,6 +452,32 @@ def test_returned_residual_of_a_mixed_solve_is_the_fp64_one(sloppy, delta):
         lat.close()
 
 
+@pytest.mark.parametrize("sloppy,delta,tol", [(1, 1e-3, 2e-4), (3, 0.05, 0.03), (2, 0.1, 0.05)])
+def test_a_chosen_update_threshold_is_kept_near_the_target(sloppy, delta, tol):
+    """A leg ends at delta ||r|| for a delta that the caller chose, however near the
+    target is: two updates at least.  Under the library's own threshold one leg reaches
+    a target that near."""
+    dims = (6, 4, 6, 10)
+    _, lat = _lat(dims, 1260)
+    tm = lat.tm
+    own = {1: 2e-3, 2: 0.06, 3: 0.02}[sloppy]
+    try:
+        b = to_dev(F.odd_spinor(dims, 2260))
+        for d, t, updates in ((delta, tol, 2), (0.0, own * tol / delta, 1)):
+            sp = tm.solve_params(tol=t, sloppy=sloppy, delta=d)
+            x, xb = 0 * b, 0 * b
+            infos = [tm.tm_solve_cg(lat.ctx, tm.TM_MDAGM, sp, x, b)]
+            infos += tm.tm_solve_batch([lat.ctx], tm.TM_MDAGM, sp, [xb], [b])
+            for info in infos:
+                assert info.status == 0 and info.true_rel_res <= t
+                # (under the own threshold the leg may end just above the target)
+                assert info.reliable_updates >= 2 if updates == 2 else info.reliable_updates <= 2
+            if updates == 1 and sloppy == 1:
+                assert infos[0].reliable_updates == 1
+    finally:
+        lat.close()
+
+
 def test_heavy_fp64_cg_with_the_flavours_over_thread_pairs():
     """6,000 sites per parity (a ragged last block), above the small-lattice line of the
     two-flavour FP64 passes: plain FP64 CG and FP64 multishift reach the tolerance."""
