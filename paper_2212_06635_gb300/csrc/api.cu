@@ -1404,9 +1404,11 @@ static tm_status solve_core(tm_ctx* c, tm_op op, const tm_solve_params* sp, std:
             SolverCtl& h = c->h_ctl[q];
             if (y.done || h.flag == CTL_RUN) continue;
             // the steps of the ring that x does not hold yet: the iteration that stopped the
-            // run ended before its ring's update, one that broke down does not count
+            // run ended before its ring's update; one that found no step (alpha, with ||r||^2
+            // still finite) is not counted and has nothing to add
             const int done = h.iter - y.base;
-            const int left = h.flag == CTL_BREAKDOWN ? done % m : (done > 0 ? (done - 1) % m + 1 : 0);
+            const bool no_step = h.flag == CTL_BREAKDOWN && std::isfinite(h.rr);
+            const int left = no_step ? done % m : (done > 0 ? (done - 1) % m + 1 : 0);
             if (left > 0)
                 CK((launch_cg_xupdate<PS, PS == P64 ? P64 : P32, NC, 1>(vb_ring(c, y.x, y.p, m, q), left, true, nb, st)));
             if (h.flag == CTL_BREAKDOWN) {

@@ -499,3 +499,27 @@ def test_heavy_fp64_cg_with_the_flavours_over_thread_pairs():
             assert i.status == 0 and np.linalg.norm(r) <= 1.05e-12 * np.linalg.norm(host), s
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("chunk", [1, 2, 3, 16])
+def test_a_breakdown_of_the_residual_keeps_the_step_that_led_to_it(chunk):
+    """FP64 CG scaled so that ||r_1||^2 overflows while <p, A p> does not: the first step
+    is complete, so x = alpha b for every length of the ring of directions."""
+    dims = (4, 4, 4, 4)
+    op, lat = _lat(dims, 1270)
+    tm = lat.tm
+    try:
+        b, _ = S.cg(op.MdagM, F.odd_spinor(dims, 1271), tol=1e-10)[:2]
+        bb = S.norm2(b)
+        alpha = bb / S.dot(b, op.MdagM(b)).real
+        r1 = b - alpha * op.MdagM(b)
+        scale = np.sqrt(1.6e308 / bb)
+        assert S.norm2(r1) / bb * 1.6 > 1.85   # FP64 ends at 1.797e308
+        x = to_dev(np.zeros_like(b))
+        sp = tm.solve_params(tol=1e-10, sloppy=0, chunk=chunk)
+        info = tm.tm_solve_cg(lat.ctx, tm.TM_MDAGM, sp, x, to_dev(scale * b), check=False)
+        assert info.status == tm.TM_ERR_BREAKDOWN and info.iters == 1
+        got = from_dev(x, b.shape) / scale
+        assert np.linalg.norm(got - alpha * b) <= 1e-12 * alpha * np.sqrt(bb)
+    finally:
+        lat.close()
