@@ -457,12 +457,15 @@ static const void* clovH_ptr(const tm_ctx* c, int P) {
 // over several warps (dslash_split.cu).  M_hat^dagger M_hat, calls back to back, direct
 // / split, us, at 4,096 / 10,000 / 20,736 sites:
 //   light FP32 20.6 / 16.0, 20.7 / 18.6, 22.7 / 22.7; light FP16 22.7 / 16.7,
-//   22.6 / 20.7, 22.8 / 22.7; light FP64 156 / 62, 161 / 132, 233 / 216 (38,416 sites:
-//   305 / 348); heavy FP32 24.8 / 20.7, 27.7 / 34.9; heavy FP16 26.9 / 22.7,
-//   28.8 / 39.1; heavy FP64 178 / 102, 262 / 294, 447 / 498 (6,144 sites: 182 / 198;
-//   4864 are one wave of the split kernel).
+//   22.6 / 20.7, 22.8 / 22.7; heavy FP32 24.8 / 20.7, 27.7 / 34.9; heavy FP16
+//   26.9 / 22.7, 28.8 / 39.1.
+// FP64 goes by waves of blocks of the split kernel, one block on each of the 152 SMs:
+//   light 162 / 63 (4,096), 168 / 137 (10,368), 170 / 178 (19,208), 245 / 225 (20,736),
+//   248 / 229 (24,192: five waves), 248 / 265 (24,576), 319 / 319 (32,928);
+//   heavy 182 / 106 (4,096: one wave), 187 / 206 (5,000), 275 / 307 (10,368).
+constexpr long SPLIT_WAVE = 152 * SPLIT_SITES;
 static long split_limit(int P, int nf) {
-    if (P == P64) return nf == 1 ? 24576 : 4864;
+    if (P == P64) return nf == 1 ? 5 * SPLIT_WAVE : SPLIT_WAVE;
     return nf == 1 ? 12288 : 6144;
 }
 

@@ -52,29 +52,16 @@ __device__ __forceinline__ void hop_mu(cpx<typename PT<P>::R> (&acc)[NF][4][3], 
     cpx<R> u[9];
     cpx<R> psi[NF * 12];
     float sc;
-    if constexpr (P == P64) {   // bound by FP64 arithmetic: the form with the fewest instructions
-        cpx<R> gf[NF][2][3];
-        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nf, psi, sc);
-        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
+    load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nf, psi, sc);
+    load_link<P>(pr.gauge[po], g.vh, MU, i, u);
 #pragma unroll
-        for (int f = 0; f < NF; ++f) hop_forward<R, MU, SC>(gf[f][0], gf[f][1], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
-        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nb, psi, sc);
-        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
+    for (int f = 0; f < NF; ++f)
+        hop_dir<R, MU, -1, false, SC, FIRST, NF == 2>(acc[f], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
+    load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nb, psi, sc);
+    load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
 #pragma unroll
-        for (int f = 0; f < NF; ++f)
-            hop_backward<R, MU, SC, FIRST>(acc[f], gf[f][0], gf[f][1], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
-    } else {
-        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nf, psi, sc);
-        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-            hop_dir<R, MU, -1, false, SC, FIRST, NF == 2>(acc[f], psi + 12 * f, u, SC ? ph_f * (R)sc : ph_f);
-        load_spinor_unscaled<P, NF * 12>(pr.in, g.vh, nb, psi, sc);
-        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-            hop_dir<R, MU, +1, true, SC, false, NF == 2>(acc[f], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
-    }
+    for (int f = 0; f < NF; ++f)
+        hop_dir<R, MU, +1, true, SC, false, NF == 2>(acc[f], psi + 12 * f, u, SC ? ph_b * (R)sc : ph_b);
 }
 
 // out = B_c v (CONJ: B_c^dagger v) per chirality block c of the even-site inverse.
@@ -129,10 +116,13 @@ __device__ __forceinline__ void inverse_blocks(cpx<typename PT<P>::R>* out, cons
 //   two-flavour odd pass: 4 blocks in 16-bit storage (128 registers; 3 / 5
 //     blocks: 63.8 -> 67.7 / 75.0 us FP16) and 3 in FP32 (168 registers, 8 B
 //     spilled: 94.8 -> 78.1 us at 24^3x48; 2 / 4 blocks: 94.5 / 84.4 us);
-//   FP64: 8 blocks of 64 threads (128 registers).  The FP64 units bound the passes,
-//     but the waits for operands show at 8 warps per SM: 16^3x32 even / odd
-//     149.8 / 153.2 -> 141.6 / 143.4 us against 4 blocks (253 registers, none
-//     spilled); at 24^3x48, where many waves even this out, 636 / 653 -> 640 / 664 us.
+//   FP64: 8 blocks of 64 threads (128 registers; 172 B stored to and 176 B loaded from
+//     the stack in the even pass, 264 / 300 B in the odd one, 80 / 80 B in the
+//     update).  The FP64 units bound the passes, but the waits for operands show at 8
+//     warps per SM on lattices of few waves: 4 / 6 / 8 blocks (254 and 168 registers,
+//     none spilled) take, even + odd, 320 / 318 / 300 us at 16^3x32, 1377 / 1376 /
+//     1378 us at 24^3x48 and 4121 / 4114 / 4116 us at 32^3x64.  4 blocks of 128 threads:
+//     320 / 1379 / 4112 us.
 // (The two-flavour even pass splits the flavours over a thread pair: dslash_heavy.cu.)
 template <int P, int NF, int KIND>
 constexpr int dslash_min_blocks() {

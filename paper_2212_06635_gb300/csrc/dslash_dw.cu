@@ -28,8 +28,8 @@
 //   hide the loads.
 // M_hat^dagger M_hat at 24^3x48 with its conversions 1232 -> 912 us, the heavy
 // operator 3022 -> 2264 us against loads at the point of use, rows unrolled, at the
-// same errors (8.0e-15 / 8.5e-15).  Pairing the two hops of a direction as the FP64
-// passes do (36 compensated additions instead of 48) gives 8.1e-15 and is not used.
+// same errors (8.0e-15 / 8.5e-15).  Pairing the two hops of a direction (dslash_common.cuh;
+// 36 compensated additions instead of 48) gives 8.1e-15 and is not used.
 // The operator's last pass stores FP64 itself: its conversions (2 per cycle and SM) hide
 // behind the FP32 work, as a kernel of their own they took 43 us (light, 905 -> 865 us).
 #include "tm_internal.h"

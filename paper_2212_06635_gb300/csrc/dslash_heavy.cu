@@ -95,30 +95,21 @@ __device__ __forceinline__ void hop_mu_flavour(cpx<typename PT<P>::R> (&acc)[4][
     cpx<R> psi[12];
     float sc;
     constexpr bool FIRST = MU == 0 && heavy_first<P>();
-    if constexpr (P == P64) {
-        cpx<R> gf0[3], gf1[3];
-        load_flavour_unscaled<P>(pr.in, g.vh, nf, f, psi, sc);
-        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
-        hop_forward<R, MU, SC>(gf0, gf1, psi, u, SC ? ph_f * (R)sc : ph_f);
-        load_flavour_unscaled<P>(pr.in, g.vh, nb, f, psi, sc);
-        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
-        hop_backward<R, MU, SC, FIRST>(acc, gf0, gf1, psi, u, SC ? ph_b * (R)sc : ph_b);
-    } else {
-        load_flavour_unscaled<P>(pr.in, g.vh, nf, f, psi, sc);
-        load_link<P>(pr.gauge[po], g.vh, MU, i, u);
-        hop_dir<R, MU, -1, false, SC, FIRST, true>(acc, psi, u, SC ? ph_f * (R)sc : ph_f);
-        load_flavour_unscaled<P>(pr.in, g.vh, nb, f, psi, sc);
-        load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
-        hop_dir<R, MU, +1, true, SC, false, true>(acc, psi, u, SC ? ph_b * (R)sc : ph_b);
-    }
+    load_flavour_unscaled<P>(pr.in, g.vh, nf, f, psi, sc);
+    load_link<P>(pr.gauge[po], g.vh, MU, i, u);
+    hop_dir<R, MU, -1, false, SC, FIRST, true>(acc, psi, u, SC ? ph_f * (R)sc : ph_f);
+    load_flavour_unscaled<P>(pr.in, g.vh, nb, f, psi, sc);
+    load_link<P>(pr.gauge[1 - po], g.vh, MU, nb, u);
+    hop_dir<R, MU, +1, true, SC, false, true>(acc, psi, u, SC ? ph_b * (R)sc : ph_b);
 }
 
 // Resident blocks per SM the register allocation must allow (128 threads = 64
 // sites).  At 24^3x48: 16-bit 4 / 5 / 6 blocks take 73.9 / 73.5 / 73.9 us (FP16)
 // and 72.1 / 69.8 / 72.7 us (BF16), with the spinor's factor multiplying the half
 // spinors (folded into the FMAs as now, BF16 at 5 blocks: 66.7 us); FP32 3 / 4 / 5
-// blocks 96.4 / 96.4 / 89.7 us.  FP64 (64-thread blocks): 8 as in dslash.cu; 4 / 8
-// blocks 317.4 / 317.6 us at 16^3x32.
+// blocks 96.4 / 96.4 / 89.7 us.  FP64 (64-thread blocks): 8 as in dslash.cu; both
+// passes at 4 / 6 / 8 blocks 614 / 616 / 618 us at 16^3x32, 3005 / 3008 / 3013 us at
+// 24^3x48, but 266 / 237 / 236 us at 12^3x24.
 template <int P, int KIND>
 constexpr int heavy_min_blocks() {
     return (P == PF16 || P == PB16) ? 5 : (P == P32 ? 5 : 8);
@@ -194,11 +185,11 @@ __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, KIND>())) dslash_heav
 
 // Odd pass of the same operator (formula as in dslash.cu), the flavours over a thread
 // pair: twice the threads and half the chain of each.  In FP64, where one thread per
-// site spills, it is the faster form at every size (normal operator at 12^4 313 -> 262 us,
-// 12^3x24 487 -> 447, 16^3x32 1213 -> 1172, 24^3x48 5843 -> 5742 us; 5 or 6 resident blocks
-// measure as 8); in FP32 and 16 bits
-// one thread per site is (24^3x48 322 against 343 us, 257 against 272 us), also on
-// lattices of 10,000 sites.
+// site spills, it is the faster form at every size (normal operator, with the hops of a
+// direction as a pair in both forms, 12^4 313 -> 262 us, 12^3x24 487 -> 447, 16^3x32
+// 1213 -> 1172, 24^3x48 5843 -> 5742 us; with single hops, as here, the last three take
+// 471, 1229 and 6021 us); in FP32 and 16 bits one thread per site is (24^3x48 322 against
+// 343 us, 257 against 272 us), also on lattices of 10,000 sites.
 template <int P, int KIND, int BS>
 __global__ void __launch_bounds__(BS, (heavy_min_blocks<P, K1_EO_INV>())) dslash_pair_kernel(const __grid_constant__ OpBatch<1> b) {
     static_assert(P == P64, "other precisions: dslash.cu");

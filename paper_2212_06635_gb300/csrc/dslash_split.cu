@@ -95,9 +95,8 @@ __device__ __forceinline__ void split_hops(cpx<typename PT<P>::R> (&acc)[4][3], 
         ff *= scale[nf];
         fb *= scale[nb];
     }
-    cpx<R> g0[3], g1[3];
-    hop_forward<R, MU, SC>(g0, g1, pf, uf, ff);
-    hop_backward<R, MU, SC, true>(acc, g0, g1, pb, ub, fb);
+    hop_dir<R, MU, -1, false, SC, true>(acc, pf, uf, ff);
+    hop_dir<R, MU, +1, true, SC>(acc, pb, ub, fb);
 }
 
 template <int P, int NF>

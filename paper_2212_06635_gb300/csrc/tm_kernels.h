@@ -9,7 +9,8 @@ namespace tmk {
 
 constexpr int DSLASH_BS = 128;   // direct stencil kernel
 // FP64 passes take half-size blocks: their work is even, so the last wave is what
-// differs (24^3x48: 827 / 666 us at 128 threads, 813 / 652 us at 64, 32 the same)
+// differs (both light passes at 128 / 64 threads: 16^3x32 320 / 300 us, 24^3x48 1379 /
+// 1378 us; both two-flavour ones at 12^3x24 266 / 236 us)
 constexpr int dslash_bs(int P) { return P == P64 ? 64 : DSLASH_BS; }
 constexpr int STAGED_BS = 64;    // shared-memory staged stencil kernel
 constexpr int BLAS_BS = 256;
