@@ -403,3 +403,79 @@ def test_fp64_hops_round_alike_in_all_spins(dims, heavy):
         assert abs(ratio - 1.0) < 0.03, ratio
     finally:
         lat.close()
+
+
+@pytest.mark.parametrize("heavy,bound", [(False, 3.1e-16), (True, 2.86e-16)], ids=["light", "two flavours"])
+def test_even_inverses_round_no_more_than_plain_products(heavy, bound):
+    """Rounding error of the clover term's even-site inverses.  From a unit vector on one
+    odd site a hop gives a column of a link exactly, so the even pass's error is that of
+    the inverse blocks and of three products.  Bound: the relative error of the blocks
+    alone when every 6x6 product is formed in full in the order of its indices (3.1e-16
+    for (A + i s mu)^-1, 2.86e-16 for D - 1), by an extended-precision comparison on the
+    host; with the largest term of each sum last the blocks have 2.1e-16 and 2.2e-16."""
+    import inspect
+    import types
+    from tests.gpu_util import from_dev, to_dev
+    ext = types.ModuleType("dirac_extended")
+    exec(inspect.getsource(D).replace("np.complex128", "np.clongdouble"), ext.__dict__)
+    ld, dims, seed = np.clongdouble, (6, 6, 8, 8), 2100
+    nf = 2 if heavy else 1
+    mu, mubar, epsbar = (0.0, MUBAR, EPSBAR) if heavy else (MU, 0.0, 0.0)
+    u = F.gauge_field(dims, seed)
+    geo = ext.Geometry(dims)
+    U = ext.links_flat(u)
+    A = ext.clover_matrix(geo, U.astype(ld), KAPPA, CSW, geo.even)
+    A = np.stack([A[:, :6, :6], A[:, 6:, 6:]], axis=1)                      # [site][chirality]
+    s = np.array([1, -1])[None, :, None, None]
+    one = np.eye(6)
+
+    def inverse(m):
+        x = np.linalg.inv(m.astype(complex)).astype(ld)
+        for _ in range(2):   # Newton steps: 1e-16 squared is below the extended precision
+            x = x @ (2 * one - m @ x)
+        return x
+    if heavy:
+        tm_, te_ = ld(2 * KAPPA * mubar), ld(2 * KAPPA * epsbar)
+        dinv = inverse(A @ A + (tm_ ** 2 - te_ ** 2) * one)
+        same = [(A - 1j * s * tm_ * one) @ dinv, (A + 1j * s * tm_ * one) @ dinv]
+        cross = te_ * dinv
+    else:
+        same, cross = [inverse(A + 1j * s * ld(2 * KAPPA * mu) * one)], None
+    # odd sites whose neighbours are all different
+    index = np.full(geo.V, -1)
+    index[geo.even] = np.arange(len(geo.even))
+    taken, sites = np.zeros(len(geo.even), bool), []
+    for k, x in enumerate(geo.odd):
+        nb = index[[n[mu_][x] for mu_ in range(4) for n in (geo.fwd, geo.bwd)]]
+        if not taken[nb].any() and len(set(nb)) == 8:
+            taken[nb] = True
+            sites.append(k)
+    assert len(sites) >= 40
+    lat = Lat(u, dims, KAPPA, CSW, mu=mu, mubar=mubar, epsbar=epsbar)
+    tm = lat.tm
+    try:
+        a, o = lat.native(0, nf), lat.native(0, nf)
+        err = norm = 0.0
+        for spin in range(4):
+            for col in range(3):
+                psi = np.zeros((len(geo.odd), nf, 4, 3), complex)
+                psi[sites, 0, spin, col] = 1.0
+                psi = psi if heavy else psi[:, 0]
+                src = to_dev(psi)
+                tm.tm_field_import(lat.ctx, 0, nf, a, src)
+                tm.tm_apply_even(lat.ctx, tm.TM_QH if heavy else tm.TM_QHAT_PLUS, 0, o, a)
+                out = src.clone()
+                tm.tm_field_export(lat.ctx, 0, nf, out, o)
+                got = from_dev(out, psi.shape).reshape(-1, nf, 2, 6)
+                w = D.hop(geo, D.links_flat(u), geo.embed_odd(psi).astype(complex), -1.0, geo.even)
+                w = w.reshape(-1, nf, 2, 6).astype(ld)
+                for f in range(nf):
+                    ref = np.einsum("ncij,ncj->nci", same[f], w[:, f])
+                    if heavy:
+                        ref = ref + np.einsum("ncij,ncj->nci", cross, w[:, 1 - f])
+                    e = np.abs(got[:, f] - ref).astype(float)
+                    err += float(np.sum(e * e))
+                    norm += float(np.sum(np.abs(ref).astype(float) ** 2))
+        assert norm > 0.0 and np.sqrt(err / norm) < bound, np.sqrt(err / norm)
+    finally:
+        lat.close()
