@@ -307,6 +307,8 @@ __host__ __device__ constexpr int herm_off(int i, int j) {   // i > j
 // ---------------------------------------------------------------------------
 // solver control word (device memory, one per problem)
 // ---------------------------------------------------------------------------
+constexpr int RING = 4;   // search directions (residuals) kept between two updates of the solutions
+
 enum CtlFlag { CTL_RUN = 0, CTL_STOP = 1, CTL_BREAKDOWN = 2, CTL_MAXITER = 3 };
 
 struct SolverCtl {
@@ -322,7 +324,7 @@ struct SolverCtl {
     int maxiter;
     int flag;
     int slot, ring;   // iteration within the current ring of directions, and the ring's length
-    double alpha_ring[4];
+    double alpha_ring[RING];
 };
 
 // Multishift state (one per multishift solve), up to MAX_SHIFTS shifts.
@@ -338,7 +340,7 @@ struct MsCtl {
     int n_active;
     // of the iterations of the current ring: the steps, and zeta and beta of the
     // direction that follows
-    double alpha_ring[4][MAX_SHIFTS], zeta_ring[4][MAX_SHIFTS], beta_ring[4][MAX_SHIFTS];
+    double alpha_ring[RING][MAX_SHIFTS], zeta_ring[RING][MAX_SHIFTS], beta_ring[RING][MAX_SHIFTS];
 };
 
 // ---------------------------------------------------------------------------
@@ -348,6 +350,9 @@ constexpr int MAXP = 32;
 // a group: right-hand sides of one operator on one lattice (the shifts of a multishift
 // solve while they are refined)
 constexpr int GROUP = MAX_SHIFTS;
+// (the size of a table tells one problem, a group and a batch apart: find_problem)
+static_assert(GROUP != 1 && GROUP != MAXP, "a group's table must differ from a problem's and from a batch's");
+static_assert(MAX_SHIFTS <= 32, "the shifts' recurrences run a lane each (ms_alpha, ms_update)");
 
 struct Geom {
     int X, Y, Z, T;

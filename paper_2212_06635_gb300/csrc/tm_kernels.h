@@ -21,7 +21,6 @@ constexpr int MIN_BS = 32;       // fewest sites per block of any reducing kerne
 // update in its epilogue, r_out = r - alpha (out + shift p), ||r_out||^2
 // K2_OUT64 (double-word passes): K2_OE_LOCAL with the result stored as FP64
 enum DslashKind { K1_EO_INV = 0, K2_OE_LOCAL = 1, K2_UPDATE = 2, K2_OUT64 = 3 };
-constexpr int RING = 4;   // search directions kept between two updates of the solutions
 
 // FinOp codes beyond those in tm_internal.h
 enum { FIN_PP = 4, FIN_CG_UPDATE = 5, FIN_MS_UPDATE = 6 };
@@ -203,10 +202,11 @@ __device__ __forceinline__ void reduce_finalize(double* partial, unsigned int* c
 // ---------------------------------------------------------------------------
 // vector (BLAS-1) problem tables
 // ---------------------------------------------------------------------------
+static_assert(RING >= 2, "VecProb::v");
 struct VecProb {
     long vh;
     int nblk;
-    void* v[2 + RING];
+    void* v[2 + RING];   // (batches use four)
     SolverCtl* ctl;
     MsCtl* ms;
     double* partial;
