@@ -455,18 +455,20 @@ static const void* clovH_ptr(const tm_ctx* c, int P) {
 // ---------------------------------------------------------------------------
 // Sites per parity up to which the direct passes run as the kernel that splits a site
 // over several warps (dslash_split.cu).  M_hat^dagger M_hat, calls back to back, direct
-// / split, us, at 4,096 / 10,000 / 20,736 sites:
-//   light FP32 20.6 / 16.0, 20.7 / 18.6, 22.7 / 22.7; light FP16 22.7 / 16.7,
-//   22.6 / 20.7, 22.8 / 22.7; heavy FP32 24.8 / 20.7, 27.7 / 34.9; heavy FP16
-//   26.9 / 22.7, 28.8 / 39.1.
-// FP64 goes by waves of blocks of the split kernel, one block on each of the 152 SMs:
-//   light 162 / 63 (4,096), 168 / 137 (10,368), 170 / 178 (19,208), 245 / 225 (20,736),
-//   248 / 229 (24,192: five waves), 248 / 265 (24,576), 319 / 319 (32,928);
-//   heavy 182 / 106 (4,096: one wave), 187 / 206 (5,000), 275 / 307 (10,368).
+// / split, us:
+//   light FP32 18.7 / 16.3 (4,096), 20.5 / 18.6 (10,000), 20.6 / 18.6 (12,096), 20.6 / 22.6
+//   (20,736); light FP16 20.6 / 18.7, 22.6 / 21.4, 22.6 / 20.7, 22.6 / 22.6.
+// Two flavours, and FP64, go by waves of blocks of the split kernel, one block on each
+// of the 152 SMs:
+//   heavy FP32 22.7 / 20.7 (4,096: one wave), 22.6 / 23.1 (6,144), 26.7 / 33.0 (10,000);
+//   heavy FP16 24.6 / 23.0, 24.7 / 26.7, 27.8 / 39.0;
+//   heavy FP64 182 / 106 (4,096), 187 / 206 (5,000), 275 / 307 (10,368);
+//   light FP64 162 / 63 (4,096), 168 / 137 (10,368), 170 / 178 (19,208), 245 / 225 (20,736),
+//   248 / 229 (24,192: five waves), 248 / 265 (24,576), 319 / 319 (32,928).
 constexpr long SPLIT_WAVE = 152 * SPLIT_SITES;
 static long split_limit(int P, int nf) {
-    if (P == P64) return nf == 1 ? 5 * SPLIT_WAVE : SPLIT_WAVE;
-    return nf == 1 ? 12288 : 6144;
+    if (nf == 2) return SPLIT_WAVE;
+    return P == P64 ? 5 * SPLIT_WAVE : 12288;
 }
 
 // Kernel of a pass: the tuned choice (0 direct, 1 staged), or the split kernel in place

@@ -11,8 +11,8 @@
 // lane shuffles, the odd pass reads the partner flavour of psi_o directly.
 //
 // Values are double words (df64.h), held as (hi, lo) FP32 pairs in the FP64
-// layouts.  The passes are bound by FP32 issue (17,000-18,400 instructions per
-// site, 74-80 % of the issue slots busy), so the code
+// layouts.  The passes are bound by FP32 issue (17,100-18,700 instructions per
+// site, 73-77 % of the issue slots busy), so the code
 // - forms every sum of products as a compensated dot product (Ogita, Rump and
 //   Oishi, "Accurate sum and dot product", SIAM J. Sci. Comput. 26 (2005), Dot2):
 //   the high parts are summed with two_sum, the product errors (two_prod with one
