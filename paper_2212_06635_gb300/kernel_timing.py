@@ -3,7 +3,7 @@ algorithmic bytes each launch moves.  bench.py takes its per-kernel figures from
 here, and the ncu captures under profiles/ run these same launch sequences.
 
   python -m paper_2212_06635_gb300.kernel_timing --dims 32 32 32 32 --prec f16 --reps 3
-      even pass x (1 + reps), then odd pass x reps (tm_kernel_times)
+      even pass x (1 + reps), then odd pass x (1 + reps) (tm_kernel_times)
   ... --heavy                     the two-flavour passes
   ... --force NPAIRS [--heavy]    tm_force_outer on NPAIRS field pairs, 1 + reps launches
   ... --ptc                       a 1-8-8-8-1 PTC network applied 1 + reps times

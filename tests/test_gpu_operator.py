@@ -479,3 +479,30 @@ def test_even_inverses_round_no_more_than_plain_products(heavy, bound):
         assert norm > 0.0 and np.sqrt(err / norm) < bound, np.sqrt(err / norm)
     finally:
         lat.close()
+
+
+def test_kernel_times_of_a_fresh_process_are_those_of_a_warm_one():
+    """The first launch of a kernel loads its module (milliseconds); neither pass's time
+    may hold it, or tm_autotune, which compares such times, chooses by it."""
+    import json
+    import os
+    import subprocess
+    import sys
+    code = """
+import json, sys
+import numpy as np, torch
+from paper_2212_06635_gb300 import tm
+from synth import fields as F
+dims = (8, 12, 12, 16)
+ctx = tm.tm_create(dims)
+tm.tm_gauge_load(ctx, np.ascontiguousarray(F.gauge_field(dims, 5)), 1.0)
+tm.tm_clover_compute(ctx, 0.1394, 1.69, mubar=0.1246, epsbar=0.135)
+f = torch.zeros(tm.tm_field_bytes(ctx, tm.TM_F16, 2), dtype=torch.uint8, device="cuda:0")
+print(json.dumps([tm.tm_kernel_times(ctx, tm.TM_QH, tm.TM_F16, f, reps=20) for _ in range(3)]))
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    first, *warm = json.loads(out.stdout.strip().splitlines()[-1])
+    for k in range(2):   # a load takes 100 times a pass of this size; clocks vary by a few per cent
+        assert first[k] < 3 * max(w[k] for w in warm), (first, warm)
